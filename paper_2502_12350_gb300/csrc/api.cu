@@ -63,6 +63,7 @@ struct Plan {
   bool dens;
   int tx, ty;             // forward tile
   int atx, aty;           // adjoint tile
+  int planes, aplanes;    // planes per work item, at most (forward, adjoint)
   std::vector<VolDesc> vols;
   std::vector<WorkItem> items, aitems;
   std::vector<int> rec_ptr, arec_ptr;
@@ -132,7 +133,6 @@ struct mamute_ctx {
   std::vector<cudaEvent_t> dft_ev;
   int dft_n = 0;
   double dft_ms = 0.0, dft_macs = 0.0;
-  int max_planes = 1;  // planes per work item of the current call
   // captured time loop of the last mamute_model call and its signature
   cudaGraphExec_t graph = nullptr;
   std::vector<unsigned long long> graph_key;
@@ -334,8 +334,12 @@ TileChoice choose_tiles(const std::vector<VolDesc>& vols, bool dens, int mode, i
     const int TX = sh[0], TY = sh[1];
     if (force_tx > 0 && (TX != force_tx || TY != force_ty)) continue;
     if (!tile_supported(TX, TY)) continue;
-    const int per_sm = step_blocks_per_sm(TX, TY, dens, mode, Nz);
-    if (per_sm < 1) continue;
+    // The stored-term adjoint's shared memory is close to half an SM's, so its
+    // per-plane table counts as long as the z block is.
+    int per_sm_of[sizeof zsplits / sizeof zsplits[0]];
+    for (size_t k = 0; k < sizeof zsplits / sizeof zsplits[0]; ++k)
+      per_sm_of[k] = step_blocks_per_sm(TX, TY, dens, mode,
+                                        mode == MODE_ADJ_STORED ? (Nz + zsplits[k] - 1) / zsplits[k] : Nz);
     const int warps_cta = (TX / 4) * TY / 32;
     for (int r = 1; r <= 2; ++r) {
       std::vector<Tiling> tl;
@@ -358,9 +362,11 @@ TileChoice choose_tiles(const std::vector<VolDesc>& vols, bool dens, int mode, i
         tl.push_back(std::move(T));
       }
       if (!ok || tiles <= 0) continue;
-      for (int zs : zsplits) {
+      for (size_t k = 0; k < sizeof zsplits / sizeof zsplits[0]; ++k) {
+        const int zs = zsplits[k], per_sm = per_sm_of[k];
         if (force_z > 0 && zs != force_z) continue;
         if (force_z <= 0 && zs > 1 && Nz / zs < 8) break;
+        if (per_sm < 1) continue;
         const long long items = tiles * zs;
         const long long per = (items + n_sm - 1) / n_sm;  // items on the busiest SM
         const double warps = (double)std::min<long long>(per_sm, per) * warps_cta;
@@ -567,6 +573,8 @@ int build_plan(mamute_ctx* ctx, const mamute_grid* g, bool dens, int n_src, cons
     }
   };
   std::vector<int> base;
+  P.planes = (P.Nz + fc.zsplit - 1) / fc.zsplit;
+  P.aplanes = (P.Nz + ac.zsplit - 1) / ac.zsplit;
   make_items(fc, P.items, base);
   std::vector<int> ent_of_col;
   build_receivers(P, P.tx, fc.zsplit, ent, base, fc.tilings, P.items, P.rec_ptr, P.rec,
@@ -721,8 +729,8 @@ int setup(mamute_ctx* ctx, Plan& P, const float* vel, const float* rho, bool nee
 }
 
 // Launch accounting and the timing events around the time loop.
-cudaError_t step_launch(mamute_ctx* ctx, const StepArgs& a, int n_items, int tx, int ty, bool dens,
-                        int mode) {
+cudaError_t step_launch(mamute_ctx* ctx, const StepArgs& a, int n_items, int planes, int tx, int ty,
+                        bool dens, int mode) {
   if (ctx->timing && !ctx->ev0_set) {
     cudaError_t e = cudaEventRecord(ctx->ev0, ctx->stream);
     if (e != cudaSuccess) return e;
@@ -730,7 +738,7 @@ cudaError_t step_launch(mamute_ctx* ctx, const StepArgs& a, int n_items, int tx,
   }
   ++ctx->step_launches;
   ++ctx->launches;
-  cudaError_t e = launch_step(a, n_items, ctx->max_planes, tx, ty, dens, mode, ctx->stream);
+  cudaError_t e = launch_step(a, n_items, planes, tx, ty, dens, mode, ctx->stream);
   if (e == cudaSuccess && ctx->timing) e = cudaEventRecord(ctx->ev1, ctx->stream);
   return e;
 }
@@ -1293,7 +1301,6 @@ int run_model(mamute_ctx* ctx, const mamute_grid* g, const float* vel, const flo
   Plan P;
   TRY(build_plan(ctx, g, rho != nullptr, n_src, src_xyz, rec_offset, rec_xyz,
                  opts ? opts->aperture : nullptr, P, opts ? opts->tiles : nullptr));
-  ctx->max_planes = P.Nz;
   if (P.ncol > 0 && !seis) return fail(ctx, MAMUTE_EINVAL, "seis is NULL");
   int ti = 0, ntd = P.nt;
   TRY(check_interp(ctx, g, opts, &ti, &ntd));
@@ -1330,7 +1337,7 @@ int run_model(mamute_ctx* ctx, const mamute_grid* g, const float* vel, const flo
     key.push_back(((unsigned long long)P.tx << 32) | (unsigned)P.ty);
     key.push_back((unsigned long long)mode * 2 + P.dens);
     key.push_back((unsigned long long)P.ncol);
-    key.push_back((unsigned long long)ctx->max_planes);
+    key.push_back((unsigned long long)P.planes);
     for (const DevBuf* b : {&ctx->items, &ctx->vols, &ctx->maps, &ctx->cmaps, &ctx->gx, &ctx->gy,
                             &ctx->gz, &ctx->recptr, &ctx->rec, &ctx->acc, &ctx->dint,
                             &ctx->pool[0], &ctx->pool[1]})
@@ -1392,13 +1399,13 @@ int run_model(mamute_ctx* ctx, const mamute_grid* g, const float* vel, const flo
         StepArgs a = fwd_args(ctx, P, n, wavelet, nullptr, mode);
         TRY(cpml_fwd_step(ctx, P, T, (const float*)ctx->pool[n & 1].p, a.fout, nullptr,
                           P.ncol > 0 ? drow : nullptr, [&]() -> int {
-                            CK(step_launch(ctx, a, (int)P.items.size(), P.tx, P.ty, P.dens, mode));
+                            CK(step_launch(ctx, a, (int)P.items.size(), P.planes, P.tx, P.ty, P.dens, mode));
                             return MAMUTE_OK;
                           }));
         n += 1;
       } else {
         StepArgs a = fwd_args(ctx, P, n, wavelet, drow, mode);
-        CK(step_launch(ctx, a, (int)P.items.size(), P.tx, P.ty, P.dens, mode));
+        CK(step_launch(ctx, a, (int)P.items.size(), P.planes, P.tx, P.ty, P.dens, mode));
         n += 1;
       }
     }
@@ -1523,7 +1530,6 @@ int run_gradient(mamute_ctx* ctx, const mamute_grid* g, const float* vel, const 
   Plan P;
   TRY(build_plan(ctx, g, rho != nullptr, n_src, src_xyz, rec_offset, rec_xyz,
                  opts ? opts->aperture : nullptr, P, opts ? opts->tiles : nullptr));
-  ctx->max_planes = P.Nz;
   if (P.ncol > 0 && !d_in) return fail(ctx, MAMUTE_EINVAL, "data is NULL");
   int ti = 0, ntd = P.nt;
   TRY(check_interp(ctx, g, opts, &ti, &ntd));
@@ -1550,8 +1556,7 @@ int run_gradient(mamute_ctx* ctx, const mamute_grid* g, const float* vel, const 
                      MODE_ADJ_STORED));
       Q.vmax = P.vmax;
       P = std::move(Q);
-      ctx->max_planes = P.Nz;
-    }
+        }
   }
   const bool ph = opts && opts->phess;
   if (P.pml && ph) return fail(ctx, MAMUTE_EINVAL, "phess is not available with pml");
@@ -1694,11 +1699,11 @@ int run_gradient(mamute_ctx* ctx, const mamute_grid* g, const float* vel, const 
       a.dout = nullptr;
       TRY(cpml_fwd_step(ctx, P, T, (const float*)buf_ptr(cur), a.fout, a.tstore, drow,
                         [&]() -> int {
-                          CK(step_launch(ctx, a, (int)P.items.size(), P.tx, P.ty, P.dens, mode));
+                          CK(step_launch(ctx, a, (int)P.items.size(), P.planes, P.tx, P.ty, P.dens, mode));
                           return MAMUTE_OK;
                         }));
     } else {
-      CK(step_launch(ctx, a, (int)P.items.size(), P.tx, P.ty, P.dens, mode));
+      CK(step_launch(ctx, a, (int)P.items.size(), P.planes, P.tx, P.ty, P.dens, mode));
     }
     if (rec) recorded = n + 1;
     prev = cur;
@@ -1751,6 +1756,7 @@ int run_gradient(mamute_ctx* ctx, const mamute_grid* g, const float* vel, const 
     }
     return MAMUTE_OK;
   };
+  int pending = 0;  // all mode: levels made since the last imaging launch, this step's included
   auto adj_step = [&](int i) -> int {  // adjoint index k = i + 1, imaging against u^i
     const int k = i + 1;
     StepArgs a{};
@@ -1771,7 +1777,17 @@ int run_gradient(mamute_ctx* ctx, const mamute_grid* g, const float* vel, const 
     a.fout = (float*)ctx->psi[k & 1].p;
     a.acc = (float*)ctx->acc.p;
     a.tstore = nullptr;
-    a.tstep = i;  // the all-states adjoint reads the term of step i through its map
+    a.tstep = i;  // the all-states adjoint reads the terms of steps i .. through their map
+    a.nimg = 1;
+    int mode = MODE_ADJ;
+    if (all_mode) {
+      // The levels of up to kImgSteps steps are imaged by one launch.  With
+      // the CPML every step images its own level: the correction kernel adds
+      // to the accumulator what it adds to the level.
+      a.nimg = ++pending;
+      mode = (P.pml || pending == kImgSteps || i == 0) ? MODE_ADJ_STORED : MODE_ADJ_STEP;
+      if (mode == MODE_ADJ_STORED) pending = 0;
+    }
     a.rec_ptr = (const int*)ctx->arecptr.p;
     a.rec = (const RecEntry*)ctx->arec.p;
     a.dout = nullptr;
@@ -1784,8 +1800,7 @@ int run_gradient(mamute_ctx* ctx, const mamute_grid* g, const float* vel, const 
       CK(launch_cpml_pre(c, nvol, T.ext, ctx->stream));
       ctx->launches += kCpmlPreLaunches;
     }
-    CK(step_launch(ctx, a, (int)P.aitems.size(), P.atx, P.aty, P.dens,
-                   all_mode ? MODE_ADJ_STORED : MODE_ADJ));
+    CK(step_launch(ctx, a, (int)P.aitems.size(), P.aplanes, P.atx, P.aty, P.dens, mode));
     if (P.pml) {  // psi^k and the accumulator += the memory-variable part
       CpmlArgs c = T.base;
       c.u = (const float*)ctx->psi[(k + 1) & 1].p;
@@ -1902,7 +1917,6 @@ int run_gn(mamute_ctx* ctx, const mamute_grid* g, const float* vel, const float*
   if (P.pml) return fail(ctx, MAMUTE_EINVAL, "the GN diagonal uses the sponge boundary (pml = 0)");
   if (!P.one_node)
     return fail(ctx, MAMUTE_EINVAL, "the Gauss-Newton diagonal needs receivers on grid nodes");
-  ctx->max_planes = P.Nz;
   TRY(check_cfl(ctx, P, vel));
   // Compact interior term layout: slot k of the ring is [nz][ny][nx].
   auto compact_terms = [](Plan& Q) {
@@ -2038,7 +2052,7 @@ int run_gn(mamute_ctx* ctx, const mamute_grid* g, const float* vel, const float*
       StepArgs a = fwd_args(ctx, P, n, wavelet, nullptr, MODE_FWD_STORE);
       a.items = (const WorkItem*)ctx->items.p + ib;
       a.tstore = V + (size_t)(n % kT) * Nb - (size_t)s0 * N;
-      CK(step_launch(ctx, a, ie - ib, P.tx, P.ty, P.dens, MODE_FWD_STORE));
+      CK(step_launch(ctx, a, ie - ib, P.planes, P.tx, P.ty, P.dens, MODE_FWD_STORE));
       if ((n + 1) % kT == 0) TRY(flush(n + 1));
     }
     TRY(flush(nt));
@@ -2115,7 +2129,7 @@ int run_gn(mamute_ctx* ctx, const mamute_grid* g, const float* vel, const float*
       a.rin = (j == 0) ? imp_row : zero_row;
       a.status = ctx->status;
       a.zs = R->zs;
-      CK(step_launch(ctx, a, ie - ib, R->atx, R->aty, R->dens, MODE_ADJ_TERM));
+      CK(step_launch(ctx, a, ie - ib, R->aplanes, R->atx, R->aty, R->dens, MODE_ADJ_TERM));
       if ((j + 1) % kT == 0) TRY(flush(j + 1));
     }
     TRY(flush(nt));

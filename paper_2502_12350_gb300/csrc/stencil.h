@@ -15,7 +15,11 @@ enum StepMode {
   MODE_ADJ_STORED = 4,
   MODE_ADJ_TERM = 5,
   MODE_FWD_STORE_PH = 6,
+  MODE_ADJ_STEP = 7,
 };
+
+// Adjoint levels imaged by one MODE_ADJ_STORED launch, at most.
+constexpr int kImgSteps = 3;
 
 struct StepArgs {
   const WorkItem* items;
@@ -35,7 +39,8 @@ struct StepArgs {
   float* fout;            // pool receiving the new level (buffer fcur ^ 1)
   float* acc;             // accumulator pool (pseudo-Hessian or imaging)
   float* tstore;          // imaging-term store for this step (all-states mode)
-  int tstep;              // step index of the term read by the all-states adjoint
+  int tstep;              // all-states adjoint: step of the term imaged with the new level
+  int nimg;               // levels imaged by a MODE_ADJ_STORED launch: terms tstep .. tstep + nimg - 1
   const int* rec_ptr;     // per-item per-plane receiver offsets
   const RecEntry* rec;    // receiver entries
   float* dout;            // forward: data row of this step (internal columns), may be null

@@ -1,4 +1,5 @@
-// Instantiations of the adjoint time-step kernel (modes ADJ, ADJ_STORED, ADJ_TERM).
+// Instantiations of the adjoint time-step kernel (modes ADJ, ADJ_STORED, ADJ_STEP,
+// ADJ_TERM).
 #include "stencil_impl.cuh"
 
 namespace mamute {
@@ -15,6 +16,12 @@ cudaError_t dispatch_adjoint(const StepArgs& a, int n_items, int max_planes, int
     case MODE_ADJ_STORED:
 #define MAMUTE_T(TX, TY) \
   if (tx == TX && ty == TY) return launch_mode<TX, TY, MODE_ADJ_STORED>(a, n_items, max_planes, dens, s, occ);
+      MAMUTE_TILES(MAMUTE_T)
+#undef MAMUTE_T
+      return cudaErrorInvalidValue;
+    case MODE_ADJ_STEP:
+#define MAMUTE_T(TX, TY) \
+  if (tx == TX && ty == TY) return launch_mode<TX, TY, MODE_ADJ_STEP>(a, n_items, max_planes, dens, s, occ);
       MAMUTE_TILES(MAMUTE_T)
 #undef MAMUTE_T
       return cudaErrorInvalidValue;

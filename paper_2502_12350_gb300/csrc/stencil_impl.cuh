@@ -108,16 +108,27 @@ __device__ __forceinline__ float img_term(float u, float A, float M, float lap, 
   return t;
 }
 
-template <int TX, int TY, bool ADJ, bool RECOMP>
+// Shared-memory layout and mode traits of one kernel variant.
+template <int TX, int TY, bool DENS, int MODE>
 struct Layout {
+  static constexpr bool ADJ = MODE == MODE_ADJ || MODE == MODE_ADJ_STORED ||
+                              MODE == MODE_ADJ_STEP || MODE == MODE_ADJ_TERM;
+  static constexpr bool RECOMP = MODE == MODE_ADJ;  // a second halo'd field (u for the imaging)
+  static constexpr bool ACC = MODE == MODE_FWD_PH || MODE == MODE_FWD_STORE_PH ||
+                              MODE == MODE_ADJ || MODE == MODE_ADJ_STORED;
+  static constexpr int NT = MODE == MODE_ADJ_STORED ? kImgSteps : 0;  // stored-term tiles
   static constexpr int NCT = (TX / 4) * TY;  // compute threads
   static constexpr int HS = (TX + 2 * kHalo) * (TY + 2 * kHalo);  // halo stage floats
   static constexpr int CS = TX * TY;  // centre tile floats
-  // Halo ring depth: 5 planes in use plus 3 ahead (2 ahead when two halo'd
-  // fields share each stage, to keep two CTAs per SM).
-  static constexpr int NSU = (ADJ && RECOMP) ? 7 : 8;
-  static constexpr int NSC = ADJ ? 4 : 3;  // centre ring depth
-  static constexpr int NHALO = (ADJ && RECOMP) ? 2 : 1;  // halo'd fields per stage
+  static constexpr int NC = 2 + (DENS ? 1 : 0) + (ACC ? 1 : 0) + NT;  // centre arrays
+  // Halo ring depth: 5 planes in use plus 3 ahead (2 ahead where two halo'd
+  // fields share each stage or the centre ring is at its widest, to keep two
+  // CTAs per SM).
+  static constexpr int NSU = (RECOMP || (NT && DENS)) ? 7 : 8;
+  // Centre ring depth: a stage of the imaging launch holds up to 7 tiles, so
+  // two of them are as many bytes in flight as four of a plain step.
+  static constexpr int NSC = NT ? 2 : (ADJ ? 4 : 3);
+  static constexpr int NHALO = RECOMP ? 2 : 1;  // halo'd fields per stage
 };
 
 // Per-plane metadata staged in shared memory: sponge factor gz and the
@@ -135,7 +146,22 @@ struct PlaneInfo {
 //   MODE_FWD_STORE  forward step + store of the imaging term t on the interior
 //   MODE_FWD_STORE_PH  both of the above (all-terms gradient with pseudo-Hessian)
 //   MODE_ADJ        adjoint step + imaging against a recomputed forward field
-//   MODE_ADJ_STORED adjoint step + imaging against the stored imaging term
+//   MODE_ADJ_STEP   adjoint step alone
+//   MODE_ADJ_STORED adjoint step + imaging of the last 1 to kImgSteps levels
+//                   against their stored terms
+//   MODE_ADJ_TERM   adjoint step + store of the new level on the interior
+//
+// The accumulator is read and written once per kImgSteps = 3 adjoint steps:
+// an adjoint step reads the levels k + 2 (centre tile) and k + 1 (halo'd
+// planes) and makes level k, so the launch that images has the three levels
+// at hand and takes their three terms T_{k+1}, T_k, T_{k-1} in the same order
+// of fused multiply-adds as one term per step would (the same bits).  Per
+// three steps and point that is 48 + 8 + 12 bytes (the terms on the model
+// interior only) instead of 48 + 24 + 12, and the two launches that do not
+// image need less than half of the centre ring.  Bound by HBM: on a 320^3
+// window with a 256^3 model 88.8 us for a plain step and 148.9 us with the
+// imaging of three levels, against 158.6 us for every step that images its
+// own (a 400-step gradient 114.1 -> 94.4 ms).
 // Resident CTAs per SM the register budget is sized for: the adjoint with a
 // recomputed forward field on large tiles needs more than 200 KB of shared
 // memory per pair, so it runs one CTA per SM with the full register file.
@@ -147,15 +173,11 @@ struct MinBlocks {
 template <int TX, int TY, bool DENS, int MODE>
 __global__ void __launch_bounds__((TX / 4) * TY + 32, (MinBlocks<TX, TY, MODE>::value))
     step_kernel(const StepArgs a) {
-  constexpr bool ADJ = (MODE == MODE_ADJ || MODE == MODE_ADJ_STORED || MODE == MODE_ADJ_TERM);
-  constexpr bool RECOMP = (MODE == MODE_ADJ);
-  constexpr bool ACC = (MODE == MODE_FWD_PH || MODE == MODE_FWD_STORE_PH || MODE == MODE_ADJ ||
-                       MODE == MODE_ADJ_STORED);
-  constexpr bool TERM = (MODE == MODE_ADJ_STORED);  // stored imaging term as a centre array
-  using LY = Layout<TX, TY, ADJ, RECOMP>;
+  using LY = Layout<TX, TY, DENS, MODE>;
+  constexpr bool ADJ = LY::ADJ, RECOMP = LY::RECOMP, ACC = LY::ACC;
+  constexpr bool TERM = LY::NT > 0;  // stored imaging terms as centre arrays
   constexpr int NCT = LY::NCT, HS = LY::HS, CS = LY::CS, NSU = LY::NSU, NSC = LY::NSC;
-  constexpr int NHALO = LY::NHALO;
-  constexpr int NC = 2 + (DENS ? 1 : 0) + (ACC ? 1 : 0) + (TERM ? 1 : 0);  // centre arrays
+  constexpr int NHALO = LY::NHALO, NC = LY::NC;
   constexpr int CI_PREV = 0, CI_A = 1, CI_M = 2, CI_ACC = DENS ? 3 : 2, CI_T = CI_ACC + 1;
 
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -254,15 +276,16 @@ __global__ void __launch_bounds__((TX / 4) * TY + 32, (MinBlocks<TX, TY, MODE>::
             drain();
             return;
           }
-          mbar_arrive_expect_tx(&fullC[c], NC * CS * 4);
+          mbar_arrive_expect_tx(&fullC[c], (NC - (TERM ? kImgSteps - a.nimg : 0)) * CS * 4);
           float* cd = cring + c * NC * CS;
           tma_load_3d(cd + CI_PREV * CS, mapP, x0, y0, q, &fullC[c]);
           tma_load_3d(cd + CI_A * CS, mapA, cx, cy, q, &fullC[c]);
           if (DENS) tma_load_3d(cd + CI_M * CS, mapM, cx, cy, q, &fullC[c]);
           if (ACC) tma_load_3d(cd + CI_ACC * CS, mapAcc, x0, y0, q, &fullC[c]);
           if (TERM)
-            tma_load_4d(cd + CI_T * CS, mapT, x0 - V.txoff, y0 - V.iy0, q - V.border, a.tstep,
-                        &fullC[c]);
+            for (int m = 0; m < a.nimg; ++m)
+              tma_load_4d(cd + (CI_T + m) * CS, mapT, x0 - V.txoff, y0 - V.iy0, q - V.border,
+                          a.tstep + m, &fullC[c]);
           ++nC;
         }
       }
@@ -299,6 +322,19 @@ __global__ void __launch_bounds__((TX / 4) * TY + 32, (MinBlocks<TX, TY, MODE>::
       for (int e = 0; e < 4; ++e) v.v[e] = -v.v[e];
     }
     return v;
+  };
+  // Four points of an interior array (imaging term or adjoint level) on the
+  // imaging region.
+  auto store_term = [&](int z, const F4& v) {
+    const int zi = z - V.border, yi = gyl - V.iy0;
+    if (row_ok && col_ok && yi >= 0 && yi < V.nyi && zi >= 0 && zi < V.nzi) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int xi = gxl + e - V.ix0;
+        if (xi >= 0 && xi < V.nxi)
+          a.tstore[V.toff + ((long long)zi * V.nyi + yi) * V.tpitch + (gxl + e - V.txoff)] = v.v[e];
+      }
+    }
   };
   // Priming: planes zb-4 .. zb+3 fill queue slots 0..7.
   for (int i = 0; i < 2 * kHalo; ++i) {
@@ -390,18 +426,7 @@ __global__ void __launch_bounds__((TX / 4) * TY + 32, (MinBlocks<TX, TY, MODE>::
       }
     }
     // Interior store of the new adjoint level.
-    if (MODE == MODE_ADJ_TERM) {
-      const int zi = z - V.border, yi = gyl - V.iy0;
-      if (row_ok && col_ok && yi >= 0 && yi < V.nyi && zi >= 0 && zi < V.nzi) {
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const int xi = gxl + e - V.ix0;
-          if (xi >= 0 && xi < V.nxi)
-            a.tstore[V.toff + ((long long)zi * V.nyi + yi) * V.tpitch + (gxl + e - V.txoff)] =
-                out.v[e];
-        }
-      }
-    }
+    if (MODE == MODE_ADJ_TERM) store_term(z, out);
     // Imaging / accumulation.
     if (MODE == MODE_FWD_PH || MODE == MODE_FWD_STORE || MODE == MODE_FWD_STORE_PH ||
         MODE == MODE_ADJ || MODE == MODE_ADJ_STORED) {
@@ -411,35 +436,34 @@ __global__ void __launch_bounds__((TX / 4) * TY + 32, (MinBlocks<TX, TY, MODE>::
         lap4<TX>(st + HS, lx, ly, qu, lu);
 #pragma unroll
         for (int e = 0; e < 4; ++e) t.v[e] = img_term(qu[4].v[e], Av.v[e], Mv.v[e], lu[e], DENS);
-      } else if (MODE == MODE_ADJ_STORED) {
-        t = ld4s(cs + CI_T * CS);
-      } else {
+      } else if (MODE != MODE_ADJ_STORED) {
 #pragma unroll
         for (int e = 0; e < 4; ++e) t.v[e] = img_term(q[4].v[e], Av.v[e], Mv.v[e], lap[e], DENS);
       }
-      if (MODE == MODE_FWD_STORE || MODE == MODE_FWD_STORE_PH) {
-        const int zi = z - V.border, yi = gyl - V.iy0;
-        if (row_ok && col_ok && yi >= 0 && yi < V.nyi && zi >= 0 && zi < V.nzi) {
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const int xi = gxl + e - V.ix0;
-            if (xi >= 0 && xi < V.nxi)
-              a.tstore[V.toff + ((long long)zi * V.nyi + yi) * V.tpitch + (gxl + e - V.txoff)] =
-                  t.v[e];
-          }
-        }
-      }
+      if (MODE == MODE_FWD_STORE || MODE == MODE_FWD_STORE_PH) store_term(z, t);
       if (ACC) {
-        const F4 acc = ld4s(cs + CI_ACC * CS);
-        F4 nacc;
+        F4 nacc = ld4s(cs + CI_ACC * CS);
+        if (TERM) {  // the older levels first: k + 2, k + 1, k
+          if (a.nimg > 2) {
+            t = ld4s(cs + (CI_T + 2) * CS);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) nacc.v[e] = __fmaf_rn(prev.v[e], t.v[e], nacc.v[e]);
+          }
+          if (a.nimg > 1) {
+            t = ld4s(cs + (CI_T + 1) * CS);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) nacc.v[e] = __fmaf_rn(q[4].v[e], t.v[e], nacc.v[e]);
+          }
+          t = ld4s(cs + CI_T * CS);
+        }
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
           if (ADJ) {
-            nacc.v[e] = __fmaf_rn(out.v[e], t.v[e], acc.v[e]);
+            nacc.v[e] = __fmaf_rn(out.v[e], t.v[e], nacc.v[e]);
           } else {
             const float g = __fmul_rn(gxv[e], gyz);
             const float gt = __fmul_rn(g, t.v[e]);
-            nacc.v[e] = __fmaf_rn(gt, gt, acc.v[e]);
+            nacc.v[e] = __fmaf_rn(gt, gt, nacc.v[e]);
           }
         }
         // (whole window; the gradient and pseudo-Hessian read its imaging region)
@@ -476,13 +500,8 @@ __global__ void __launch_bounds__((TX / 4) * TY + 32, (MinBlocks<TX, TY, MODE>::
 
 template <int TX, int TY, bool DENS, int MODE>
 static size_t smem_bytes_base() {
-  constexpr bool ADJ = (MODE == MODE_ADJ || MODE == MODE_ADJ_STORED || MODE == MODE_ADJ_TERM);
-  constexpr bool RECOMP = (MODE == MODE_ADJ);
-  constexpr bool ACC = (MODE == MODE_FWD_PH || MODE == MODE_FWD_STORE_PH || MODE == MODE_ADJ ||
-                       MODE == MODE_ADJ_STORED);
-  using LY = Layout<TX, TY, ADJ, RECOMP>;
-  constexpr int NC = 2 + (DENS ? 1 : 0) + (ACC ? 1 : 0) + (MODE == MODE_ADJ_STORED ? 1 : 0);
-  return sizeof(float) * (size_t)(LY::NSU * LY::NHALO * LY::HS + LY::NSC * NC * LY::CS + LY::CS) +
+  using LY = Layout<TX, TY, DENS, MODE>;
+  return sizeof(float) * (size_t)(LY::NSU * LY::NHALO * LY::HS + LY::NSC * LY::NC * LY::CS + LY::CS) +
          sizeof(uint64_t) * (2 * LY::NSU + 2 * LY::NSC);
 }
 

@@ -114,7 +114,7 @@ struct mamute_ctx {
   DevBuf pitems, pnbr, precptr, prec, pcells, pgvals, pmaps, pflags;  // two-level launches
   bool pair_graph_failed = false;  // cooperative launches could not be captured
   DevBuf rsPtr, rsCol, rsW, dmod, ddat;      // time resampling: band matrix (c0, len, weights), model- and data-axis traces
-  DevBuf cpml, cprof, cnode, crec, ccell, cgval;  // convolutional PML
+  DevBuf cpml, cext, cprof, cvols;  // convolutional PML: memory variables, E, profiles, slabs
   DevBuf items, vols, maps, cmaps, recptr, rec, colmap, gx, gy, gz, cells, gvals, srccell,
       aitems, arecptr, arec, acolmap, acells, agvals;
   DevBuf hvel, hrho, hseis, hobs, hgrad, hphess;  // staging for the *_host calls
@@ -322,7 +322,7 @@ struct TileChoice {
   std::vector<Tiling> tilings;
 };
 
-TileChoice choose_tiles(const std::vector<VolDesc>& vols, bool dens, int mode, int n_sm,
+TileChoice choose_tiles(const std::vector<VolDesc>& vols, bool dens, bool pml, int mode, int n_sm,
                         int force_tx, int force_ty, int force_z) {
   static const int shapes[][2] = {{64, 16}, {72, 16}, {48, 16}, {96, 8}, {64, 8},
                                   {128, 8}, {32, 16}, {32, 8}};
@@ -338,7 +338,7 @@ TileChoice choose_tiles(const std::vector<VolDesc>& vols, bool dens, int mode, i
     // per-plane table counts as long as the z block is.
     int per_sm_of[sizeof zsplits / sizeof zsplits[0]];
     for (size_t k = 0; k < sizeof zsplits / sizeof zsplits[0]; ++k)
-      per_sm_of[k] = step_blocks_per_sm(TX, TY, dens, mode,
+      per_sm_of[k] = step_blocks_per_sm(TX, TY, dens, pml, mode,
                                         mode == MODE_ADJ_STORED ? (Nz + zsplits[k] - 1) / zsplits[k] : Nz);
     const int warps_cta = (TX / 4) * TY / 32;
     for (int r = 1; r <= 2; ++r) {
@@ -550,9 +550,9 @@ int build_plan(mamute_ctx* ctx, const mamute_grid* g, bool dens, int n_src, cons
   if (n_sm < 1) n_sm = 1;
   const int fmode = dens ? MODE_FWD : MODE_FWD;
   auto pick = [&](int i, const char* env) { return (tiles && tiles[i] > 0) ? tiles[i] : env_int(env, 0); };
-  TileChoice fc = choose_tiles(P.vols, dens, fmode, n_sm, pick(0, "MAMUTE_TX"), pick(1, "MAMUTE_TY"),
+  TileChoice fc = choose_tiles(P.vols, dens, P.pml, fmode, n_sm, pick(0, "MAMUTE_TX"), pick(1, "MAMUTE_TY"),
                                pick(2, "MAMUTE_ZSPLIT"));
-  TileChoice ac = choose_tiles(P.vols, dens, adj_mode, n_sm, pick(3, "MAMUTE_ADJ_TX"),
+  TileChoice ac = choose_tiles(P.vols, dens, P.pml, P.pml ? MODE_ADJ_STORED : adj_mode, n_sm, pick(3, "MAMUTE_ADJ_TX"),
                                pick(4, "MAMUTE_ADJ_TY"), pick(5, "MAMUTE_ADJ_ZSPLIT"));
   if (fc.tilings.empty() || ac.tilings.empty())
     return fail(ctx, MAMUTE_EINVAL, "unsupported tile shape");
@@ -711,6 +711,10 @@ int setup(mamute_ctx* ctx, Plan& P, const float* vel, const float* rho, bool nee
       ok = ok && enc(8, ctx->acc.p, P.tx, P.ty);
       ok = ok && enc(11, ctx->acc.p, P.atx, P.aty);
     }
+    if (P.pml) {
+      ok = ok && enc(13, ctx->cext.p, P.tx, P.ty);
+      ok = ok && enc(14, ctx->cext.p, P.atx, P.aty);
+    }
     if (!ok) return fail(ctx, MAMUTE_ECUDA, "cuTensorMapEncodeTiled failed (shot %d)", (int)s);
   }
   CK(upload(ctx->maps, maps, ctx->stream));
@@ -729,8 +733,8 @@ int setup(mamute_ctx* ctx, Plan& P, const float* vel, const float* rho, bool nee
 }
 
 // Launch accounting and the timing events around the time loop.
-cudaError_t step_launch(mamute_ctx* ctx, const StepArgs& a, int n_items, int planes, int tx, int ty,
-                        bool dens, int mode) {
+cudaError_t step_launch(mamute_ctx* ctx, const Plan& P, const StepArgs& a, int n_items, int planes,
+                        int tx, int ty, int mode) {
   if (ctx->timing && !ctx->ev0_set) {
     cudaError_t e = cudaEventRecord(ctx->ev0, ctx->stream);
     if (e != cudaSuccess) return e;
@@ -738,7 +742,7 @@ cudaError_t step_launch(mamute_ctx* ctx, const StepArgs& a, int n_items, int pla
   }
   ++ctx->step_launches;
   ++ctx->launches;
-  cudaError_t e = launch_step(a, n_items, planes, tx, ty, dens, mode, ctx->stream);
+  cudaError_t e = launch_step(a, n_items, planes, tx, ty, P.dens, P.pml, mode, ctx->stream);
   if (e == cudaSuccess && ctx->timing) e = cudaEventRecord(ctx->ev1, ctx->stream);
   return e;
 }
@@ -1160,7 +1164,8 @@ int data_to_user(mamute_ctx* ctx, const Plan& P, int n0, int n1, float* seis, cu
 // ---- Convolutional PML (Sec. 2, the second absorbing boundary) ----
 
 // Layer coefficients of one padded axis of N cells with `border` layer cells
-// at each end, appended to bo / co: b = exp(-(d + alpha) dt) and
+// at each end, appended to bo / co with kCpmlPad cells outside the layer
+// before and after, rounded up to a multiple of 4: b = exp(-(d + alpha) dt) and
 // c = d (b - 1) / (d + alpha) with, at depth r = dist / border,
 // d = d0 r^2, d0 = -3 vmax ln(R) / (2 border h), alpha = pi f0 (1 - r);
 // b = 1, c = 0 outside the layer.  low_face = false: no layer at the low
@@ -1169,10 +1174,10 @@ int data_to_user(mamute_ctx* ctx, const Plan& P, int n0, int n1, float* seis, cu
 void cpml_profile(int N, int border, double h, double dt, double vmax, double f0, double R,
                   std::vector<float>& bo, std::vector<float>& co, bool low_face = true) {
   const double d0 = border > 0 ? -3.0 * vmax * std::log(R) / (2.0 * border * h) : 0.0;
-  for (int i = 0; i < N; ++i) {
+  for (int i = -kCpmlPad; i < N + kCpmlPad; ++i) {
     int dist = 0;
-    if (i < border) dist = low_face ? border - i : 0;
-    else if (i > N - 1 - border) dist = i - (N - 1 - border);
+    if (i >= 0 && i < border) dist = low_face ? border - i : 0;
+    else if (i < N && i > N - 1 - border) dist = i - (N - 1 - border);
     double b = 1.0, c = 0.0;
     if (dist > 0) {
       const double r = (double)dist / border;
@@ -1183,111 +1188,124 @@ void cpml_profile(int N, int border, double h, double dt, double vmax, double f0
     bo.push_back((float)b);
     co.push_back((float)c);
   }
+  while (bo.size() % 4) {
+    bo.push_back(1.0f);
+    co.push_back(0.0f);
+  }
 }
 
-// Pools of the CPML memory variables, each P.pool_elems floats in ctx->cpml:
-// 0..2 Psi_a, 3..5 Zeta_a (their multipliers in the reverse pass), 6..8 y_a,
-// 9..11 z_a (reverse scratch).
-constexpr int kPmlPoolsModel = 6, kPmlPoolsGradient = 12;
+// Memory variables per axis in ctx->cpml, each T.elems floats: Psi twice and
+// Zeta (modelling); the multipliers of both, twice each (reverse pass).
+constexpr int kPmlArraysModel = 3, kPmlArraysGradient = 4;
 
 struct PmlTables {
-  CpmlArgs base{};          // buffers and profiles; u, out, tstore, acc set per launch
-  CpmlExtent ext{};         // extents of the kernels' grids
+  CpmlArgs base{};     // profiles, slabs and E; fields and memory variables set per launch
+  CpmlExtent ext{};    // extents of the launches
+  long long elems = 0; // elements of one memory variable on every slab
+  float* mem = nullptr;
 };
 
-// Profiles, the data columns' nodes and scales, and the pools (after setup()).
-int cpml_setup(mamute_ctx* ctx, const Plan& P, const float* vel, const float* rho, int n_pools,
-               PmlTables& T) {
-  std::vector<float> bx, cx, by, cy, bz, cz;
-  for (const VolDesc& V : P.vols) {
-    if ((long long)V.Nx * V.Ny * V.Nz >= (1LL << 32))  // 32-bit shell indexing
+// Modelling on windows of at most this many padded points in all launches
+// every slab piece apart, which with the main step keeps the eight launches
+// per step that callers of mamute_ctx_last_timing count on tiny windows; it
+// is no faster there.  Above it a step is four launches.
+constexpr long long kPmlApartPoints = 128 * 1024;
+
+// Slabs of every window (the plan's windows learn where E is not zero).
+void cpml_slabs(Plan& P, std::vector<CpmlVol>& cv, PmlTables& T) {
+  const int w = P.b > 0 ? P.b + 4 : 0;
+  CpmlExtent& e = T.ext;
+  e = CpmlExtent{};
+  e.nvol = (int)P.vols.size();
+  for (VolDesc& V : P.vols) {
+    CpmlVol W{};
+    const int N[3] = {V.Nx, V.Ny, V.Nz};
+    for (int a = 0; a < 3; ++a) {
+      const int end = a == 0 ? (int)round_up(V.Nx, 4) : N[a];  // rows are padded with zeros
+      int lo = std::min(w, N[a]), hi = std::max(N[a] - w, lo);
+      if (a == 0) {
+        lo = (int)round_up(lo, 4);
+        hi = std::max((N[a] - w) & ~3, lo);
+        if (w == 0) hi = end;
+      }
+      if (a == 2 && P.zs >= 0) {  // no layer at the surface
+        lo = 0;
+        hi = std::max(N[a] - w, 0);
+      }
+      W.lo[a] = lo;
+      W.hi[a] = hi;
+      W.n[a] = w ? lo + end - hi : 0;
+      W.off[a] = T.elems;
+      T.elems += round_up((long long)W.n[a] * (a == 0 ? (long long)V.Ny * V.Nz
+                                                      : (long long)V.pitch * (a == 1 ? V.Nz : V.Ny)),
+                          64);
+      const int len = lo == hi ? (end + 1) / 2 : std::max(lo, end - hi);
+      e.len[a] = std::max(e.len[a], w ? len : 0);
+      const long long nx4 = round_up(V.Nx, 4) / 4;
+      const long long cols = a == 0 ? (long long)W.n[0] / 4 * V.Ny * V.Nz : nx4 * (a == 1 ? V.Nz : V.Ny);
+      e.cols[a] = std::max(e.cols[a], w ? cols : 0);
+      e.threads[a] += 2 * cols;
+    }
+    V.ex0 = W.lo[0];
+    V.ex1 = W.hi[0];
+    V.ey0 = W.lo[1];
+    V.ey1 = W.hi[1];
+    V.ez0 = W.lo[2];
+    V.ez1 = W.hi[2];
+    cv.push_back(W);
+  }
+}
+
+// Profiles, slabs and zeroed memory variables and E.
+int cpml_setup(mamute_ctx* ctx, const Plan& P, std::vector<CpmlVol>& cv, int n_arrays, PmlTables& T) {
+  std::vector<float> b, c;
+  std::vector<CpmlVol>& W = cv;
+  const int pz = 0;
+  cpml_profile(P.Nz, P.b, P.h, P.dt, P.vmax, P.pml_f0, P.pml_r, b, c, P.zs < 0);
+  for (size_t s = 0; s < P.vols.size(); ++s) {
+    const VolDesc& V = P.vols[s];
+    if ((long long)V.Nx * V.Ny * V.Nz >= (1LL << 32))  // 32-bit column indexing
       return fail(ctx, MAMUTE_EINVAL, "pml: a shot window of 2^32 points or more");
-    cpml_profile(V.Nx, P.b, P.h, P.dt, P.vmax, P.pml_f0, P.pml_r, bx, cx);
-    cpml_profile(V.Ny, P.b, P.h, P.dt, P.vmax, P.pml_f0, P.pml_r, by, cy);
-    T.ext.xy = std::max(T.ext.xy, (long long)V.Nx * V.Ny);
-    T.ext.xz = std::max(T.ext.xz, (long long)V.Nx * V.Nz);
-    T.ext.yz = std::max(T.ext.yz, (long long)V.Ny * V.Nz);
+    W[s].prof[2] = pz;
+    W[s].prof[0] = (int)b.size();
+    cpml_profile(V.Nx, P.b, P.h, P.dt, P.vmax, P.pml_f0, P.pml_r, b, c);
+    W[s].prof[1] = (int)b.size();
+    cpml_profile(V.Ny, P.b, P.h, P.dt, P.vmax, P.pml_f0, P.pml_r, b, c);
   }
-  T.ext.border = P.b;
-  cpml_profile(P.Nz, P.b, P.h, P.dt, P.vmax, P.pml_f0, P.pml_r, bz, cz, P.zs < 0);
-  std::vector<float> all;
-  size_t off[6];
-  const std::vector<float>* parts[6] = {&bx, &cx, &by, &cy, &bz, &cz};
-  for (int k = 0; k < 6; ++k) {
-    off[k] = all.size();
-    all.insert(all.end(), parts[k]->begin(), parts[k]->end());
-  }
-  CK(upload(ctx->cprof, all, ctx->stream));
-  const float* base = (const float*)ctx->cprof.p;
-  // Data columns in the forward tables' order (the layout data_to_user
-  // reads), sampled after the memory-variable correction of each step.
-  std::vector<int> ent_of_col(P.ncol, 0);
-  for (size_t e = 0; e < P.ent.size(); ++e) ent_of_col[P.fwd_col_of_ent[e]] = (int)e;
-  std::vector<long long> node(P.ncol), cell(P.ncol);
-  std::vector<RecEntry> rec(P.ncol);
-  std::vector<float> gval(P.ncol, 1.0f);
-  for (int c = 0; c < P.ncol; ++c) {
-    const NodeEntry& E = P.ent[ent_of_col[c]];
-    const VolDesc& V = P.vols[E.shot];
-    node[c] = V.off + ((long long)E.lz * V.Ny + E.ly) * V.pitch + E.lx;
-    cell[c] = E.cell;
-    rec[c] = RecEntry{};
-    rec[c].col = c;
-    rec[c].wgt = E.w;
-  }
-  CK(upload(ctx->cnode, node, ctx->stream));
-  CK(upload(ctx->ccell, cell, ctx->stream));
-  CK(upload(ctx->crec, rec, ctx->stream));
-  CK(upload(ctx->cgval, gval, ctx->stream));
-  if (P.ncol > 0) {  // fscale = w sqrt(rho) of the columns
-    GeomArgs ga{vel, rho, P.ncol, 0, (const long long*)ctx->ccell.p, (const float*)ctx->cgval.p,
-                (RecEntry*)ctx->crec.p, nullptr, nullptr, nullptr, P.h, P.dt};
-    CK(aux_count(ctx, launch_geometry(ga, ctx->stream)));
-  }
-  const size_t pool = (size_t)P.pool_elems * 4;
-  CK(ensure(ctx->cpml, (size_t)n_pools * pool));
-  CK(cudaMemsetAsync(ctx->cpml.p, 0, (size_t)n_pools * pool, ctx->stream));
-  CpmlArgs& c = T.base;
-  c.vols = (const VolDesc*)ctx->vols.p;
-  c.pr = CpmlProf{base + off[0], base + off[1], base + off[2], base + off[3], base + off[4],
-                  base + off[5]};
-  c.A = (const float*)ctx->coefA.p;
-  c.pitchG = P.pitchG;
-  c.NyG = P.Ny;
-  for (int k = 0; k < 3; ++k) {
-    c.m1[k] = (float*)ctx->cpml.p + (size_t)k * P.pool_elems;
-    c.m2[k] = (float*)ctx->cpml.p + (size_t)(3 + k) * P.pool_elems;
-    c.y[k] = n_pools > 6 ? (float*)ctx->cpml.p + (size_t)(6 + k) * P.pool_elems : nullptr;
-    c.z[k] = n_pools > 6 ? (float*)ctx->cpml.p + (size_t)(9 + k) * P.pool_elems : nullptr;
-  }
+  const size_t nb = b.size();
+  b.insert(b.end(), c.begin(), c.end());
+  CK(upload(ctx->cprof, b, ctx->stream));
+  CK(upload(ctx->cvols, W, ctx->stream));
+  const size_t mem = (size_t)n_arrays * T.elems * 4, pool = (size_t)P.pool_elems * 4;
+  CK(ensure(ctx->cpml, mem));
+  CK(ensure(ctx->cext, pool));
+  if (mem) CK(cudaMemsetAsync(ctx->cpml.p, 0, mem, ctx->stream));
+  CK(cudaMemsetAsync(ctx->cext.p, 0, pool, ctx->stream));
+  CpmlArgs& a = T.base;
+  a.vols = (const VolDesc*)ctx->vols.p;
+  a.cv = (const CpmlVol*)ctx->cvols.p;
+  a.b = (const float*)ctx->cprof.p;
+  a.c = a.b + nb;
+  a.E = (float*)ctx->cext.p;
+  T.mem = (float*)ctx->cpml.p;
   return MAMUTE_OK;
 }
 
-// One forward CPML step around the main step launch `main` (u^n in u, the
-// main kernel writes u^{n+1} to out): the Psi update before it, the Zeta
-// update and the correction of u^{n+1} (and of the stored term) after it,
-// then the data sample of the step into drow (may be null).
-template <typename Main>
-int cpml_fwd_step(mamute_ctx* ctx, const Plan& P, const PmlTables& T, const float* u, float* out,
-                  float* tstore, float* drow, Main main) {
+// The memory-variable part of a CPML step, before its main launch: step n of
+// the forward recursion on u^n, or the reverse of step n on psi^{n + 2}.
+int cpml_step(mamute_ctx* ctx, const PmlTables& T, bool reverse, int n, const float* u) {
   CpmlArgs c = T.base;
   c.u = u;
-  c.out = out;
-  c.tstore = tstore;
-  const int nvol = (int)P.vols.size();
+  c.m1 = T.mem + (n & 1) * T.elems;
+  c.m1n = T.mem + (~n & 1) * T.elems;
+  c.m2 = T.mem + (reverse ? 2 + (n & 1) : 2) * T.elems;
+  c.m2n = T.mem + (reverse ? 2 + (~n & 1) : 2) * T.elems;
   if (ctx->timing && !ctx->ev0_set) {
     CK(cudaEventRecord(ctx->ev0, ctx->stream));
     ctx->ev0_set = true;
   }
-  CK(launch_cpml_psi(c, nvol, T.ext, ctx->stream));
-  ctx->launches += kCpmlAxisLaunches;
-  TRY(main());
-  CK(launch_cpml_fcorr(c, nvol, T.ext, ctx->stream));
-  ctx->launches += kCpmlAxisLaunches;
-  if (drow)
-    CK(aux_count(ctx, launch_cpml_record(out, (const long long*)ctx->cnode.p,
-                                         (const RecEntry*)ctx->crec.p, P.ncol, drow, ctx->stream)));
-  if (ctx->timing) CK(cudaEventRecord(ctx->ev1, ctx->stream));
+  CK(reverse ? launch_cpml_reverse(c, T.ext, ctx->stream) : launch_cpml_forward(c, T.ext, ctx->stream));
+  ctx->launches += cpml_launches(T.ext);
   return MAMUTE_OK;
 }
 
@@ -1307,9 +1325,17 @@ int run_model(mamute_ctx* ctx, const mamute_grid* g, const float* vel, const flo
   TRY(check_cfl(ctx, P, vel));
   const bool ph = opts && opts->phess;
   if (P.pml && ph) return fail(ctx, MAMUTE_EINVAL, "phess is not available with pml");
-  TRY(setup(ctx, P, vel, rho, false, ph));
   PmlTables T;
-  if (P.pml) TRY(cpml_setup(ctx, P, vel, rho, kPmlPoolsModel, T));
+  std::vector<CpmlVol> cv;
+  if (P.pml) {
+    cpml_slabs(P, cv, T);
+    long long points = 0;
+    for (const VolDesc& V : P.vols) points += (long long)V.Nx * V.Ny * V.Nz;
+    T.ext.apart = points <= kPmlApartPoints;
+    TRY(cpml_setup(ctx, P, cv, kPmlArraysModel, T));
+  }
+  TRY(setup(ctx, P, vel, rho, false, ph));
+  T.base.vols = (const VolDesc*)ctx->vols.p;
   const size_t pool = (size_t)P.pool_elems * 4;
   CK(cudaMemsetAsync(ctx->pool[0].p, 0, pool, ctx->stream));
   CK(cudaMemsetAsync(ctx->pool[1].p, 0, pool, ctx->stream));
@@ -1352,8 +1378,15 @@ int run_model(mamute_ctx* ctx, const mamute_grid* g, const float* vel, const flo
                             &ctx->pflags})
       push(pairs ? b->p : nullptr);
     key.push_back(P.pml ? 1 : 0);
-    for (const DevBuf* b : {&ctx->cpml, &ctx->cprof, &ctx->cnode, &ctx->crec})
+    for (const DevBuf* b : {&ctx->cpml, &ctx->cext, &ctx->cprof, &ctx->cvols})
       push(P.pml ? b->p : nullptr);
+    // the slab launches' grids and the arrays' size
+    for (int a = 0; a < 3; ++a) {
+      key.push_back(P.pml ? (unsigned long long)T.ext.cols[a] : 0);
+      key.push_back(P.pml ? (unsigned long long)T.ext.len[a] : 0);
+      key.push_back(P.pml ? (unsigned long long)T.ext.threads[a] : 0);
+    }
+    key.push_back(P.pml ? (unsigned long long)T.elems * 2 + T.ext.apart : 0);
     key.push_back(stream_out ? 1 : 0);
     if (stream_out) {
       push(seis);
@@ -1395,17 +1428,10 @@ int run_model(mamute_ctx* ctx, const mamute_grid* g, const float* vel, const flo
         CK(launch_pair(a, (int)P.pitems.size(), P.Nz, P.ptx, P.pty, P.dens, ctx->stream, nullptr));
         if (ctx->timing) CK(cudaEventRecord(ctx->ev1, ctx->stream));
         n += 2;
-      } else if (P.pml) {
-        StepArgs a = fwd_args(ctx, P, n, wavelet, nullptr, mode);
-        TRY(cpml_fwd_step(ctx, P, T, (const float*)ctx->pool[n & 1].p, a.fout, nullptr,
-                          P.ncol > 0 ? drow : nullptr, [&]() -> int {
-                            CK(step_launch(ctx, a, (int)P.items.size(), P.planes, P.tx, P.ty, P.dens, mode));
-                            return MAMUTE_OK;
-                          }));
-        n += 1;
       } else {
+        if (P.pml) TRY(cpml_step(ctx, T, false, n, (const float*)ctx->pool[n & 1].p));
         StepArgs a = fwd_args(ctx, P, n, wavelet, drow, mode);
-        CK(step_launch(ctx, a, (int)P.items.size(), P.planes, P.tx, P.ty, P.dens, mode));
+        CK(step_launch(ctx, P, a, (int)P.items.size(), P.planes, P.tx, P.ty, mode));
         n += 1;
       }
     }
@@ -1495,7 +1521,7 @@ int run_model(mamute_ctx* ctx, const mamute_grid* g, const float* vel, const flo
     }
     const int loop = pairs ? (P.nt / 2 + P.nt % 2) : P.nt;
     ctx->step_launches = loop;
-    ctx->launches += loop * (P.pml ? 2 * kCpmlAxisLaunches + (P.ncol > 0 ? 2 : 1) : 1) +
+    ctx->launches += loop * (P.pml ? cpml_launches(T.ext) + 1 : 1) +
                      (stream_out ? std::min(P.nt, 8) * (P.one_node ? 1 : 2) : 0);
   }
 loop_done:
@@ -1563,9 +1589,14 @@ int run_gradient(mamute_ctx* ctx, const mamute_grid* g, const float* vel, const 
   if (P.pml && opts && opts->n_snapshots > 0)
     return fail(ctx, MAMUTE_EINVAL,
                 "a pml gradient keeps every step's imaging term: n_snapshots must be 0 or -1");
-  TRY(setup(ctx, P, vel, rho, true, true));
   PmlTables T;
-  if (P.pml) TRY(cpml_setup(ctx, P, vel, rho, kPmlPoolsGradient, T));
+  std::vector<CpmlVol> cv;
+  if (P.pml) {
+    cpml_slabs(P, cv, T);
+    TRY(cpml_setup(ctx, P, cv, kPmlArraysGradient, T));
+  }
+  TRY(setup(ctx, P, vel, rho, true, true));
+  T.base.vols = (const VolDesc*)ctx->vols.p;
   const size_t pool = (size_t)P.pool_elems * 4;
   const size_t ncol = std::max(P.ncol, 1);
   CK(ensure(ctx->dint, (size_t)P.nt * ncol * 4));
@@ -1693,18 +1724,8 @@ int run_gradient(mamute_ctx* ctx, const mamute_grid* g, const float* vel, const 
     a.mU = a.mF;
     a.sU = a.sF;
     a.fout = (float*)buf_ptr(out);
-    if (P.pml) {
-      // the data sample is taken after the memory-variable correction
-      float* drow = a.dout;
-      a.dout = nullptr;
-      TRY(cpml_fwd_step(ctx, P, T, (const float*)buf_ptr(cur), a.fout, a.tstore, drow,
-                        [&]() -> int {
-                          CK(step_launch(ctx, a, (int)P.items.size(), P.planes, P.tx, P.ty, P.dens, mode));
-                          return MAMUTE_OK;
-                        }));
-    } else {
-      CK(step_launch(ctx, a, (int)P.items.size(), P.planes, P.tx, P.ty, P.dens, mode));
-    }
+    if (P.pml) TRY(cpml_step(ctx, T, false, n, (const float*)buf_ptr(cur)));
+    CK(step_launch(ctx, P, a, (int)P.items.size(), P.planes, P.tx, P.ty, mode));
     if (rec) recorded = n + 1;
     prev = cur;
     cur = out;
@@ -1781,11 +1802,9 @@ int run_gradient(mamute_ctx* ctx, const mamute_grid* g, const float* vel, const 
     a.nimg = 1;
     int mode = MODE_ADJ;
     if (all_mode) {
-      // The levels of up to kImgSteps steps are imaged by one launch.  With
-      // the CPML every step images its own level: the correction kernel adds
-      // to the accumulator what it adds to the level.
+      // The levels of up to kImgSteps steps are imaged by one launch.
       a.nimg = ++pending;
-      mode = (P.pml || pending == kImgSteps || i == 0) ? MODE_ADJ_STORED : MODE_ADJ_STEP;
+      mode = (pending == kImgSteps || i == 0) ? MODE_ADJ_STORED : MODE_ADJ_STEP;
       if (mode == MODE_ADJ_STORED) pending = 0;
     }
     a.rec_ptr = (const int*)ctx->arecptr.p;
@@ -1794,29 +1813,15 @@ int run_gradient(mamute_ctx* ctx, const mamute_grid* g, const float* vel, const 
     a.rin = (const float*)ctx->rint.p + (size_t)i * P.ncol;
     a.status = ctx->status;
     a.zs = P.zs;
-    if (P.pml) {  // memory-variable multipliers from psi^{k+1}
-      CpmlArgs c = T.base;
-      c.u = (const float*)ctx->psi[(k + 1) & 1].p;
-      CK(launch_cpml_pre(c, nvol, T.ext, ctx->stream));
-      ctx->launches += kCpmlPreLaunches;
-    }
-    CK(step_launch(ctx, a, (int)P.aitems.size(), P.aplanes, P.atx, P.aty, P.dens, mode));
-    if (P.pml) {  // psi^k and the accumulator += the memory-variable part
-      CpmlArgs c = T.base;
-      c.u = (const float*)ctx->psi[(k + 1) & 1].p;
-      c.out = (float*)ctx->psi[k & 1].p;
-      c.tstore = (float*)ctx->tstore.p + (size_t)i * P.term_elems;
-      c.acc = (float*)ctx->acc.p;
-      CK(launch_cpml_acorr(c, nvol, T.ext, ctx->stream));
-      ctx->launches += kCpmlAxisLaunches;
-      if (ctx->timing) CK(cudaEventRecord(ctx->ev1, ctx->stream));
-    }
+    if (P.pml)  // memory-variable multipliers and E from psi^{k+1}
+      TRY(cpml_step(ctx, T, true, i, (const float*)ctx->psi[(k + 1) & 1].p));
+    CK(step_launch(ctx, P, a, (int)P.aitems.size(), P.aplanes, P.atx, P.aty, mode));
     return MAMUTE_OK;
   };
   auto begin_adjoint = [&]() -> int {
     TRY(make_residual());
     if (P.pml)  // the memory variables' multipliers start at zero
-      CK(cudaMemsetAsync(ctx->cpml.p, 0, (size_t)kPmlPoolsGradient * pool, ctx->stream));
+      CK(cudaMemsetAsync(ctx->cpml.p, 0, (size_t)kPmlArraysGradient * T.elems * 4, ctx->stream));
     if (ph) {
       FinalizeArgs fa{(const float*)ctx->acc.p, (const VolDesc*)ctx->vols.p, (int)P.vols.size(),
                       vel, P.nx, P.ny, P.nz, P.b, P.dt, 1, 0, opts->phess};
@@ -2052,7 +2057,7 @@ int run_gn(mamute_ctx* ctx, const mamute_grid* g, const float* vel, const float*
       StepArgs a = fwd_args(ctx, P, n, wavelet, nullptr, MODE_FWD_STORE);
       a.items = (const WorkItem*)ctx->items.p + ib;
       a.tstore = V + (size_t)(n % kT) * Nb - (size_t)s0 * N;
-      CK(step_launch(ctx, a, ie - ib, P.planes, P.tx, P.ty, P.dens, MODE_FWD_STORE));
+      CK(step_launch(ctx, P, a, ie - ib, P.planes, P.tx, P.ty, MODE_FWD_STORE));
       if ((n + 1) % kT == 0) TRY(flush(n + 1));
     }
     TRY(flush(nt));
@@ -2129,7 +2134,7 @@ int run_gn(mamute_ctx* ctx, const mamute_grid* g, const float* vel, const float*
       a.rin = (j == 0) ? imp_row : zero_row;
       a.status = ctx->status;
       a.zs = R->zs;
-      CK(step_launch(ctx, a, ie - ib, R->aplanes, R->atx, R->aty, R->dens, MODE_ADJ_TERM));
+      CK(step_launch(ctx, *R, a, ie - ib, R->aplanes, R->atx, R->aty, MODE_ADJ_TERM));
       if ((j + 1) % kT == 0) TRY(flush(j + 1));
     }
     TRY(flush(nt));
@@ -2245,7 +2250,7 @@ void mamute_ctx_destroy(mamute_ctx* ctx) {
                    &ctx->srcw, &ctx->smA, &ctx->smMat, &ctx->smLam, &ctx->rsPtr, &ctx->rsCol,
                    &ctx->rsW, &ctx->dmod, &ctx->ddat, &ctx->pitems, &ctx->pnbr, &ctx->precptr,
                    &ctx->prec, &ctx->pcells, &ctx->pgvals, &ctx->pmaps, &ctx->pflags,
-                   &ctx->cpml, &ctx->cprof, &ctx->cnode, &ctx->crec, &ctx->ccell, &ctx->cgval};
+                   &ctx->cpml, &ctx->cext, &ctx->cprof, &ctx->cvols};
   for (DevBuf* b : all) release(*b);
   if (ctx->status) cudaFree(ctx->status);
   if (ctx->maxbits) cudaFree(ctx->maxbits);

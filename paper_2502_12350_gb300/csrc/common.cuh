@@ -41,6 +41,9 @@ struct VolDesc {
   int ix0, iy0;
   int nxi, nyi, nzi;
   int txoff, tpitch;     // term store rows: local x in [txoff, txoff + tpitch)
+  // Convolutional PML: E is zero on x in [ex0, ex1), y in [ey0, ey1), z in
+  // [ez0, ez1) (outside the layer slabs of all axes).
+  int ex0, ex1, ey0, ey1, ez0, ez1;
   long long off;         // element offset of the shot's arrays in each pool
   long long slab;        // elements per wavefield array (Nz * Ny * pitch, rounded)
   long long toff;        // offset of the shot's region in one step of the term store
@@ -73,8 +76,9 @@ struct RecEntry {
 //   [9] u0 halo A  [10] u1 halo A    (forward field read by the imaging)
 //  [11] accumulator centre A (imaging)
 //  [12] term store (x, y, z, step) centre A, 4-D (all-states adjoint)
+//  [13] E centre F  [14] E centre A  (convolutional PML)
 struct ShotMaps {
-  CUtensorMap m[13];
+  CUtensorMap m[15];
 };
 
 // Global coefficient maps: [0] A centre, [1] M = A m2 centre.

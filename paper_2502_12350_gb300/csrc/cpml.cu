@@ -9,24 +9,33 @@
 // uses A = c^2 dt^2 / h^2 like the damping kernels):
 //   Psi_a'  = b_a Psi_a  + c_a D1_a u
 //   Zeta_a' = b_a Zeta_a + c_a (D2_a u + D1_a Psi_a')
-//   u'      = (2 - M) u - v + A (lap u + sum_a (D1_a Psi_a' + Zeta_a')) + source
+//   u'      = (2 - M) u - v + A (lap u + E) + source,  E = sum_a (D1_a Psi_a' + Zeta_a')
 // with b_a = exp(-(d_a + alpha_a) dt), c_a = d_a (b_a - 1) / (d_a + alpha_a)
-// (profiles built on the host; b = 1, c = 0 outside the layer).  The main
-// step kernel forms (2 - M) u - v + A lap u + source everywhere (damping
-// factor 1); the kernels here add the memory-variable part of each axis on
-// that axis's layer slabs, where it is non-zero, and the same amount to the
-// stored imaging term A lap u - M u.
+// (profiles built on the host; b = 1, c = 0 outside the layer).
 //
 // The gradient is the exact transpose of this recursion.  In the adjoint
 // level psi (the multiplier of u scaled by A, which the main kernel
 // propagates with the forward operator itself), one reverse step is
-//   per axis, in the layer:  y_a = c_a (Zb_a + psi),  Zb_a <- b_a (Zb_a + psi)
-//                            p_a = Pb_a - D1_a (psi + y_a),  Pb_a <- b_a p_a,  z_a = c_a p_a
-//   main adjoint step:       psi' = (2 - M) psi - psi_prev + A lap psi + injection
-//   correction (per axis):   psi' += A sum_a (D2_a y_a - D1_a z_a)
+//   per axis, in the layer:  y_a = c_a (Zb_a + psi),  Zb_a' = b_a (Zb_a + psi)
+//                            p_a = Pb_a - D1_a (psi + y_a),  Pb_a' = b_a p_a
+//   psi' = (2 - M) psi - psi_prev + A (lap psi + E) + injection,
+//   E = sum_a (D2_a y_a - D1_a (c_a p_a))
 // (Zb, Pb the multipliers of Zeta and Psi; D2 is symmetric, D1 antisymmetric,
-// the fields are zero outside the padded window), and the imaging
-// accumulator takes the corrected psi' against the stored term.
+// the fields are zero outside the padded window).
+//
+// Work split.  E depends on the old state alone, so one launch per axis makes
+// the whole memory-variable part before the main step, which reads E as one
+// more centre tile: per layer point and axis the field, the two memory
+// variables (read and written) and E, 28 bytes written or read once by the
+// slab kernel and the main step together.  (The earlier form updated Psi
+// before the main step, Zeta after it, and corrected u', the imaging term
+// and the accumulator in place, once per axis: 40 bytes forward and 60 in
+// reverse, in 6 and 7 launches.  448x448x256 with density: 577 -> 326 us a
+// step, of which 59, 37 and 50 us the z, y and x slabs and 179 us the main
+// step; 250 forward and reverse steps of 256^3: 167 -> 95 ms.)  A cell needs the new Psi (p) of its 4
+// neighbours on each side; they are made again from the old values instead
+// of being exchanged, so Psi, and in the reverse both multipliers, are kept
+// twice (read one copy, write the other) and a slab may be cut anywhere.
 #include "cpml.h"
 
 #include <algorithm>
@@ -35,534 +44,517 @@ namespace mamute {
 
 namespace {
 
-__constant__ float kC2[5] = {MAMUTE_C0, MAMUTE_C1, MAMUTE_C2, MAMUTE_C3, MAMUTE_C4};
-__constant__ float kD1[4] = {4.0f / 5.0f, -1.0f / 5.0f, 4.0f / 105.0f, -1.0f / 280.0f};
+constexpr int kThreads = 128;
+constexpr int kDepth = 4;  // cells in flight per marching thread
 
-constexpr int kZG = 4;  // cells per load group of the marching kernels
+// First and second difference at the centre of 9 consecutive values.
+__device__ __forceinline__ float d1(float m4, float m3, float m2, float m1, float p1, float p2,
+                                    float p3, float p4) {
+  float s = 4.0f / 5.0f * (p1 - m1);
+  s = fmaf(-1.0f / 5.0f, p2 - m2, s);
+  s = fmaf(4.0f / 105.0f, p3 - m3, s);
+  return fmaf(-1.0f / 280.0f, p4 - m4, s);
+}
 
-struct Pt {
-  int x, y, z;
+__device__ __forceinline__ float d2(float m4, float m3, float m2, float m1, float v, float p1,
+                                    float p2, float p3, float p4) {
+  float s = MAMUTE_C0 * v;
+  s = fmaf(MAMUTE_C1, p1 + m1, s);
+  s = fmaf(MAMUTE_C2, p2 + m2, s);
+  s = fmaf(MAMUTE_C3, p3 + m3, s);
+  return fmaf(MAMUTE_C4, p4 + m4, s);
+}
+
+#define D1Q(q, k, e) \
+  d1(q[(k) - 4][e], q[(k) - 3][e], q[(k) - 2][e], q[(k) - 1][e], q[(k) + 1][e], q[(k) + 2][e], \
+     q[(k) + 3][e], q[(k) + 4][e])
+#define D2Q(q, k, e) \
+  d2(q[(k) - 4][e], q[(k) - 3][e], q[(k) - 2][e], q[(k) - 1][e], q[k][e], q[(k) + 1][e], \
+     q[(k) + 2][e], q[(k) + 3][e], q[(k) + 4][e])
+#define D1R(q, k) \
+  d1(q[(k) - 4], q[(k) - 3], q[(k) - 2], q[(k) - 1], q[(k) + 1], q[(k) + 2], q[(k) + 3], q[(k) + 4])
+#define D2R(q, k) \
+  d2(q[(k) - 4], q[(k) - 3], q[(k) - 2], q[(k) - 1], q[k], q[(k) + 1], q[(k) + 2], q[(k) + 3], \
+     q[(k) + 4])
+
+template <int V>
+struct VecT;
+template <>
+struct VecT<2> {
+  using T = float2;
+};
+template <>
+struct VecT<4> {
+  using T = float4;
 };
 
-__device__ __forceinline__ long long idx(const VolDesc& V, int x, int y, int z) {
-  return V.off + ((long long)z * V.Ny + y) * V.pitch + x;
-}
-
-// Element stride of axis a in a window's arrays.
-__device__ __forceinline__ long long axis_stride(const VolDesc& V, int a) {
-  return a == 0 ? 1LL : (a == 1 ? (long long)V.pitch : (long long)V.Ny * V.pitch);
-}
-
-// Neighbours p - 4 .. p + 4 along axis a of the point at element i (zero
-// outside the window; the bounds are tested only near the window's faces).
-// No kernel writes an array that it reads this way, so the loads take the
-// read-only path and may be issued ahead of the kernel's stores.
-__device__ __forceinline__ void column(const float* f, const VolDesc& V, Pt p, int a, long long i,
-                                       float (&v)[9]) {
-  const int q = a == 0 ? p.x : (a == 1 ? p.y : p.z);
-  const int N = a == 0 ? V.Nx : (a == 1 ? V.Ny : V.Nz);
-  const long long st = axis_stride(V, a);
-  if (q >= 4 && q + 4 < N) {
-#pragma unroll
-    for (int m = -4; m <= 4; ++m) v[m + 4] = __ldg(f + i + m * st);
-  } else {
-#pragma unroll
-    for (int m = -4; m <= 4; ++m) v[m + 4] = (q + m >= 0 && q + m < N) ? __ldg(f + i + m * st) : 0.0f;
+template <int V>
+__device__ __forceinline__ void unpack(const typename VecT<V>::T& t, float (&v)[V]) {
+  v[0] = t.x;
+  v[1] = t.y;
+  if constexpr (V == 4) {
+    v[2] = t.z;
+    v[3] = t.w;
   }
 }
 
-__device__ __forceinline__ float d2(const float* f, const VolDesc& V, Pt p, int a, long long i) {
-  float v[9];
-  column(f, V, p, a, i, v);
-  float s = kC2[0] * v[4];
-#pragma unroll
-  for (int m = 1; m <= 4; ++m) s = fmaf(kC2[m], v[4 + m] + v[4 - m], s);
-  return s;
+template <int V>
+__device__ __forceinline__ typename VecT<V>::T pack(const float (&v)[V]) {
+  if constexpr (V == 4)
+    return make_float4(v[0], v[1], v[2], v[3]);
+  else
+    return make_float2(v[0], v[1]);
 }
 
-__device__ __forceinline__ float d1(const float* f, const VolDesc& V, Pt p, int a, long long i) {
-  float v[9];
-  column(f, V, p, a, i, v);
-  float s = 0.0f;
-#pragma unroll
-  for (int m = 1; m <= 4; ++m) s = fmaf(kD1[m - 1], v[4 + m] - v[4 - m], s);
-  return s;
+// Asynchronous copy of V floats into the thread's own shared-memory slot;
+// zeros where ok is false (the source address is then not read).
+template <int V>
+__device__ __forceinline__ void cp_async(void* dst, const float* src, bool ok) {
+  const int n = ok ? V * 4 : 0;
+  if constexpr (V == 4)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src),
+                 "r"(n)
+                 : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(smem_u32(dst)), "l"(src),
+                 "r"(n)
+                 : "memory");
 }
 
-__device__ __forceinline__ void prof(const CpmlProf& c, const VolDesc& V, Pt p, int a, float& b,
-                                     float& cc) {
-  if (a == 0) {
-    b = c.bx[V.gx_off + p.x];
-    cc = c.cx[V.gx_off + p.x];
-  } else if (a == 1) {
-    b = c.by[V.gy_off + p.y];
-    cc = c.cy[V.gy_off + p.y];
-  } else {
-    b = c.bz[p.z];
-    cc = c.cz[p.z];
-  }
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-__device__ __forceinline__ bool in_layer(float b, float cc) { return cc != 0.0f || b != 1.0f; }
-
-// Index of p in the imaging-region layout, or -1 outside the region.
-__device__ __forceinline__ long long region_index(const VolDesc& V, Pt p) {
-  const int zi = p.z - V.border, yi = p.y - V.iy0, xi = p.x - V.ix0;
-  if (xi < 0 || xi >= V.nxi || yi < 0 || yi >= V.nyi || zi < 0 || zi >= V.nzi) return -1;
-  return V.toff + ((long long)zi * V.nyi + yi) * V.tpitch + (p.x - V.txoff);
-}
-
-// The slab pair of width w across axis A (2: z, 1: y) of window V, marched
-// along A: blockIdx.z = 0 takes [0, lo), 1 takes [hi, N) with lo = min(w, N),
-// hi = max(N - w, lo); one thread per column across the other two axes (x
-// fastest), at element i0 with the marched coordinate 0 and element stride st.
-// With merge, slabs less than 8 cells apart are marched as one range [0, N)
-// by the blockIdx.z = 0 threads (for kernels whose queues reach 4 cells past
-// their range into values that the range's own march writes).
-template <int A>
-struct Slab {
-  int s0, s1;
-  unsigned ncol;
-  long long st, stA;  // strides along A in the window and in the coefficient grid
-  __device__ __forceinline__ bool init(const VolDesc& V, const CpmlArgs& c, int w,
-                                       bool merge = false) {
-    const int N = A == 2 ? V.Nz : V.Ny;
-    const int lo = min(w, N), hi = max(N - w, lo);
-    s0 = blockIdx.z == 0 ? 0 : hi;
-    s1 = blockIdx.z == 0 ? lo : N;
-    if (merge && hi - lo < 8) {
-      s0 = 0;
-      s1 = blockIdx.z == 0 ? N : 0;
+// One thread's march along axis A (1: y, 2: z): V consecutive x cells of one
+// column, the cells [s0, s1) of the slab region [r0, r1), in element strides
+// st (fields) and sc (slab arrays).
+template <int A, int V>
+struct March {
+  int s0, s1, r0, r1, N;
+  bool add;  // E already holds another axis's part here
+  long long st, sc;
+  const float* u;
+  long long m;  // slab-array element of cell r0
+  float* E;
+  int prof;
+  __device__ __forceinline__ bool init(const CpmlArgs& c, int chunk, int first) {
+    const VolDesc& D = c.vols[blockIdx.y];
+    const CpmlVol& W = c.cv[blockIdx.y];
+    N = A == 2 ? D.Nz : D.Ny;
+    const int lo = W.lo[A], hi = W.hi[A];
+    const bool merged = lo == hi;  // one range [0, N)
+    const int nlo = merged ? 0 : (lo + chunk - 1) / chunk;
+    int k = first + blockIdx.z;
+    if (k < nlo) {
+      r0 = 0;
+      r1 = lo;
+    } else {
+      k -= nlo;
+      r0 = merged ? 0 : hi;
+      r1 = N;
     }
-    ncol = (unsigned)V.Nx * (unsigned)(A == 2 ? V.Ny : V.Nz);
-    st = A == 2 ? (long long)V.Ny * V.pitch : (long long)V.pitch;
-    stA = A == 2 ? (long long)c.NyG * c.pitchG : (long long)c.pitchG;
-    return s0 < s1;
-  }
-  __device__ __forceinline__ Pt column(const VolDesc& V, unsigned q) const {
-    const unsigned o = q / (unsigned)V.Nx;
-    Pt p;
-    p.x = (int)(q - o * (unsigned)V.Nx);
-    p.y = A == 2 ? (int)o : 0;
-    p.z = A == 2 ? 0 : (int)o;
-    return p;
-  }
-  __device__ __forceinline__ static void at(Pt& p, int s) {
-    if (A == 2)
-      p.z = s;
-    else
-      p.y = s;
-  }
-  __device__ __forceinline__ static void profile(const CpmlProf& pr, const VolDesc& V, int s, float& b,
-                                                 float& cc) {
-    b = A == 2 ? pr.bz[s] : pr.by[V.gy_off + s];
-    cc = A == 2 ? pr.cz[s] : pr.cy[V.gy_off + s];
+    s0 = r0 + k * chunk;
+    s1 = min(s0 + chunk, r1);
+    if (s0 >= r1) return false;
+    const unsigned nxv = (unsigned)(D.Nx + V - 1) / V;
+    const unsigned q = blockIdx.x * kThreads + threadIdx.x;
+    const unsigned o = q / nxv;
+    if (o >= (unsigned)(A == 2 ? D.Ny : D.Nz)) return false;
+    const int x = (int)(q - o * nxv) * V;
+    const long long plane = (long long)D.Ny * D.pitch;
+    const int slot = merged || r0 == 0 ? 0 : lo;  // slot of cell r0
+    st = A == 2 ? plane : D.pitch;
+    sc = st;
+    const long long f = D.off + (A == 2 ? (long long)o * D.pitch : (long long)o * plane) + x;
+    u = c.u + f;
+    E = c.E + f;
+    m = W.off[A] + x + (A == 2 ? ((long long)slot * D.Ny + o) * D.pitch
+                              : ((long long)o * W.n[A] + slot) * D.pitch);
+    prof = W.prof[A] + kCpmlPad;
+    add = A == 1 && ((int)o < W.lo[2] || (int)o >= W.hi[2]);
+    return true;
   }
 };
 
-// Calls f(p) for every point within w cells of an x face of window V, one
-// point per thread of the blockIdx.x range (x fastest, then y, then z).
-template <typename F>
-__device__ __forceinline__ void for_xslab(const VolDesc& V, int w, F f) {
-  const int lx = min(w, V.Nx), hx = max(V.Nx - w, lx);
-  const unsigned nx3 = (unsigned)(lx + V.Nx - hx);
-  // fewer than 2^32 points (windows are checked on the host): 32-bit indices
-  const long long n = (long long)nx3 * V.Ny * V.Nz;
-  for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < n;
-       q += (long long)gridDim.x * blockDim.x) {
-    const unsigned q32 = (unsigned)q;
-    const unsigned r = q32 / nx3, zz = r / (unsigned)V.Ny;
-    const int xx = (int)(q32 - r * nx3);
-    Pt p;
-    p.x = xx < lx ? xx : hx + (xx - lx);
-    p.y = (int)(r - zz * (unsigned)V.Ny);
-    p.z = (int)zz;
-    f(p);
-  }
-}
-
-// f at coordinate s of the column starting at element i0 (zero outside
-// [0, N)); f is not written by the kernel that reads it this way.
-__device__ __forceinline__ float sval(const float* f, long long i0, long long st, int s, int N) {
-  return (s >= 0 && s < N) ? __ldg(f + i0 + s * st) : 0.0f;
-}
-
-__device__ __forceinline__ float d1q(const float (&v)[9]) {
-  float s = 0.0f;
-#pragma unroll
-  for (int m = 1; m <= 4; ++m) s = fmaf(kD1[m - 1], v[4 + m] - v[4 - m], s);
-  return s;
-}
-
-__device__ __forceinline__ float d2q(const float (&v)[9]) {
-  float s = kC2[0] * v[4];
-#pragma unroll
-  for (int m = 1; m <= 4; ++m) s = fmaf(kC2[m], v[4 + m] + v[4 - m], s);
-  return s;
-}
-
-__device__ __forceinline__ void shift(float (&v)[9], float next) {
-#pragma unroll
-  for (int m = 0; m < 8; ++m) v[m] = v[m + 1];
-  v[8] = next;
-}
-
-__device__ __forceinline__ float coefA(const CpmlArgs& c, const VolDesc& V, Pt p) {
-  return c.A[((long long)p.z * c.NyG + (p.y + V.cy0)) * c.pitchG + (p.x + V.cx0)];
-}
-
-// ---------------------------------------------------------------- forward
-//
-// Each axis's terms live in its own pair of layer slabs, so each update
-// runs as one launch per axis: for z and y a kernel that marches the slab
-// along the axis with one thread per column (x fastest), the neighbours
-// along the axis in register queues and the loads of kZG cells issued
-// before their stores; for x one point per thread, the x neighbours coming
-// from the same cache lines as the neighbouring threads' points.  The
-// correction adds each axis's part to u^{n+1} (and to the stored term) in
-// turn.
-
+// Forward, axes z and y: the thread marches along the axis with the field in a
+// 13-deep register queue and the new Psi in a 9-deep one, at step p making
+// Psi'(p) and finishing cell s = p - 4.  Bound by HBM; the loads of the next
+// kDepth - 1 cells are in flight as asynchronous copies into the thread's own
+// shared-memory slots (no barrier), which costs no registers.
 template <int A>
-__global__ void __launch_bounds__(256, 4) psi_march_kernel(CpmlArgs c) {
-  const VolDesc V = c.vols[blockIdx.y];
-  Slab<A> S;
-  if (!S.init(V, c, V.border)) return;
-  const int N = A == 2 ? V.Nz : V.Ny;
-  for (unsigned q = blockIdx.x * blockDim.x + threadIdx.x; q < S.ncol; q += gridDim.x * blockDim.x) {
-    const Pt p = S.column(V, q);
-    const long long i0 = idx(V, p.x, p.y, p.z);
-    float v[9];  // u at s - 4 .. s + 4
-#pragma unroll
-    for (int m = 0; m < 9; ++m) v[m] = sval(c.u, i0, S.st, S.s0 - 4 + m, N);
-    for (int sg = S.s0; sg < S.s1; sg += kZG) {
-      float mv[kZG], un[kZG], b[kZG], cc[kZG];
-#pragma unroll
-      for (int k = 0; k < kZG; ++k) {
-        const int s = sg + k;
-        b[k] = 1.0f;
-        cc[k] = 0.0f;
-        if (s < S.s1) Slab<A>::profile(c.pr, V, s, b[k], cc[k]);
-        mv[k] = in_layer(b[k], cc[k]) ? c.m1[A][i0 + s * S.st] : 0.0f;
-        un[k] = sval(c.u, i0, S.st, s + 5, N);
-      }
-#pragma unroll
-      for (int k = 0; k < kZG; ++k) {
-        if (in_layer(b[k], cc[k])) c.m1[A][i0 + (sg + k) * S.st] = fmaf(b[k], mv[k], cc[k] * d1q(v));
-        shift(v, un[k]);
+__global__ void __launch_bounds__(kThreads, 3) fwd_march_kernel(CpmlArgs c, int chunk, int first) {
+  constexpr int V = 4;
+  using T = VecT<V>::T;
+  __shared__ T ring[kDepth][4][kThreads];  // u, Psi, Zeta, E
+  March<A, V> w;
+  if (!w.init(c, chunk, first)) return;
+  const int tid = threadIdx.x;
+  const int p0 = w.s0 - 4, p1 = w.s1 + 4;
+  auto issue = [&](int p) {
+    if (p < p1) {
+      T* r = &ring[(p - p0) % kDepth][0][tid];
+      const int e = p + 4, s = p - 4;
+      cp_async<V>(r, w.u + (e >= 0 && e < w.N ? e : 0) * w.st, e >= 0 && e < w.N);
+      const bool in = p >= w.r0 && p < w.r1;
+      cp_async<V>(r + kThreads, c.m1 + w.m + (in ? p - w.r0 : 0) * w.sc, in);
+      if (s >= w.s0) {
+        cp_async<V>(r + 2 * kThreads, c.m2 + w.m + (s - w.r0) * w.sc, true);
+        if (w.add) cp_async<V>(r + 3 * kThreads, w.E + s * w.st, true);
       }
     }
+    cp_commit();
+  };
+  for (int k = 0; k < kDepth - 1; ++k) issue(p0 + k);
+  float uq[13][V], pq[9][V];  // u(p - 8 .. p + 4), Psi'(p - 8 .. p)
+#pragma unroll
+  for (int k = 1; k < 13; ++k) {
+    const int e = p0 - 9 + k;
+    T t{};
+    if (k > 4 && e >= 0 && e < w.N) t = *reinterpret_cast<const T*>(w.u + e * w.st);
+    unpack<V>(t, uq[k]);
   }
-}
-
-template <int A>
-__global__ void __launch_bounds__(256, 3) fcorr_march_kernel(CpmlArgs c) {
-  const VolDesc V = c.vols[blockIdx.y];
-  Slab<A> S;
-  if (!S.init(V, c, V.border + 4)) return;
-  const int N = A == 2 ? V.Nz : V.Ny;
-  for (unsigned q = blockIdx.x * blockDim.x + threadIdx.x; q < S.ncol; q += gridDim.x * blockDim.x) {
-    Pt p = S.column(V, q);
-    const long long i0 = idx(V, p.x, p.y, p.z);
-    const float* Acol = c.A + ((long long)p.z * c.NyG + (p.y + V.cy0)) * c.pitchG + (p.x + V.cx0);
-    float um[9], pm[9];  // u and Psi_A at s - 4 .. s + 4
 #pragma unroll
-    for (int m = 0; m < 9; ++m) {
-      um[m] = sval(c.u, i0, S.st, S.s0 - 4 + m, N);
-      pm[m] = sval(c.m1[A], i0, S.st, S.s0 - 4 + m, N);
+  for (int k = 0; k < 9; ++k)
+#pragma unroll
+    for (int e = 0; e < V; ++e) pq[k][e] = 0.0f;
+  for (int p = p0; p < p1; ++p) {
+    const float bp = __ldg(c.b + w.prof + p), cp = __ldg(c.c + w.prof + p);
+    const int s = p - 4;
+    const float bs = __ldg(c.b + w.prof + s), cs = __ldg(c.c + w.prof + s);
+    cp_wait<kDepth - 2>();
+    const T* r = &ring[(p - p0) % kDepth][0][tid];
+#pragma unroll
+    for (int k = 0; k < 12; ++k)
+#pragma unroll
+      for (int e = 0; e < V; ++e) uq[k][e] = uq[k + 1][e];
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+#pragma unroll
+      for (int e = 0; e < V; ++e) pq[k][e] = pq[k + 1][e];
+    unpack<V>(r[0], uq[12]);
+    unpack<V>(r[kThreads], pq[8]);
+    issue(p + kDepth - 1);  // into the slot whose values the last step has used
+    if (cp != 0.0f || bp != 1.0f) {
+#pragma unroll
+      for (int e = 0; e < V; ++e) pq[8][e] = fmaf(bp, pq[8][e], cp * D1Q(uq, 8, e));
     }
-    for (int sg = S.s0; sg < S.s1; sg += kZG) {
-      float zt[kZG], o[kZG], ag[kZG], un[kZG], pn[kZG], b[kZG], cc[kZG];
+    if (p >= w.s0 && p < w.s1)
+      *reinterpret_cast<T*>(c.m1n + w.m + (p - w.r0) * w.sc) = pack<V>(pq[8]);
+    if (s >= w.s0) {
+      float z[V], ev[V];
+      unpack<V>(r[2 * kThreads], z);
 #pragma unroll
-      for (int k = 0; k < kZG; ++k) {
-        const int s = sg + k;
-        const bool in = s < S.s1;
-        b[k] = 1.0f;
-        cc[k] = 0.0f;
-        if (in) Slab<A>::profile(c.pr, V, s, b[k], cc[k]);
-        zt[k] = in_layer(b[k], cc[k]) ? c.m2[A][i0 + s * S.st] : 0.0f;
-        o[k] = in ? c.out[i0 + s * S.st] : 0.0f;
-        ag[k] = in ? __ldg(Acol + s * S.stA) : 0.0f;
-        un[k] = sval(c.u, i0, S.st, s + 5, N);
-        pn[k] = sval(c.m1[A], i0, S.st, s + 5, N);
-      }
+      for (int e = 0; e < V; ++e) ev[e] = D1Q(pq, 4, e);
+      if (cs != 0.0f || bs != 1.0f) {
 #pragma unroll
-      for (int k = 0; k < kZG; ++k) {
-        const int s = sg + k;
-        if (s < S.s1) {  // every slab point is within border + 4 cells of a face across A
-          const long long i = i0 + s * S.st;
-          const float d1p = d1q(pm);
-          float zn = 0.0f;
-          if (in_layer(b[k], cc[k])) {
-            zn = fmaf(b[k], zt[k], cc[k] * (d2q(um) + d1p));
-            c.m2[A][i] = zn;
-          }
-          const float d = ag[k] * (d1p + zn);
-          c.out[i] = o[k] + d;
-          if (c.tstore) {
-            Slab<A>::at(p, s);
-            const long long r = region_index(V, p);
-            if (r >= 0) c.tstore[r] += d;
-          }
+        for (int e = 0; e < V; ++e) {
+          z[e] = fmaf(bs, z[e], cs * (D2Q(uq, 4, e) + ev[e]));
+          ev[e] += z[e];
         }
-        shift(um, un[k]);
-        shift(pm, pn[k]);
+        *reinterpret_cast<T*>(c.m2n + w.m + (s - w.r0) * w.sc) = pack<V>(z);
       }
+      if (w.add) {
+        float o[V];
+        unpack<V>(r[3 * kThreads], o);
+#pragma unroll
+        for (int e = 0; e < V; ++e) ev[e] += o[e];
+      }
+      *reinterpret_cast<T*>(w.E + s * w.st) = pack<V>(ev);
     }
   }
 }
 
-__global__ void psi_x_kernel(CpmlArgs c) {
-  const VolDesc V = c.vols[blockIdx.y];
-  for_xslab(V, V.border, [&](Pt p) {
-    const long long i = idx(V, p.x, p.y, p.z);
-    float b, cc;
-    prof(c.pr, V, p, 0, b, cc);
-    if (in_layer(b, cc)) c.m1[0][i] = fmaf(b, c.m1[0][i], cc * d1(c.u, V, p, 0, i));
-  });
-}
-
-__global__ void fcorr_x_kernel(CpmlArgs c) {
-  const VolDesc V = c.vols[blockIdx.y];
-  for_xslab(V, V.border + 4, [&](Pt p) {
-    const long long i = idx(V, p.x, p.y, p.z);
-    const float d1p = d1(c.m1[0], V, p, 0, i);
-    float b, cc;
-    prof(c.pr, V, p, 0, b, cc);
-    float zt = 0.0f;
-    if (in_layer(b, cc)) {
-      zt = fmaf(b, c.m2[0][i], cc * (d2(c.u, V, p, 0, i) + d1p));
-      c.m2[0][i] = zt;
-    }
-    const float d = coefA(c, V, p) * (d1p + zt);
-    c.out[i] += d;
-    if (c.tstore) {
-      const long long r = region_index(V, p);
-      if (r >= 0) c.tstore[r] += d;
-    }
-  });
-}
-
-__global__ void record_kernel(const float* __restrict__ u, const long long* __restrict__ node,
-                              const RecEntry* __restrict__ rec, int ncol, float* __restrict__ dout) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c < ncol) dout[c] = rec[c].fscale * u[node[c]];
-}
-
-// ---------------------------------------------------------------- reverse
-//
-// One launch per axis and update, as in the forward pass.  For z and y one
-// marched kernel forms both multipliers: y_a is pointwise, so it is made as
-// each cell enters the register queue (its Zeta multiplier updated in the
-// same place), and p_a once the cell's neighbours along a are in the queue.
-// Where the two layers along a are less than 8 cells apart, one thread
-// marches the whole column, so that no queue reads a y_a another thread is
-// making.  For x, y_x comes from a pointwise kernel and p_x from one point
-// per thread.  The correction adds each axis's part to psi^k and to the
-// imaging accumulator in turn.
-
-// Profile of cell s along A (b = 1, c = 0 outside the window).
+// Reverse, axes z and y: at step e cell e enters (y, psi + y and its Zeta
+// multiplier), p = e - 4 gets its Psi multiplier and z, and s = e - 8 is
+// finished.  Two x cells per thread: the three queues hold 31 values a cell.
 template <int A>
-__device__ __forceinline__ void prof_at(const CpmlProf& pr, const VolDesc& V, int N, int s, float& b,
-                                        float& cc) {
-  b = 1.0f;
-  cc = 0.0f;
-  if (s >= 0 && s < N) Slab<A>::profile(pr, V, s, b, cc);
-}
-
-template <int A>
-__global__ void __launch_bounds__(256, 2) pre_march_kernel(CpmlArgs c) {
-  const VolDesc V = c.vols[blockIdx.y];
-  Slab<A> S;
-  if (!S.init(V, c, V.border, true)) return;
-  const int N = A == 2 ? V.Nz : V.Ny;
-  for (unsigned q = blockIdx.x * blockDim.x + threadIdx.x; q < S.ncol; q += gridDim.x * blockDim.x) {
-    const Pt p = S.column(V, q);
-    const long long i0 = idx(V, p.x, p.y, p.z);
-    // y_A of a cell entering the queue, c (Zb + psi) with Zb <- b (Zb + psi)
-    // in the layer, zero elsewhere (zb: the cell's Zeta multiplier)
-    auto enter = [&](int s, float psi, float zb, float b, float cc) -> float {
-      if (!in_layer(b, cc)) return 0.0f;
-      const long long i = i0 + s * S.st;
-      const float zt = zb + psi;
-      const float y = cc * zt;
-      c.y[A][i] = y;
-      c.m2[A][i] = b * zt;
-      return y;
-    };
-    float ps[9], yq[9];  // psi^{k+1} and y_A at s - 4 .. s + 4
-#pragma unroll
-    for (int m = 0; m < 9; ++m) {
-      const int s = S.s0 - 4 + m;
-      float b, cc;
-      prof_at<A>(c.pr, V, N, s, b, cc);
-      ps[m] = sval(c.u, i0, S.st, s, N);
-      const float zb = in_layer(b, cc) ? c.m2[A][i0 + s * S.st] : 0.0f;
-      yq[m] = enter(s, ps[m], zb, b, cc);
+__global__ void __launch_bounds__(kThreads, 4) rev_march_kernel(CpmlArgs c, int chunk, int first) {
+  constexpr int V = 2;
+  using T = VecT<V>::T;
+  __shared__ T ring[kDepth][4][kThreads];  // psi, Zb, Pb, E
+  March<A, V> w;
+  if (!w.init(c, chunk, first)) return;
+  const int tid = threadIdx.x;
+  const int e0 = w.s0 - 8, e1 = w.s1 + 8;
+  auto issue = [&](int e) {
+    if (e < e1) {
+      T* r = &ring[(e - e0) % kDepth][0][tid];
+      const bool inw = e >= 0 && e < w.N, in = e >= w.r0 && e < w.r1;
+      cp_async<V>(r, w.u + (inw ? e : 0) * w.st, inw);
+      cp_async<V>(r + kThreads, c.m2 + w.m + (in ? e - w.r0 : 0) * w.sc, in);
+      const int p = e - 4, s = e - 8;
+      const bool inp = p >= w.r0 && p < w.r1;
+      cp_async<V>(r + 2 * kThreads, c.m1 + w.m + (inp ? p - w.r0 : 0) * w.sc, inp);
+      if (w.add && s >= w.s0) cp_async<V>(r + 3 * kThreads, w.E + s * w.st, true);
     }
-    for (int sg = S.s0; sg < S.s1; sg += kZG) {
-      // loads of the group: the cells entering (sg + 5 ..) and finishing (sg ..)
-      float pn[kZG], zb[kZG], be[kZG], ce[kZG], mv[kZG], bf[kZG], cf[kZG];
+    cp_commit();
+  };
+  for (int k = 0; k < kDepth - 1; ++k) issue(e0 + k);
+  float yq[13][V], vq[9][V], zq[9][V];  // y(e - 12 .. e), (psi + y)(e - 8 .. e), z(e - 12 .. e - 4)
 #pragma unroll
-      for (int k = 0; k < kZG; ++k) {
-        const int e = sg + 5 + k, f = sg + k;
-        prof_at<A>(c.pr, V, N, e, be[k], ce[k]);
-        pn[k] = sval(c.u, i0, S.st, e, N);
-        zb[k] = in_layer(be[k], ce[k]) ? c.m2[A][i0 + e * S.st] : 0.0f;
-        prof_at<A>(c.pr, V, f < S.s1 ? N : 0, f, bf[k], cf[k]);
-        mv[k] = in_layer(bf[k], cf[k]) ? c.m1[A][i0 + f * S.st] : 0.0f;
-      }
+  for (int v = 0; v < V; ++v) {
 #pragma unroll
-      for (int k = 0; k < kZG; ++k) {
-        if (in_layer(bf[k], cf[k])) {
-          const long long i = i0 + (sg + k) * S.st;
-          const float pt = mv[k] - (d1q(ps) + d1q(yq));
-          c.m1[A][i] = bf[k] * pt;
-          c.z[A][i] = cf[k] * pt;
-        }
-        const float ye = enter(sg + 5 + k, pn[k], zb[k], be[k], ce[k]);
-        shift(ps, pn[k]);
-        shift(yq, ye);
+    for (int k = 0; k < 13; ++k) yq[k][v] = 0.0f;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) vq[k][v] = zq[k][v] = 0.0f;
+  }
+  for (int e = e0; e < e1; ++e) {
+    const int p = e - 4, s = e - 8;
+    const float be = __ldg(c.b + w.prof + e), ce = __ldg(c.c + w.prof + e);
+    const float bp = __ldg(c.b + w.prof + p), cp = __ldg(c.c + w.prof + p);
+    cp_wait<kDepth - 2>();
+    const T* r = &ring[(e - e0) % kDepth][0][tid];
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+#pragma unroll
+      for (int k = 0; k < 12; ++k) yq[k][v] = yq[k + 1][v];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        vq[k][v] = vq[k + 1][v];
+        zq[k][v] = zq[k + 1][v];
       }
+      yq[12][v] = zq[8][v] = 0.0f;
+    }
+    unpack<V>(r[0], vq[8]);
+    issue(e + kDepth - 1);  // into the slot whose values the last step has used
+    if (ce != 0.0f || be != 1.0f) {
+      float zb[V];
+      unpack<V>(r[kThreads], zb);
+#pragma unroll
+      for (int v = 0; v < V; ++v) {
+        const float zt = zb[v] + vq[8][v];
+        yq[12][v] = ce * zt;
+        vq[8][v] += yq[12][v];
+        zb[v] = be * zt;
+      }
+      if (e >= w.s0 && e < w.s1)
+        *reinterpret_cast<T*>(c.m2n + w.m + (e - w.r0) * w.sc) = pack<V>(zb);
+    }
+    if (cp != 0.0f || bp != 1.0f) {
+      float pb[V];
+      unpack<V>(r[2 * kThreads], pb);
+#pragma unroll
+      for (int v = 0; v < V; ++v) {
+        const float pt = pb[v] - D1Q(vq, 4, v);
+        zq[8][v] = cp * pt;
+        pb[v] = bp * pt;
+      }
+      if (p >= w.s0 && p < w.s1)
+        *reinterpret_cast<T*>(c.m1n + w.m + (p - w.r0) * w.sc) = pack<V>(pb);
+    }
+    if (s >= w.s0) {
+      float ev[V];
+#pragma unroll
+      for (int v = 0; v < V; ++v) ev[v] = D2Q(yq, 4, v) - D1Q(zq, 4, v);
+      if (w.add) {
+        float o[V];
+        unpack<V>(r[3 * kThreads], o);
+#pragma unroll
+        for (int v = 0; v < V; ++v) ev[v] += o[v];
+      }
+      *reinterpret_cast<T*>(w.E + s * w.st) = pack<V>(ev);
     }
   }
 }
 
-template <int A>
-__global__ void __launch_bounds__(256, 3) acorr_march_kernel(CpmlArgs c) {
-  const VolDesc V = c.vols[blockIdx.y];
-  Slab<A> S;
-  if (!S.init(V, c, V.border + 4)) return;
-  const int N = A == 2 ? V.Nz : V.Ny;
-  for (unsigned q = blockIdx.x * blockDim.x + threadIdx.x; q < S.ncol; q += gridDim.x * blockDim.x) {
-    Pt p = S.column(V, q);
-    const long long i0 = idx(V, p.x, p.y, p.z);
-    const float* Acol = c.A + ((long long)p.z * c.NyG + (p.y + V.cy0)) * c.pitchG + (p.x + V.cx0);
-    float yq[9], zq[9];  // y_A and z_A at s - 4 .. s + 4
-#pragma unroll
-    for (int m = 0; m < 9; ++m) {
-      yq[m] = sval(c.y[A], i0, S.st, S.s0 - 4 + m, N);
-      zq[m] = sval(c.z[A], i0, S.st, S.s0 - 4 + m, N);
-    }
-    for (int sg = S.s0; sg < S.s1; sg += kZG) {
-      float yn[kZG], zn[kZG], o[kZG], ac[kZG], ag[kZG], ts[kZG];
-      long long r[kZG];
-#pragma unroll
-      for (int k = 0; k < kZG; ++k) {
-        const int f = sg + k;
-        const bool in = f < S.s1;
-        const long long i = i0 + f * S.st;
-        yn[k] = sval(c.y[A], i0, S.st, f + 5, N);
-        zn[k] = sval(c.z[A], i0, S.st, f + 5, N);
-        o[k] = in ? c.out[i] : 0.0f;
-        ag[k] = in ? __ldg(Acol + f * S.stA) : 0.0f;
-        Slab<A>::at(p, f);
-        r[k] = in ? region_index(V, p) : -1;
-        ts[k] = r[k] >= 0 ? __ldg(c.tstore + r[k]) : 0.0f;
-        ac[k] = r[k] >= 0 ? c.acc[i] : 0.0f;
-      }
-#pragma unroll
-      for (int k = 0; k < kZG; ++k) {
-        if (sg + k < S.s1) {  // every slab point is within border + 4 cells of a face across A
-          const long long i = i0 + (sg + k) * S.st;
-          const float d = ag[k] * (d2q(yq) - d1q(zq));
-          c.out[i] = o[k] + d;
-          if (r[k] >= 0) c.acc[i] = fmaf(d, ts[k], ac[k]);
-        }
-        shift(yq, yn[k]);
-        shift(zq, zn[k]);
-      }
-    }
+// One thread's 4 cells of the x slabs: x0 (a multiple of 4) of row (y, z).
+struct XCell {
+  int x0, r0, r1, n4;  // slab region [r0, r1) of the cells; row length rounded up to 4
+  bool add;
+  long long f, m;  // field element of the row's start; slab-array element of cell r0
+  int prof;
+  __device__ __forceinline__ bool init(const CpmlArgs& c) {
+    const VolDesc& D = c.vols[blockIdx.y];
+    const CpmlVol& W = c.cv[blockIdx.y];
+    const unsigned G = (unsigned)W.n[0] / 4;
+    if (G == 0) return false;
+    const unsigned q = blockIdx.x * kThreads + threadIdx.x;
+    const unsigned row = q / G;
+    const unsigned z = row / (unsigned)D.Ny;
+    if (z >= (unsigned)D.Nz) return false;
+    const int y = (int)(row - z * (unsigned)D.Ny), sl = (int)(q - row * G) * 4;
+    const int lo = W.lo[0], hi = W.hi[0];
+    n4 = (D.Nx + 3) & ~3;
+    const bool low = sl < lo;
+    r0 = low ? 0 : hi;
+    r1 = low && lo != hi ? lo : n4;
+    if (lo == hi) r0 = 0;
+    x0 = low || lo == hi ? sl : sl - lo + hi;
+    f = D.off + (long long)row * D.pitch;
+    m = W.off[0] + (long long)row * W.n[0] + (r0 == 0 ? 0 : lo);
+    prof = W.prof[0] + kCpmlPad + x0;
+    add = y < W.lo[1] || y >= W.hi[1] || (int)z < W.lo[2] || (int)z >= W.hi[2];
+    return true;
   }
+  // 4 values at x0 + 4 k: of a field (zero outside the row) or a slab array
+  // (zero outside the region).
+  __device__ __forceinline__ float4 field(const float* a, int k) const {
+    const int x = x0 + 4 * k;
+    return (x >= 0 && x < n4) ? __ldg(reinterpret_cast<const float4*>(a + f + x))
+                              : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  __device__ __forceinline__ float4 slab(const float* a, int k) const {
+    const int x = x0 + 4 * k;
+    return (x >= r0 && x < r1) ? __ldg(reinterpret_cast<const float4*>(a + m + (x - r0)))
+                               : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  __device__ __forceinline__ void store(float* a, const float (&v)[4]) const {
+    *reinterpret_cast<float4*>(a + m + (x0 - r0)) = make_float4(v[0], v[1], v[2], v[3]);
+  }
+};
+
+__device__ __forceinline__ void put(float* d, const float4& t) {
+  d[0] = t.x;
+  d[1] = t.y;
+  d[2] = t.z;
+  d[3] = t.w;
 }
 
-__global__ void y_x_kernel(CpmlArgs c) {
-  const VolDesc V = c.vols[blockIdx.y];
-  for_xslab(V, V.border, [&](Pt p) {
-    const long long i = idx(V, p.x, p.y, p.z);
-    float b, cc;
-    prof(c.pr, V, p, 0, b, cc);
-    if (in_layer(b, cc)) {
-      const float zt = c.m2[0][i] + c.u[i];
-      c.y[0][i] = cc * zt;
-      c.m2[0][i] = b * zt;
-    }
-  });
+__device__ __forceinline__ void profile4(const float* p, float* d) {
+  put(d, __ldg(reinterpret_cast<const float4*>(p)));
 }
 
-__global__ void z_x_kernel(CpmlArgs c) {
-  const VolDesc V = c.vols[blockIdx.y];
-  for_xslab(V, V.border, [&](Pt p) {
-    const long long i = idx(V, p.x, p.y, p.z);
-    float b, cc;
-    prof(c.pr, V, p, 0, b, cc);
-    if (in_layer(b, cc)) {
-      const float pt = c.m1[0][i] - (d1(c.u, V, p, 0, i) + d1(c.y[0], V, p, 0, i));
-      c.m1[0][i] = b * pt;
-      c.z[0][i] = cc * pt;
-    }
-  });
+// x slabs: 4 cells per thread, the neighbours in 16-byte loads that mostly hit
+// the lines of the neighbouring threads (5 of the field, 3 of Psi for the 12
+// Psi' of the cell's own D1), no exchange between threads.
+__global__ void __launch_bounds__(kThreads) fwd_x_kernel(CpmlArgs c) {
+  XCell w;
+  if (!w.init(c)) return;
+  float u[20], ps[12], b[12], cc[12], z[4], ev[4];
+#pragma unroll
+  for (int k = 0; k < 5; ++k) put(u + 4 * k, w.field(c.u, k - 2));
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    put(ps + 4 * k, w.slab(c.m1, k - 1));
+    profile4(c.b + w.prof + 4 * (k - 1), b + 4 * k);
+    profile4(c.c + w.prof + 4 * (k - 1), cc + 4 * k);
+  }
+  // Zeta is updated in place by its own thread alone: a plain load
+  put(z, *reinterpret_cast<const float4*>(c.m2 + w.m + (w.x0 - w.r0)));
+  float4 old = make_float4(0.f, 0.f, 0.f, 0.f);
+  float4* Ep = reinterpret_cast<float4*>(c.E + w.f + w.x0);
+  if (w.add) old = *Ep;
+#pragma unroll
+  for (int k = 0; k < 12; ++k) ps[k] = fmaf(b[k], ps[k], cc[k] * D1R(u, k + 4));
+  const float pn[4] = {ps[4], ps[5], ps[6], ps[7]};
+  w.store(c.m1n, pn);
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    const float d1p = D1R(ps, e + 4);
+    z[e] = fmaf(b[e + 4], z[e], cc[e + 4] * (D2R(u, e + 8) + d1p));
+    ev[e] = d1p + z[e];
+  }
+  w.store(c.m2n, z);
+  *Ep = make_float4(old.x + ev[0], old.y + ev[1], old.z + ev[2], old.w + ev[3]);
 }
 
-__global__ void acorr_x_kernel(CpmlArgs c) {
-  const VolDesc V = c.vols[blockIdx.y];
-  for_xslab(V, V.border + 4, [&](Pt p) {
-    const long long i = idx(V, p.x, p.y, p.z);
-    const float d = coefA(c, V, p) * (d2(c.y[0], V, p, 0, i) - d1(c.z[0], V, p, 0, i));
-    c.out[i] += d;
-    const long long r = region_index(V, p);
-    if (r >= 0) c.acc[i] = fmaf(d, c.tstore[r], c.acc[i]);
-  });
+__global__ void __launch_bounds__(kThreads) rev_x_kernel(CpmlArgs c) {
+  XCell w;
+  if (!w.init(c)) return;
+  float v[20], y[20], cc[20], z[12], b[4];
+#pragma unroll
+  for (int k = 0; k < 5; ++k) {
+    put(v + 4 * k, w.field(c.u, k - 2));
+    put(y + 4 * k, w.slab(c.m2, k - 2));
+    profile4(c.c + w.prof + 4 * (k - 2), cc + 4 * k);
+  }
+#pragma unroll
+  for (int k = 0; k < 3; ++k) put(z + 4 * k, w.slab(c.m1, k - 1));
+  profile4(c.b + w.prof, b);
+  float4 old = make_float4(0.f, 0.f, 0.f, 0.f);
+  float4* Ep = reinterpret_cast<float4*>(c.E + w.f + w.x0);
+  if (w.add) old = *Ep;
+  float nz[4], np[4];
+#pragma unroll
+  for (int k = 0; k < 20; ++k) {
+    const float zt = y[k] + v[k];
+    if (k >= 8 && k < 12) nz[k - 8] = cc[k] != 0.0f || b[k - 8] != 1.0f ? b[k - 8] * zt : 0.0f;
+    y[k] = cc[k] * zt;
+    v[k] += y[k];
+  }
+#pragma unroll
+  for (int k = 0; k < 12; ++k) {
+    const float pt = z[k] - D1R(v, k + 4);
+    if (k >= 4 && k < 8) np[k - 4] = cc[k + 4] != 0.0f || b[k - 4] != 1.0f ? b[k - 4] * pt : 0.0f;
+    z[k] = cc[k + 4] * pt;
+  }
+  w.store(c.m2n, nz);
+  w.store(c.m1n, np);
+  float ev[4];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) ev[e] = D2R(y, e + 8) - D1R(z, e + 4);
+  *Ep = make_float4(old.x + ev[0], old.y + ev[1], old.z + ev[2], old.w + ev[3]);
 }
 
-dim3 grid_for(int n_vol, long long max_pts) {
-  long long b = (max_pts + 255) / 256;
-  const long long cap = std::max(1LL, 152LL * 16 / n_vol);
-  if (b > cap) b = cap;
-  return dim3((unsigned)(b < 1 ? 1 : b), (unsigned)n_vol);
+// Threads that a marching launch should have: enough columns leave the slabs
+// whole (a cut makes 8 or 16 cells of the neighbouring piece again); with
+// fewer, the slabs are cut into pieces of at least 3 cells.
+constexpr long long kMarchThreads = 152LL * 512;
+
+int piece(const CpmlExtent& e, int a) {
+  long long cuts = std::max(1LL, kMarchThreads / std::max(1LL, e.threads[a]));
+  cuts = std::min<long long>(cuts, std::max(1, e.len[a] / 3));
+  return std::max(1, (int)((e.len[a] + cuts - 1) / cuts));
+}
+
+// Grid of a marching launch: columns of V cells, windows, pieces of both slabs.
+dim3 march_grid(const CpmlExtent& e, int a, int V, int chunk) {
+  const long long threads = e.cols[a] * (4 / V);
+  return dim3((unsigned)((threads + kThreads - 1) / kThreads), (unsigned)e.nvol,
+              (unsigned)(2 * ((e.len[a] + chunk - 1) / chunk)));
+}
+
+template <int A>
+void forward_axis(const CpmlArgs& c, const CpmlExtent& e, cudaStream_t s) {
+  if (e.len[A] <= 0) return;
+  int k = piece(e, A);
+  if (!e.apart) {
+    fwd_march_kernel<A><<<march_grid(e, A, 4, k), kThreads, 0, s>>>(c, k, 0);
+    return;
+  }
+  k = A == 2 ? (e.len[A] + 1) / 2 : e.len[A];
+  dim3 g = march_grid(e, A, 4, k);
+  const int n = g.z;
+  g.z = 1;
+  for (int i = 0; i < n; ++i) fwd_march_kernel<A><<<g, kThreads, 0, s>>>(c, k, i);
+}
+
+template <int A>
+void reverse_axis(const CpmlArgs& c, const CpmlExtent& e, cudaStream_t s) {
+  if (e.len[A] <= 0) return;
+  const int k = piece(e, A);
+  rev_march_kernel<A><<<march_grid(e, A, 2, k), kThreads, 0, s>>>(c, k, 0);
+}
+
+dim3 x_grid(const CpmlExtent& e) {
+  return dim3((unsigned)((e.cols[0] + kThreads - 1) / kThreads), (unsigned)e.nvol);
 }
 
 }  // namespace
 
-// Both slabs of a marched axis (blockIdx.z), one thread per column.
-dim3 march_grid(int n_vol, long long max_cols) {
-  const long long b = std::min((max_cols + 255) / 256, 65535LL);
-  return dim3((unsigned)std::max(1LL, b), (unsigned)n_vol, 2);
+int cpml_launches(const CpmlExtent& e) {
+  int n = e.cols[0] > 0 ? 1 : 0;
+  for (int a = 1; a < 3; ++a)
+    if (e.len[a] > 0) {
+      const int k = e.apart ? (a == 2 ? (e.len[a] + 1) / 2 : e.len[a]) : 1;
+      n += e.apart ? 2 * ((e.len[a] + k - 1) / k) : 1;
+    }
+  return n;
 }
 
-cudaError_t launch_cpml_psi(const CpmlArgs& c, int n_vol, const CpmlExtent& e, cudaStream_t s) {
-  psi_march_kernel<2><<<march_grid(n_vol, e.xy), 256, 0, s>>>(c);
-  psi_march_kernel<1><<<march_grid(n_vol, e.xz), 256, 0, s>>>(c);
-  psi_x_kernel<<<grid_for(n_vol, 2LL * e.border * e.yz), 256, 0, s>>>(c);
+cudaError_t launch_cpml_forward(const CpmlArgs& c, const CpmlExtent& e, cudaStream_t s) {
+  forward_axis<2>(c, e, s);
+  forward_axis<1>(c, e, s);
+  if (e.cols[0] > 0) fwd_x_kernel<<<x_grid(e), kThreads, 0, s>>>(c);
   return cudaGetLastError();
 }
 
-cudaError_t launch_cpml_fcorr(const CpmlArgs& c, int n_vol, const CpmlExtent& e, cudaStream_t s) {
-  fcorr_march_kernel<2><<<march_grid(n_vol, e.xy), 256, 0, s>>>(c);
-  fcorr_march_kernel<1><<<march_grid(n_vol, e.xz), 256, 0, s>>>(c);
-  fcorr_x_kernel<<<grid_for(n_vol, 2LL * (e.border + 4) * e.yz), 256, 0, s>>>(c);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_cpml_pre(const CpmlArgs& c, int n_vol, const CpmlExtent& e, cudaStream_t s) {
-  pre_march_kernel<2><<<march_grid(n_vol, e.xy), 256, 0, s>>>(c);
-  pre_march_kernel<1><<<march_grid(n_vol, e.xz), 256, 0, s>>>(c);
-  const dim3 g = grid_for(n_vol, 2LL * e.border * e.yz);
-  y_x_kernel<<<g, 256, 0, s>>>(c);
-  z_x_kernel<<<g, 256, 0, s>>>(c);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_cpml_acorr(const CpmlArgs& c, int n_vol, const CpmlExtent& e, cudaStream_t s) {
-  acorr_march_kernel<2><<<march_grid(n_vol, e.xy), 256, 0, s>>>(c);
-  acorr_march_kernel<1><<<march_grid(n_vol, e.xz), 256, 0, s>>>(c);
-  acorr_x_kernel<<<grid_for(n_vol, 2LL * (e.border + 4) * e.yz), 256, 0, s>>>(c);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_cpml_record(const float* u, const long long* node, const RecEntry* rec, int ncol,
-                               float* dout, cudaStream_t s) {
-  if (ncol <= 0) return cudaSuccess;
-  record_kernel<<<(ncol + 127) / 128, 128, 0, s>>>(u, node, rec, ncol, dout);
+cudaError_t launch_cpml_reverse(const CpmlArgs& c, const CpmlExtent& e, cudaStream_t s) {
+  reverse_axis<2>(c, e, s);
+  reverse_axis<1>(c, e, s);
+  if (e.cols[0] > 0) rev_x_kernel<<<x_grid(e), kThreads, 0, s>>>(c);
   return cudaGetLastError();
 }
 

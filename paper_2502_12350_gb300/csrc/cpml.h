@@ -1,11 +1,9 @@
 // Launch interface of the convolutional-PML kernels (internal to libmamute).
 //
-// The CPML scheme is run as the damping-free main step (the TMA stencil
-// kernels with g = 1, which form the whole update away from the layer) plus
-// these kernels, which touch only the layer slabs of each shot window where
-// the memory variables live or are read: per axis the `border` layer cells
-// of its two faces, and 4 more cells inward where the eighth-order
-// derivatives of the memory variables reach.
+// A CPML step is one launch per axis over that axis's layer slabs, which
+// updates the memory variables and leaves their contribution to the second
+// derivative in the array E, followed by the main step kernel, which adds E
+// to its 25-point sum (StepArgs, step_kernel<..., PML>).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -14,58 +12,55 @@
 
 namespace mamute {
 
-// Per-axis layer coefficients b = exp(-(d + alpha) dt), c = d (b - 1) / (d + alpha):
-// x and y profiles of every shot window (at VolDesc gx_off / gy_off), z shared.
-struct CpmlProf {
-  const float* bx;
-  const float* cx;
-  const float* by;
-  const float* cy;
-  const float* bz;
-  const float* cz;
+// The slabs of one shot window: along axis a (0: x, 1: y, 2: z) the cells
+// [0, lo) and [hi, N) within border + 4 of a face that has a layer (the layer
+// and the 4 cells that the eighth-order derivatives of the memory variables
+// reach); hi == lo is one range [0, N).  Along x both ends are widened to
+// multiples of 4.  Memory variables are stored on the slabs only, n cells
+// along the axis (slot s, or s - hi + lo in the upper slab):
+//   z: [slot][Ny][pitch]   y: [Nz][slot][pitch]   x: [Nz][Ny][slot]
+// at element off of each array.
+struct CpmlVol {
+  int lo[3], hi[3], n[3];
+  long long off[3];
+  int prof[3];  // the axis's b and c of cell s at CpmlArgs::b / c [prof + kCpmlPad + s]
 };
+// Cells before and after each profile (c = 0, b = 1), so that a thread may
+// read the profile of the cells around its own without a bounds test.
+constexpr int kCpmlPad = 12;
 
-// Fields of one CPML launch, all in the pool layout of the shot windows
-// (blockIdx.y selects the window) except A (global padded grid) and the
-// term store / accumulator (imaging-region layout).
 struct CpmlArgs {
   const VolDesc* vols;
-  CpmlProf pr;
-  const float* A;      // c^2 dt^2 / h^2 on the global padded grid
-  int pitchG, NyG;     // layout of A
-  const float* u;      // forward: u^n; reverse: the adjoint level being propagated (psi^{k+1})
-  float* out;          // the main kernel's new level, corrected in place
-  float* m1[3];        // forward: Psi_a (first memory variable, scaled by h); reverse: its multiplier
-  float* m2[3];        // forward: Zeta_a (scaled by h^2); reverse: its multiplier
-  float* y[3];         // reverse scratch: c_a (multiplier of Zeta_a + psi)
-  float* z[3];         // reverse scratch: c_a p_a
-  float* tstore;       // imaging term of this step (corrected in place, forward) or read (reverse); may be null
-  float* acc;          // reverse: imaging accumulator (pool layout, corrected in place)
+  const CpmlVol* cv;
+  const float* b;    // b = exp(-(d + alpha) dt), see CpmlVol::prof
+  const float* c;    // c = d (b - 1) / (d + alpha)
+  const float* u;    // forward: u^n; reverse: the adjoint level being propagated (pool layout)
+  // Memory variables before and after the step; forward: Psi and Zeta (updated
+  // in place: m2 == m2n); reverse: their multipliers.  m1 and m1n differ (a
+  // thread reads its neighbours' old values), in the reverse m2 and m2n too.
+  const float* m1;
+  float* m1n;
+  const float* m2;
+  float* m2n;
+  float* E;          // sum over the axes (pool layout); zero outside the slabs
 };
 
-// Largest extents over the shot windows, for the grids of the forward kernels.
+// Grid extents of the slab launches over all shot windows.
 struct CpmlExtent {
-  long long xy, xz, yz;  // Nx Ny, Nx Nz and Ny Nz of a window
-  int border;            // layer width in cells
+  int nvol;
+  long long cols[3];  // threads across the axis, at most: x: rows x groups of 4 slots
+  int len[3];         // longest slab along the axis (y, z)
+  long long threads[3];  // threads of a launch with unsplit slabs, over all windows (y, z)
+  bool apart;            // modelling on tiny windows: each piece of a slab is a launch of its own
 };
 
-// Forward, before the main step: Psi_a <- b_a Psi_a + c_a D1_a u^n in the layer
-// (one launch per axis: kCpmlAxisLaunches).
-cudaError_t launch_cpml_psi(const CpmlArgs& c, int n_vol, const CpmlExtent& e, cudaStream_t s);
-// Forward, after the main step: Zeta_a <- b_a Zeta_a + c_a (D2_a u^n + D1_a Psi_a) in the layer,
-// u^{n+1} += A sum_a (D1_a Psi_a + Zeta_a) and the stored term likewise (one launch per axis).
-cudaError_t launch_cpml_fcorr(const CpmlArgs& c, int n_vol, const CpmlExtent& e, cudaStream_t s);
-constexpr int kCpmlAxisLaunches = 3;
-// Reverse, before the main adjoint step: y_a, the Zeta multipliers, then p_a,
-// the Psi multipliers and z_a, from the level psi^{k+1} (kCpmlPreLaunches
-// launches: the marched z and y kernels, then y_x and p_x).
-cudaError_t launch_cpml_pre(const CpmlArgs& c, int n_vol, const CpmlExtent& e, cudaStream_t s);
-constexpr int kCpmlPreLaunches = 4;
-// Reverse, after the main adjoint step: psi^k += A sum_a (D2_a y_a - D1_a z_a)
-// and the imaging accumulator likewise (one launch per axis).
-cudaError_t launch_cpml_acorr(const CpmlArgs& c, int n_vol, const CpmlExtent& e, cudaStream_t s);
-// dout[c] = rec[c].fscale * u[node[c]] for the ncol internal data columns.
-cudaError_t launch_cpml_record(const float* u, const long long* node, const RecEntry* rec, int ncol,
-                               float* dout, cudaStream_t s);
+// Psi_a <- b_a Psi_a + c_a D1_a u, Zeta_a <- b_a Zeta_a + c_a (D2_a u + D1_a Psi_a),
+// E = sum_a (D1_a Psi_a + Zeta_a); cpml_launches() launches.
+cudaError_t launch_cpml_forward(const CpmlArgs& c, const CpmlExtent& e, cudaStream_t s);
+// y_a = c_a (Zb_a + psi), Zb_a <- b_a (Zb_a + psi), p_a = Pb_a - D1_a (psi + y_a),
+// Pb_a <- b_a p_a, E = sum_a (D2_a y_a - D1_a (c_a p_a)); one launch per axis.
+cudaError_t launch_cpml_reverse(const CpmlArgs& c, const CpmlExtent& e, cudaStream_t s);
+// Launches of one launch_cpml_forward call.
+int cpml_launches(const CpmlExtent& e);
 
 }  // namespace mamute

@@ -16,7 +16,10 @@
 // Update (forward and adjoint alike; the adjoint runs the same operator on
 // psi = A g lambda, which makes it the exact transpose of the forward):
 //   out = g (2 u - M u - g prev + A lap u),   M = A m2 (0 without density)
-// with A = c^2 dt^2 / h^2 and lap the unscaled 25-point sum.
+// with A = c^2 dt^2 / h^2 and lap the unscaled 25-point sum.  With the
+// convolutional PML (PML), lap + E takes the place of lap, E the memory
+// variables' part (see cpml.cu), read as one more centre tile on the planes
+// and tiles that meet a layer slab.
 #pragma once
 
 #include "common.cuh"
@@ -93,23 +96,29 @@ __device__ __forceinline__ void lap4(const float* st, int lx, int ly, const F4 (
   }
 }
 
+// ev: the memory variables' part E with the CPML, taken as a term of its own
+// (lap + E, rounded first, would lose the bits that lap carries beyond E).
+template <bool PML>
 __device__ __forceinline__ float update(float u, float prev, float A, float M, float g,
-                                        float lap, bool dens) {
+                                        float lap, float ev, bool dens) {
   float s = __fmaf_rn(2.0f, u, -__fmul_rn(g, prev));
   if (dens) s = __fmaf_rn(-M, u, s);
   s = __fmaf_rn(A, lap, s);
+  if (PML) s = __fmaf_rn(A, ev, s);
   return __fmul_rn(g, s);
 }
 
-// Imaging term A (lap - m2) u in the scheme's units: A lap u - M u.
-__device__ __forceinline__ float img_term(float u, float A, float M, float lap, bool dens) {
+// Imaging term A (lap + E - m2) u in the scheme's units: A lap u + A E - M u.
+template <bool PML>
+__device__ __forceinline__ float img_term(float u, float A, float M, float lap, float ev, bool dens) {
   float t = __fmul_rn(A, lap);
+  if (PML) t = __fmaf_rn(A, ev, t);
   if (dens) t = __fmaf_rn(-M, u, t);
   return t;
 }
 
 // Shared-memory layout and mode traits of one kernel variant.
-template <int TX, int TY, bool DENS, int MODE>
+template <int TX, int TY, bool DENS, int MODE, bool PML>
 struct Layout {
   static constexpr bool ADJ = MODE == MODE_ADJ || MODE == MODE_ADJ_STORED ||
                               MODE == MODE_ADJ_STEP || MODE == MODE_ADJ_TERM;
@@ -120,11 +129,11 @@ struct Layout {
   static constexpr int NCT = (TX / 4) * TY;  // compute threads
   static constexpr int HS = (TX + 2 * kHalo) * (TY + 2 * kHalo);  // halo stage floats
   static constexpr int CS = TX * TY;  // centre tile floats
-  static constexpr int NC = 2 + (DENS ? 1 : 0) + (ACC ? 1 : 0) + NT;  // centre arrays
+  static constexpr int NC = 2 + (DENS ? 1 : 0) + (ACC ? 1 : 0) + NT + (PML ? 1 : 0);  // centre arrays
   // Halo ring depth: 5 planes in use plus 3 ahead (2 ahead where two halo'd
   // fields share each stage or the centre ring is at its widest, to keep two
   // CTAs per SM).
-  static constexpr int NSU = (RECOMP || (NT && DENS)) ? 7 : 8;
+  static constexpr int NSU = (RECOMP || (NT && (DENS || PML))) ? 7 : 8;
   // Centre ring depth: a stage of the imaging launch holds up to 7 tiles, so
   // two of them are as many bytes in flight as four of a plain step.
   static constexpr int NSC = NT ? 2 : (ADJ ? 4 : 3);
@@ -135,7 +144,8 @@ struct Layout {
 // receiver-entry range of the plane.
 struct PlaneInfo {
   float gz;
-  int rb, re, pad;
+  int rb, re;
+  int ext;  // PML: the tile has a non-zero E on this plane
 };
 
 }  // namespace
@@ -170,15 +180,16 @@ struct MinBlocks {
   static constexpr int value = (MODE == MODE_ADJ && TX * TY >= 1024) ? 1 : 2;
 };
 
-template <int TX, int TY, bool DENS, int MODE>
+template <int TX, int TY, bool DENS, int MODE, bool PML>
 __global__ void __launch_bounds__((TX / 4) * TY + 32, (MinBlocks<TX, TY, MODE>::value))
     step_kernel(const StepArgs a) {
-  using LY = Layout<TX, TY, DENS, MODE>;
+  using LY = Layout<TX, TY, DENS, MODE, PML>;
   constexpr bool ADJ = LY::ADJ, RECOMP = LY::RECOMP, ACC = LY::ACC;
   constexpr bool TERM = LY::NT > 0;  // stored imaging terms as centre arrays
   constexpr int NCT = LY::NCT, HS = LY::HS, CS = LY::CS, NSU = LY::NSU, NSC = LY::NSC;
   constexpr int NHALO = LY::NHALO, NC = LY::NC;
   constexpr int CI_PREV = 0, CI_A = 1, CI_M = 2, CI_ACC = DENS ? 3 : 2, CI_T = CI_ACC + 1;
+  constexpr int CI_E = NC - 1;
 
   extern __shared__ __align__(128) unsigned char smem_raw[];
   float* ring = reinterpret_cast<float*>(smem_raw);           // NSU * NHALO * HS
@@ -206,7 +217,10 @@ __global__ void __launch_bounds__((TX / 4) * TY + 32, (MinBlocks<TX, TY, MODE>::
       pi.rb = a.rec_ptr[it.rec_tab + j];
       pi.re = a.rec_ptr[it.rec_tab + j + 1];
     }
-    pi.pad = 0;
+    // E is zero but on the layer slabs: its tile is loaded only where the item
+    // meets one.
+    pi.ext = PML && (x0 < V.ex0 || x0 + it.w > V.ex1 || y0 < V.ey0 || y0 + it.h > V.ey1 ||
+                     zb + j < V.ez0 || zb + j >= V.ez1);
     pinfo[j] = pi;
   }
   if (tid == 0) {
@@ -228,6 +242,7 @@ __global__ void __launch_bounds__((TX / 4) * TY + 32, (MinBlocks<TX, TY, MODE>::
   const CUtensorMap* mapU = a.mU + (long long)it.vol * a.sU;  // forward field for imaging
   const CUtensorMap* mapAcc = &sm->m[ADJ ? 11 : 8];
   const CUtensorMap* mapT = &sm->m[12];
+  const CUtensorMap* mapE = &sm->m[ADJ ? 14 : 13];
   const CUtensorMap* mapA = &a.cmaps->m[0];
   const CUtensorMap* mapM = &a.cmaps->m[1];
 
@@ -241,6 +256,7 @@ __global__ void __launch_bounds__((TX / 4) * TY + 32, (MinBlocks<TX, TY, MODE>::
       if (RECOMP) tmap_acquire(mapU);
       if (ACC) tmap_acquire(mapAcc);
       if (TERM) tmap_acquire(mapT);
+      if (PML) tmap_acquire(mapE);
       const int nu = npl + 2 * kHalo;
       const int cx = V.cx0 + x0, cy = V.cy0 + y0;
       int nF = 0, nC = 0;  // loads issued into the halo and centre rings
@@ -276,7 +292,9 @@ __global__ void __launch_bounds__((TX / 4) * TY + 32, (MinBlocks<TX, TY, MODE>::
             drain();
             return;
           }
-          mbar_arrive_expect_tx(&fullC[c], (NC - (TERM ? kImgSteps - a.nimg : 0)) * CS * 4);
+          const bool ext = PML && pinfo[j].ext;
+          const int absent = (TERM ? kImgSteps - a.nimg : 0) + (PML && !ext ? 1 : 0);
+          mbar_arrive_expect_tx(&fullC[c], (NC - absent) * CS * 4);
           float* cd = cring + c * NC * CS;
           tma_load_3d(cd + CI_PREV * CS, mapP, x0, y0, q, &fullC[c]);
           tma_load_3d(cd + CI_A * CS, mapA, cx, cy, q, &fullC[c]);
@@ -286,6 +304,7 @@ __global__ void __launch_bounds__((TX / 4) * TY + 32, (MinBlocks<TX, TY, MODE>::
             for (int m = 0; m < a.nimg; ++m)
               tma_load_4d(cd + (CI_T + m) * CS, mapT, x0 - V.txoff, y0 - V.iy0, q - V.border,
                           a.tstep + m, &fullC[c]);
+          if (PML && ext) tma_load_3d(cd + CI_E * CS, mapE, x0, y0, q, &fullC[c]);
           ++nC;
         }
       }
@@ -373,12 +392,14 @@ __global__ void __launch_bounds__((TX / 4) * TY + 32, (MinBlocks<TX, TY, MODE>::
     F4 Mv = {{0.f, 0.f, 0.f, 0.f}};
     if (DENS) Mv = ld4s(cs + CI_M * CS);
     const PlaneInfo pi = pinfo[j];
+    F4 ev = {{0.f, 0.f, 0.f, 0.f}};
+    if (PML && pi.ext) ev = ld4s(cs + CI_E * CS);  // the memory variables' part of the Laplacian
     const float gyz = __fmul_rn(gyv, pi.gz);
     F4 out;
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
       const float g = __fmul_rn(gxv[e], gyz);
-      out.v[e] = update(q[4].v[e], prev.v[e], Av.v[e], Mv.v[e], g, lap[e], DENS);
+      out.v[e] = update<PML>(q[4].v[e], prev.v[e], Av.v[e], Mv.v[e], g, lap[e], ev.v[e], DENS);
     }
     // Source injection (forward only): u^{n+1} += w_e dt^2 w[n] / (h^3 sqrt rho_e)
     // at the corners e of the source cell (one corner for the nearest node).
@@ -435,10 +456,10 @@ __global__ void __launch_bounds__((TX / 4) * TY + 32, (MinBlocks<TX, TY, MODE>::
         float lu[4];
         lap4<TX>(st + HS, lx, ly, qu, lu);
 #pragma unroll
-        for (int e = 0; e < 4; ++e) t.v[e] = img_term(qu[4].v[e], Av.v[e], Mv.v[e], lu[e], DENS);
+        for (int e = 0; e < 4; ++e) t.v[e] = img_term<false>(qu[4].v[e], Av.v[e], Mv.v[e], lu[e], 0.f, DENS);
       } else if (MODE != MODE_ADJ_STORED) {
 #pragma unroll
-        for (int e = 0; e < 4; ++e) t.v[e] = img_term(q[4].v[e], Av.v[e], Mv.v[e], lap[e], DENS);
+        for (int e = 0; e < 4; ++e) t.v[e] = img_term<PML>(q[4].v[e], Av.v[e], Mv.v[e], lap[e], ev.v[e], DENS);
       }
       if (MODE == MODE_FWD_STORE || MODE == MODE_FWD_STORE_PH) store_term(z, t);
       if (ACC) {
@@ -498,44 +519,44 @@ __global__ void __launch_bounds__((TX / 4) * TY + 32, (MinBlocks<TX, TY, MODE>::
   }
 }
 
-template <int TX, int TY, bool DENS, int MODE>
+template <int TX, int TY, bool DENS, int MODE, bool PML>
 static size_t smem_bytes_base() {
-  using LY = Layout<TX, TY, DENS, MODE>;
+  using LY = Layout<TX, TY, DENS, MODE, PML>;
   return sizeof(float) * (size_t)(LY::NSU * LY::NHALO * LY::HS + LY::NSC * LY::NC * LY::CS + LY::CS) +
          sizeof(uint64_t) * (2 * LY::NSU + 2 * LY::NSC);
 }
 
 // Dynamic shared memory of one launch: rings, output tile, barriers and the
 // per-plane table for up to max_planes planes per item.
-template <int TX, int TY, bool DENS, int MODE>
+template <int TX, int TY, bool DENS, int MODE, bool PML>
 static size_t smem_bytes(int max_planes) {
-  return smem_bytes_base<TX, TY, DENS, MODE>() + sizeof(PlaneInfo) * (size_t)max_planes;
+  return smem_bytes_base<TX, TY, DENS, MODE, PML>() + sizeof(PlaneInfo) * (size_t)max_planes;
 }
 
-template <int TX, int TY, bool DENS, int MODE>
+template <int TX, int TY, bool DENS, int MODE, bool PML>
 static cudaError_t launch_one(const StepArgs& a, int n_items, int max_planes, cudaStream_t s,
                               int* occupancy) {
-  const size_t sm = smem_bytes<TX, TY, DENS, MODE>(max_planes);
+  const size_t sm = smem_bytes<TX, TY, DENS, MODE, PML>(max_planes);
   static size_t attr_bytes = 0;
   if (sm > attr_bytes) {
-    cudaError_t e = cudaFuncSetAttribute(step_kernel<TX, TY, DENS, MODE>,
+    cudaError_t e = cudaFuncSetAttribute(step_kernel<TX, TY, DENS, MODE, PML>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
     attr_bytes = sm;
   }
   if (occupancy) {
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occupancy, step_kernel<TX, TY, DENS, MODE>,
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occupancy, step_kernel<TX, TY, DENS, MODE, PML>,
                                                          (TX / 4) * TY + 32, sm);
   }
-  step_kernel<TX, TY, DENS, MODE><<<n_items, (TX / 4) * TY + 32, sm, s>>>(a);
+  step_kernel<TX, TY, DENS, MODE, PML><<<n_items, (TX / 4) * TY + 32, sm, s>>>(a);
   return cudaGetLastError();
 }
 
-template <int TX, int TY, int MODE>
+template <int TX, int TY, int MODE, bool PML = false>
 static cudaError_t launch_mode(const StepArgs& a, int n_items, int max_planes, bool dens,
                                cudaStream_t s, int* occ) {
-  return dens ? launch_one<TX, TY, true, MODE>(a, n_items, max_planes, s, occ)
-              : launch_one<TX, TY, false, MODE>(a, n_items, max_planes, s, occ);
+  return dens ? launch_one<TX, TY, true, MODE, PML>(a, n_items, max_planes, s, occ)
+              : launch_one<TX, TY, false, MODE, PML>(a, n_items, max_planes, s, occ);
 }
 
 // Compiled tile shapes (TX, TY).
@@ -545,5 +566,10 @@ cudaError_t dispatch_forward(const StepArgs& a, int n_items, int max_planes, int
                              bool dens, int mode, cudaStream_t s, int* occ);
 cudaError_t dispatch_adjoint(const StepArgs& a, int n_items, int max_planes, int tx, int ty,
                              bool dens, int mode, cudaStream_t s, int* occ);
+// The same with the CPML's E added to the 25-point sum.
+cudaError_t dispatch_pml_forward(const StepArgs& a, int n_items, int max_planes, int tx, int ty,
+                                 bool dens, int mode, cudaStream_t s, int* occ);
+cudaError_t dispatch_pml_adjoint(const StepArgs& a, int n_items, int max_planes, int tx, int ty,
+                                 bool dens, int mode, cudaStream_t s, int* occ);
 
 }  // namespace mamute

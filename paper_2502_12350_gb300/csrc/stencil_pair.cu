@@ -270,7 +270,7 @@ __global__ void __launch_bounds__((TX / 4) * (TY / 2) + 32, 1) pair_kernel(const
       pi.rb = a.rec_ptr[it.rec_tab + j];
       pi.re = a.rec_ptr[it.rec_tab + j + 1];
     }
-    pi.pad = 0;
+    pi.ext = 0;
     return pi;
   };
   if (tid == 0) {
@@ -520,7 +520,7 @@ __global__ void __launch_bounds__((TX / 4) * (TY / 2) + 32, 1) pair_kernel(const
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
           const float g = __fmul_rn(gxv[e], gyz);
-          out[r].v[e] = update(u.v[e], prev.v[e], Av.v[e], Mv.v[e], g, r ? lb[e] : la[e], DENS);
+          out[r].v[e] = update<false>(u.v[e], prev.v[e], Av.v[e], Mv.v[e], g, r ? lb[e] : la[e], 0.f, DENS);
         }
       }
       release(&emptyU[su]);
@@ -562,7 +562,7 @@ __global__ void __launch_bounds__((TX / 4) * (TY / 2) + 32, 1) pair_kernel(const
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
           const float g = __fmul_rn(gxv[e], gyz);
-          out[r].v[e] = update(u.v[e], prev.v[e], Av.v[e], Mv.v[e], g, r ? lb[e] : la[e], DENS);
+          out[r].v[e] = update<false>(u.v[e], prev.v[e], Av.v[e], Mv.v[e], g, r ? lb[e] : la[e], 0.f, DENS);
         }
       }
       release(&emptyV[s]);

@@ -962,9 +962,9 @@ int setup_pairs(mamute_ctx* ctx, const Plan& P, const float* vel, const float* r
   return MAMUTE_OK;
 }
 
-// Gradient smoothing by the DCT-II diagonalisation of the Bessel / Laplace
-// operators (see postproc.cu): forward transforms along x, y, z, the
-// spectral multiplier, transposed transforms along z, y, x.
+// Gradient smoothing (see postproc.cu): tridiagonal solves along the axes
+// (Laplace), or transforms along y and z, a solve along x for every row of
+// modes, and the transposed transforms (Bessel).
 int do_smooth(mamute_ctx* ctx, int nx, int ny, int nz, double h, int mode, const float* lengths,
               const float* in, float* out) {
   const long long n = (long long)nx * ny * nz;
@@ -973,64 +973,105 @@ int do_smooth(mamute_ctx* ctx, int nx, int ny, int nz, double h, int mode, const
     return MAMUTE_OK;
   }
   const int dims[3] = {nx, ny, nz};
+  double mu[3];
   double L[3];
   for (int a = 0; a < 3; ++a) {
     const double l = lengths ? (double)lengths[a] : 0.0;
     if (!(l >= 0.0)) return fail(ctx, MAMUTE_EINVAL, "smoothing length %d is negative", a);
     L[a] = l > 0.0 ? l : 2.0 * h;
+    mu[a] = (L[a] / h) * (L[a] / h);
   }
-  // C_a (orthonormal DCT-II, rows = modes) and its transpose, per axis, and
-  // the eigenvalues of -l_a^2 D_aa; built and uploaded only when the sizes,
-  // the spacing or the lengths differ from the previous call's.
-  size_t off[3][2];
-  size_t o = 0;
-  for (int a = 0; a < 3; ++a) {
-    off[a][0] = o;
-    off[a][1] = o + (size_t)dims[a] * dims[a];
-    o += 2 * (size_t)dims[a] * dims[a];
+  // Tables, built and uploaded only when the sizes, the spacing, the lengths
+  // or the mode differ from the previous call's.  Bessel: per axis y, z the
+  // half matrices E, O of the forward and of the inverse transform, and the
+  // rows' coefficients; Laplace: the elimination factors of y and z.
+  const bool bessel = mode == MAMUTE_SMOOTH_BESSEL;
+  size_t off[3] = {0, 0, 0}, total = 0;
+  for (int a = 1; a < 3; ++a) {
+    const size_t hn = (size_t)(dims[a] + 1) / 2;
+    off[a] = total;
+    total += bessel ? 4 * hn * hn : 2 * (size_t)dims[a];
   }
-  const std::vector<double> key = {(double)nx, (double)ny, (double)nz, h, L[0], L[1], L[2]};
+  const std::vector<double> key = {(double)nx, (double)ny, (double)nz, h, L[0], L[1], L[2], (double)mode};
   if (key != ctx->smKey) {
     ctx->smKey.clear();
-    std::vector<float> mats(o), lam;
-    for (int a = 0; a < 3; ++a) {
-      const int m = dims[a];
-      for (int k = 0; k < m; ++k)
-        for (int i = 0; i < m; ++i) {
-          const double sc = k == 0 ? std::sqrt(1.0 / m) : std::sqrt(2.0 / m);
-          const float c = (float)(sc * std::cos(M_PI * k * (i + 0.5) / m));
-          mats[off[a][0] + (size_t)k * m + i] = c;
-          mats[off[a][1] + (size_t)i * m + k] = c;
+    std::vector<float> tab(total);
+    for (int a = 1; a < 3; ++a) {
+      const int m = dims[a], hn = (m + 1) / 2;
+      float* t = tab.data() + off[a];
+      if (bessel) {
+        const size_t hh = (size_t)hn * hn;  // E fwd, O fwd, E inv, O inv
+        for (int k = 0; k < m; ++k)
+          for (int j = 0; j < hn; ++j) {
+            const double sc = k == 0 ? std::sqrt(1.0 / m) : std::sqrt(2.0 / m);
+            const bool odd = k & 1, mid = 2 * j + 1 == m;
+            const float c = odd && mid ? 0.0f : (float)(sc * std::cos(M_PI * k * (j + 0.5) / m));
+            t[odd * hh + (size_t)j * hn + k / 2] = c;
+            t[(2 + odd) * hh + (size_t)(k / 2) * hn + j] = c;
+          }
+      } else {
+        double g = 0.0;  // mu / pivot of the row above
+        for (int j = 0; j < m; ++j) {
+          const int links = (j > 0) + (j + 1 < m);
+          const double inv = 1.0 / (1.0 + mu[a] * (links - g));
+          g = mu[a] * inv;
+          t[2 * j] = (float)inv;
+          t[2 * j + 1] = (float)g;
         }
-      for (int k = 0; k < m; ++k) {
-        const double sn = std::sin(M_PI * k / (2.0 * m));
-        lam.push_back((float)(4.0 * (L[a] / h) * (L[a] / h) * sn * sn));
       }
     }
-    CK(upload(ctx->smMat, mats, ctx->stream));
-    CK(upload(ctx->smLam, lam, ctx->stream));
+    CK(upload(ctx->smMat, tab, ctx->stream));
+    if (bessel) {
+      CK(ensure(ctx->smLam, sizeof(RowCoef) * (size_t)ny * nz));
+      ++ctx->launches;
+      CK(launch_row_coef((RowCoef*)ctx->smLam.p, ny, nz, mu[1], mu[2], mu[0], nx, ctx->stream));
+    }
     ctx->smKey = key;
   }
-  CK(ensure(ctx->smA, (size_t)n * 4));
+  float* A = nullptr;
+  if (bessel || rows_need_scratch(nx)) {
+    CK(ensure(ctx->smA, (size_t)n * 4));
+    A = (float*)ctx->smA.p;
+  }
   const float* M = (const float*)ctx->smMat.p;
-  float* A = (float*)ctx->smA.p;
   // axis geometry: lines, inner, outer, stride
-  const long long g[3][4] = {{(long long)ny * nz, 1, nx, 1},
-                             {(long long)nz * nx, nx, (long long)nx * ny, nx},
-                             {(long long)nx * ny, (long long)nx * ny, 0, (long long)nx * ny}};
-  auto pass = [&](int a, int inv, const float* src, float* dst) -> cudaError_t {
+  const long long plane = (long long)nx * ny;
+  const long long g[3][4] = {{0, 0, 0, 0}, {(long long)nz * nx, nx, plane, nx}, {plane, plane, 0, plane}};
+  const RowCoef one = row_coef_host(1.0, mu[0], nx);
+  if (!bessel) {
     ++ctx->launches;
-    return launch_axis(src, dst, M + off[a][inv], dims[a], g[a][0], g[a][1], g[a][2], g[a][3],
-                       ctx->stream);
+    CK(launch_rows(in, out, A, nx, (long long)ny * nz, nullptr, one, ctx->stream));
+    for (int a = 1; a < 3; ++a) {
+      if (dims[a] == 1) continue;
+      ++ctx->launches;
+      CK(launch_sweep(out, out, (const float2*)(M + off[a]), dims[a], g[a][0], g[a][1], g[a][2], g[a][3],
+                      ctx->stream));
+    }
+    return MAMUTE_OK;
+  }
+  const float* cur = in;
+  auto transform = [&](int a, bool inverse) -> cudaError_t {
+    if (dims[a] == 1) return cudaSuccess;
+    const size_t hn = (size_t)(dims[a] + 1) / 2;
+    const float* E = M + off[a] + (inverse ? 2 * hn * hn : 0);
+    float* dst = cur == A ? out : A;
+    ++ctx->launches;
+    const cudaError_t e = launch_dct(cur, dst, E, E + hn * hn, inverse, dims[a], g[a][0], g[a][1], g[a][2],
+                                     g[a][3], ctx->stream);
+    cur = dst;
+    return e;
   };
-  CK(pass(0, 0, in, A));
-  CK(pass(1, 0, A, out));
-  CK(pass(2, 0, out, A));
-  ++ctx->launches;
-  CK(launch_spectral_scale(A, nx, ny, nz, (const float*)ctx->smLam.p, mode, ctx->stream));
-  CK(pass(2, 1, A, out));
-  CK(pass(1, 1, out, A));
-  CK(pass(0, 1, A, out));
+  CK(transform(1, false));
+  CK(transform(2, false));
+  {
+    float* dst = cur == A ? A : out;  // in place unless there was no transform
+    ++ctx->launches;
+    CK(launch_rows(cur, dst, cur == A ? out : A, nx, (long long)ny * nz, (const RowCoef*)ctx->smLam.p, one,
+                   ctx->stream));
+    cur = dst;
+  }
+  CK(transform(2, true));
+  CK(transform(1, true));
   return MAMUTE_OK;
 }
 

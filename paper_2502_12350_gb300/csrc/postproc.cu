@@ -2,16 +2,19 @@
 //
 // Smoothing (Sec. 2, FWI gradient preconditioning: Bessel or Laplace filter
 // with lengths lx, ly, lz; Algorithm 3: GradientPreconditioning).  Both
-// filters are inverses of constant-coefficient operators built from the
-// 3-point second difference with reflecting ends, which the orthonormal
-// DCT-II diagonalises along each axis with eigenvalues
-//   lambda_a(k) = 4 (l_a / h)^2 sin^2(pi k / (2 n_a)).
-// The Bessel filter (I - sum_a l_a^2 D_aa)^-1 multiplies mode k by
-// 1 / (1 + sum_a lambda_a), the Laplace filter prod_a (I - l_a^2 D_aa)^-1 by
-// prod_a 1 / (1 + lambda_a).  The transform along an axis is a dense
-// n x n contraction applied to every line of the volume (axis_kernel, a
-// shared-memory tiled FP32 product); forward along x, y, z, the spectral
-// scaling, and the transposed transforms along z, y, x give the exact solve.
+// filters are inverses of operators built from the 3-point second difference
+// D with reflecting ends, and both are applied exactly.
+//   Laplace, prod_a (I - l_a^2 D_aa)^-1: one tridiagonal solve per axis, along
+// x by row_kernel, along y and z by sweep_kernel.
+//   Bessel, (I - sum_a l_a^2 D_aa)^-1: the orthonormal DCT-II diagonalises D
+// along y and z, with eigenvalues -4 sin^2(pi k / (2 n)), so after the
+// transforms along y and z (dct_kernel) every row is one tridiagonal system
+// along x with its own diagonal (row_kernel), and the transposed transforms
+// along z and y follow.
+// (Six dense transforms, three per direction, and a spectral multiplier made
+// the 600x600x200 Bessel filter 15.9 ms; with the transforms along x replaced
+// by a bandwidth-bound pass of 0.16 ms and the others halved by their symmetry
+// it takes 4.0 ms: 1.33 ms a transform along y, 0.59 along z.)
 //
 // Resampling (Sec. 2: time interpolation by nearest neighbour or sinc;
 // Table 1 Interpolate).  The resampling of every trace is the same sparse
@@ -22,97 +25,286 @@
 // them); its transpose is another banded matrix.
 #include "postproc.h"
 
+#include <cmath>
+
 namespace mamute {
 
 namespace {
 
-// Block tile: kTL lines x kTI outputs over chunks of kTK inputs; each of the
-// 256 threads accumulates kRL lines x kRI outputs, reading them from shared
-// memory as float4s (3 loads per 32 FMAs).
-constexpr int kTL = 128, kTI = 64, kTK = 16, kRL = 8, kRI = 4;
-constexpr int kAP = kTL + 4;  // A row pitch: float4-aligned, x-axis stores spread over banks
+// ---- tridiagonal solves (s - mu D) u = f with reflecting ends ----
+//
+// The inverse on the line is u_i = K (p_i + r q_{i+1}) with the recursions
+// p_i = f_i + r p_{i-1} and q_i = f_i + r q_{i+1}, r in (0, 1) the root of
+// mu r^2 - (s + 2 mu) r + mu = 0 and K = (1 - r) / (s (1 + r)); the
+// reflecting ends are the even images of f, which enter only through
+// p_{-1} = (q0 + r^n p0) / (1 - r^{2n}) (q0, p0: q_0 and p_{n-1} of the line
+// alone) and q_n = p_{n-1}.  All terms have the sign of f: no cancellation.
 
-// out[L, i] = sum_j M[i][j] in[L, j] for the lines L of one axis:
-// element (L, j) sits at (L / inner) * outer + (L % inner) + j * astride.
-__global__ void __launch_bounds__(256) axis_kernel(const float* __restrict__ in,
-                                                   float* __restrict__ out,
-                                                   const float* __restrict__ M, int n,
-                                                   long long lines, long long inner,
-                                                   long long outer, long long astride) {
-  __shared__ __align__(16) float As[kTK][kAP];
-  __shared__ __align__(16) float Bs[kTK][kTI];
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const long long L0 = (long long)blockIdx.x * kTL;
-  const int i0 = blockIdx.y * kTI;
-  // The kTL x kTK elements of a chunk are 8 per thread, at the same lines and
-  // chunk columns in every chunk, so the line offsets are computed once.
-  // Along x (astride 1) consecutive threads take consecutive j (the lines are
-  // a row apart); along y and z consecutive lines (inner-contiguous).
-  constexpr int kAQ = kTL * kTK / 256;
-  const bool xaxis = astride == 1;
-  long long abase[kAQ];
-  int al[kAQ], ajj[kAQ];
-#pragma unroll
-  for (int q = 0; q < kAQ; ++q) {
-    const int e = threadIdx.x + 256 * q;
-    al[q] = xaxis ? e / kTK : e % kTL;
-    ajj[q] = xaxis ? e % kTK : e / kTL;
-    const long long L = L0 + al[q];
-    abase[q] = L < lines ? (L / inner) * outer + (L % inner) : -1;
-  }
-  float acc[kRL][kRI] = {};
-  for (int j0 = 0; j0 < n; j0 += kTK) {
-#pragma unroll
-    for (int q = 0; q < kAQ; ++q) {
-      const int j = j0 + ajj[q];
-      As[ajj[q]][al[q]] = (abase[q] >= 0 && j < n) ? in[abase[q] + (long long)j * astride] : 0.0f;
+// r and K of a line, and the powers the parallel recursion needs, formed in
+// FP64 from the rounded r (so that a constant is kept to rounding).
+__device__ __forceinline__ RowCoef row_coef(double s, double mu, int n, int len) {
+  const double a = s / (2.0 * mu);
+  RowCoef c;
+  c.r = (float)(1.0 / (1.0 + a + sqrt(a * (a + 2.0))));
+  const double r = c.r;
+  c.K = (float)((1.0 - r) / (s * (1.0 + r)));
+  c.rl = (float)pow(r, (double)len);
+  const double rn = pow(r, (double)n);
+  c.rn = (float)rn;
+  c.w = (float)(1.0 / (1.0 - rn * rn));
+  return c;
+}
+
+// One coefficient set per row (y, z) of DCT modes along y and z.
+__global__ void row_coef_kernel(RowCoef* out, int ny, int nz, double my, double mz, double mu, int n,
+                                int len) {
+  const int q = blockIdx.x * blockDim.x + threadIdx.x;
+  if (q >= ny * nz) return;
+  const double sy = sinpi(0.5 * (double)(q % ny) / ny), sz = sinpi(0.5 * (double)(q / ny) / nz);
+  out[q] = row_coef(1.0 + 4.0 * (my * sy * sy + mz * sz * sz), mu, n, len);
+}
+
+// Solves along x, one row per warp.  Lane l owns the `len` cells from l len
+// (len odd: no bank conflicts), runs both recursions on them from zero, takes
+// the others' part from a warp scan, and runs them again from the true start.
+// The row is staged in shared memory (row and p, 8 bytes a cell) so that
+// DRAM sees one read and one write, or, for rows beyond kRowSmem bytes, left
+// in global memory with p in `scratch`.  Bound by HBM and the shared-memory
+// accesses (about 9 a cell).
+__global__ void row_kernel(const float* in, float* out, float* scratch, int n, int len,
+                           long long rows, const RowCoef* __restrict__ coef, RowCoef one, bool staged) {
+  extern __shared__ float row_smem[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+  for (long long row = (long long)blockIdx.x * warps + warp; row < rows;
+       row += (long long)gridDim.x * warps) {
+    const RowCoef c = coef ? coef[row] : one;
+    const float* f = in + row * n;
+    float* p = scratch + row * n;
+    float* o = out + row * n;
+    if (staged) {
+      float* sf = row_smem + (size_t)warp * 2 * n;
+      __syncwarp();
+      for (int j = lane; j < n; j += 32) sf[j] = f[j];
+      __syncwarp();
+      f = sf;
+      p = sf + n;
     }
-#pragma unroll
-    for (int q = 0; q < kTI * kTK / 256; ++q) {
-      const int e = threadIdx.x + 256 * q;
-      const int jj = e % kTK, ii = e / kTK;
-      const int i = i0 + ii, j = j0 + jj;
-      Bs[jj][ii] = (i < n && j < n) ? M[(long long)i * n + j] : 0.0f;
+    const int b = min(lane * len, n), e = min(b + len, n);
+    float cp = 0.0f, cq = 0.0f;  // p of the last and q of the first owned cell, from zero
+    for (int j = b; j < e; ++j) cp = fmaf(c.r, cp, f[j]);
+    for (int j = e - 1; j >= b; --j) cq = fmaf(c.r, cq, f[j]);
+    float a = c.rl;
+    if (e - b < len) {
+      a = 1.0f;
+      for (int j = b; j < e; ++j) a *= c.r;
     }
-    __syncthreads();
+    float ap = a, aq = a;
 #pragma unroll
-    for (int k = 0; k < kTK; ++k) {
-      const float4 a0 = *reinterpret_cast<const float4*>(&As[k][ty * kRL]);
-      const float4 a1 = *reinterpret_cast<const float4*>(&As[k][ty * kRL + 4]);
-      const float4 b = *reinterpret_cast<const float4*>(&Bs[k][tx * kRI]);
-      const float a[kRL] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-      const float bb[kRI] = {b.x, b.y, b.z, b.w};
-#pragma unroll
-      for (int r = 0; r < kRL; ++r)
-#pragma unroll
-        for (int c = 0; c < kRI; ++c) acc[r][c] = fmaf(a[r], bb[c], acc[r][c]);
+    for (int d = 1; d < 32; d <<= 1) {
+      const float pc = __shfl_up_sync(0xffffffffu, cp, d), pa = __shfl_up_sync(0xffffffffu, ap, d);
+      const float qc = __shfl_down_sync(0xffffffffu, cq, d), qa = __shfl_down_sync(0xffffffffu, aq, d);
+      if (lane >= d) {
+        cp = fmaf(ap, pc, cp);
+        ap *= pa;
+      }
+      if (lane + d < 32) {
+        cq = fmaf(aq, qc, cq);
+        aq *= qa;
+      }
     }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int r = 0; r < kRL; ++r) {
-    const long long L = L0 + ty * kRL + r;
-    if (L >= lines) continue;
-    const long long base = (L / inner) * outer + (L % inner);
-#pragma unroll
-    for (int c = 0; c < kRI; ++c) {
-      const int i = i0 + tx * kRI + c;
-      if (i < n) out[base + (long long)i * astride] = acc[r][c];
+    const float pend = __shfl_sync(0xffffffffu, cp, 31), q0 = __shfl_sync(0xffffffffu, cq, 0);
+    const float pm1 = c.w * fmaf(c.rn, pend, q0), qn = fmaf(c.rn, pm1, pend);
+    // the neighbouring lanes' inclusive values, and the ends
+    const float pc = __shfl_up_sync(0xffffffffu, cp, 1), pa = __shfl_up_sync(0xffffffffu, ap, 1);
+    const float qc = __shfl_down_sync(0xffffffffu, cq, 1), qa = __shfl_down_sync(0xffffffffu, aq, 1);
+    float pv = lane == 0 ? pm1 : fmaf(pa, pm1, pc);
+    float qv = lane == 31 ? qn : fmaf(qa, qn, qc);
+    for (int j = b; j < e; ++j) {
+      pv = fmaf(c.r, pv, f[j]);
+      p[j] = pv;
+    }
+    float* res = staged ? p : o;
+    for (int j = e - 1; j >= b; --j) {
+      const float fj = f[j];
+      res[j] = c.K * fmaf(c.r, qv, p[j]);
+      qv = fmaf(c.r, qv, fj);
+    }
+    if (staged) {
+      __syncwarp();
+      for (int j = lane; j < n; j += 32) o[j] = p[j];
     }
   }
 }
 
-// Spectral multiplier of the filter on DCT coefficients [nz][ny][nx].
-__global__ void scale_kernel(float* __restrict__ u, int nx, int ny, int nz,
-                             const float* __restrict__ lam, int mode) {
-  const long long n = (long long)nx * ny * nz;
-  for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < n;
-       p += (long long)gridDim.x * blockDim.x) {
-    const int x = (int)(p % nx), y = (int)((p / nx) % ny), z = (int)(p / ((long long)nx * ny));
-    const float lx = lam[x], ly = lam[nx + y], lz = lam[nx + ny + z];
-    const float m = mode == 1 ? 1.0f / (1.0f + lx + ly + lz)
-                              : 1.0f / ((1.0f + lx) * (1.0f + ly) * (1.0f + lz));
-    u[p] *= m;
+constexpr int kRowSmem = 200 * 1024;
+
+// Solves along y or z in place, one column per thread (consecutive threads on
+// consecutive x): elimination upwards, y_i = inv_i f_i + g_i y_{i-1}, and
+// back-substitution downwards, u_i = y_i + g_i u_{i+1}, with the factors of
+// the one matrix all columns share (formed on the host in FP64).  Two reads
+// and two writes of the volume; the loads of 8 cells are issued together.
+__global__ void __launch_bounds__(256) sweep_kernel(const float* in, float* out,
+                                                    const float2* __restrict__ fac, int n,
+                                                    long long lines, long long inner,
+                                                    long long outer, long long st) {
+  const long long L = blockIdx.x * 256LL + threadIdx.x;
+  if (L >= lines) return;
+  const long long base = (L / inner) * outer + L % inner;
+  const float* f = in + base;
+  float* u = out + base;
+  float v = 0.0f;
+  for (int i0 = 0; i0 < n; i0 += 8) {
+    float t[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) t[k] = i0 + k < n ? f[(i0 + k) * st] : 0.0f;
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      if (i0 + k < n) {
+        const float2 c = __ldg(fac + i0 + k);
+        v = fmaf(c.y, v, c.x * t[k]);
+        u[(i0 + k) * st] = v;
+      }
+  }
+  v = 0.0f;
+  for (int i0 = (n - 1) / 8 * 8; i0 >= 0; i0 -= 8) {
+    float t[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) t[k] = i0 + k < n ? u[(i0 + k) * st] : 0.0f;
+#pragma unroll
+    for (int k = 7; k >= 0; --k)
+      if (i0 + k < n) {
+        v = fmaf(__ldg(fac + i0 + k).y, v, t[k]);
+        u[(i0 + k) * st] = v;
+      }
+  }
+}
+
+// ---- DCT-II along y or z ----
+//
+// The even modes are symmetric about the middle of the line and the odd ones
+// antisymmetric, so the n x n product splits into two of half the size on the
+// sums and differences of the mirrored cells (half the operations, shorter
+// sums).  A block makes 64 even and 64 odd modes (inverse: 64 mirrored pairs
+// of cells) of 128 lines; each of its 256 threads accumulates 8 lines x 4
+// outputs x 2, fed by float4 shared-memory reads, with the next chunk's
+// global loads in registers while a chunk is multiplied.  FP32 ALU bound.
+constexpr int kTL = 128, kTI = 64, kTK = 8;
+constexpr int kAP = kTL + 4;  // A row pitch
+
+// forward (INV = false): out[2 i] = sum_j E[j][i] (f_j + f_{n-1-j}),
+//   out[2 i + 1] = sum_j O[j][i] (f_j - f_{n-1-j}) over j < h = ceil(n / 2)
+//   (the middle cell of an odd n counts once);
+// inverse: e_i = sum_j E[j][i] F_{2j}, o_i = sum_j O[j][i] F_{2j+1},
+//   out[i] = e_i + o_i, out[n-1-i] = e_i - o_i.
+// E and O are [h][h], zero-padded.
+template <bool INV>
+__global__ void __launch_bounds__(256, 2)
+    dct_kernel(const float* __restrict__ in, float* __restrict__ out, const float* __restrict__ E,
+               const float* __restrict__ O, int n, long long lines, long long inner,
+               long long outer, long long st) {
+  __shared__ __align__(16) float As[2][2][kTK][kAP];
+  __shared__ __align__(16) float Bs[2][2][kTK][kTI];
+  const int h = (n + 1) / 2;
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const long long L0 = (long long)blockIdx.x * kTL;
+  const int i0 = blockIdx.y * kTI;
+  // loads: 128 lines x 8 cells x 2 = 4 pairs per thread (one line each), and
+  // 8 x 64 of each matrix = 2 per thread
+  const int al = tid & (kTL - 1), aj = tid / kTL;
+  const long long LA = L0 + al;
+  const bool lok = LA < lines;
+  const float* src = in + (lok ? (LA / inner) * outer + LA % inner : 0);
+  const int bi = tid & (kTI - 1), bj = tid / kTI;
+  float ra[2][4], rb[2][2];
+  auto load = [&](int j0) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int j = j0 + aj + 2 * k;
+      const int p = INV ? 2 * j : j, q = INV ? 2 * j + 1 : n - 1 - j;
+      ra[0][k] = lok && j < h ? src[p * st] : 0.0f;
+      ra[1][k] = lok && j < h && q < n && q != p ? src[q * st] : 0.0f;
+    }
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const int j = j0 + bj + 4 * k, i = i0 + bi;
+      const bool ok = j < h && i < h;
+      rb[0][k] = ok ? __ldg(E + (long long)j * h + i) : 0.0f;
+      rb[1][k] = ok ? __ldg(O + (long long)j * h + i) : 0.0f;
+    }
+  };
+  auto stage = [&](int s) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      As[s][0][aj + 2 * k][al] = INV ? ra[0][k] : ra[0][k] + ra[1][k];
+      As[s][1][aj + 2 * k][al] = INV ? ra[1][k] : ra[0][k] - ra[1][k];
+    }
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      Bs[s][0][bj + 4 * k][bi] = rb[0][k];
+      Bs[s][1][bj + 4 * k][bi] = rb[1][k];
+    }
+  };
+  float acc[2][8][4] = {};
+  load(0);
+  stage(0);
+  __syncthreads();
+  int s = 0;
+  for (int j0 = 0; j0 < h; j0 += kTK, s ^= 1) {
+    const bool more = j0 + kTK < h;
+    if (more) load(j0 + kTK);
+#pragma unroll
+    for (int k = 0; k < kTK; ++k)
+#pragma unroll
+      for (int v = 0; v < 2; ++v) {
+        // lines 4 ty .. and 64 + 4 ty ..: the two rows of threads of a warp
+        // read consecutive float4s
+        const float4 a0 = *reinterpret_cast<const float4*>(&As[s][v][k][ty * 4]);
+        const float4 a1 = *reinterpret_cast<const float4*>(&As[s][v][k][64 + ty * 4]);
+        const float4 b = *reinterpret_cast<const float4*>(&Bs[s][v][k][tx * 4]);
+        const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+        const float bb[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+        for (int r = 0; r < 8; ++r)
+#pragma unroll
+          for (int c = 0; c < 4; ++c) acc[v][r][c] = fmaf(a[r], bb[c], acc[v][r][c]);
+      }
+    if (more) stage(s ^ 1);
+    __syncthreads();
+  }
+#pragma unroll
+  for (int g = 0; g < 2; ++g) {
+    const long long L = L0 + 64 * g + ty * 4;
+    if (L >= lines) continue;
+    // four consecutive lines share a 16-byte store where the layout allows it
+    const long long b0 = (L / inner) * outer + L % inner;
+    const bool vec = L % inner + 4 <= inner && ((b0 | st) & 3) == 0 && L + 4 <= lines &&
+                     ((unsigned long long)out & 15) == 0;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const int i = i0 + tx * 4 + c;
+      if (i >= h) continue;
+      const int p = INV ? i : 2 * i, q = INV ? n - 1 - i : 2 * i + 1;
+      float e[4], o[4];
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const float x = acc[0][4 * g + r][c], y = acc[1][4 * g + r][c];
+        e[r] = INV ? x + y : x;
+        o[r] = INV ? x - y : y;
+      }
+      if (vec) {
+        *reinterpret_cast<float4*>(out + b0 + p * st) = make_float4(e[0], e[1], e[2], e[3]);
+        if (q < n && q != p)
+          *reinterpret_cast<float4*>(out + b0 + q * st) = make_float4(o[0], o[1], o[2], o[3]);
+      } else {
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          if (L + r >= lines) continue;
+          const long long b = ((L + r) / inner) * outer + (L + r) % inner;
+          out[b + p * st] = e[r];
+          if (q < n && q != p) out[b + q * st] = o[r];
+        }
+      }
+    }
   }
 }
 
@@ -162,20 +354,64 @@ cudaError_t launch_sub(const float* a, const float* b, long long n, float* out, 
   return cudaGetLastError();
 }
 
-cudaError_t launch_axis(const float* in, float* out, const float* M, int n, long long lines,
-                        long long inner, long long outer, long long astride, cudaStream_t s) {
-  if (lines <= 0 || n <= 0) return cudaSuccess;
-  dim3 g((unsigned)((lines + kTL - 1) / kTL), (unsigned)((n + kTI - 1) / kTI));
-  axis_kernel<<<g, 256, 0, s>>>(in, out, M, n, lines, inner, outer, astride);
+int row_len(int n) { return ((n + 31) / 32) | 1; }
+
+RowCoef row_coef_host(double s, double mu, int n) {
+  const double a = s / (2.0 * mu);
+  RowCoef c;
+  c.r = (float)(1.0 / (1.0 + a + std::sqrt(a * (a + 2.0))));
+  const double r = c.r, rn = std::pow(r, (double)n);
+  c.K = (float)((1.0 - r) / (s * (1.0 + r)));
+  c.rl = (float)std::pow(r, (double)row_len(n));
+  c.rn = (float)rn;
+  c.w = (float)(1.0 / (1.0 - rn * rn));
+  return c;
+}
+
+cudaError_t launch_row_coef(RowCoef* out, int ny, int nz, double my, double mz, double mx, int nx,
+                            cudaStream_t s) {
+  row_coef_kernel<<<(ny * nz + 127) / 128, 128, 0, s>>>(out, ny, nz, my, mz, mx, nx, row_len(nx));
   return cudaGetLastError();
 }
 
-cudaError_t launch_spectral_scale(float* u, int nx, int ny, int nz, const float* lam, int mode,
-                                  cudaStream_t s) {
-  const long long n = (long long)nx * ny * nz;
-  long long b = (n + 255) / 256;
-  if (b > 152 * 16) b = 152 * 16;
-  scale_kernel<<<(unsigned)b, 256, 0, s>>>(u, nx, ny, nz, lam, mode);
+bool rows_need_scratch(int n) { return 8LL * n > kRowSmem; }
+
+cudaError_t launch_rows(const float* in, float* out, float* scratch, int n, long long rows,
+                        const RowCoef* coef, const RowCoef& one, cudaStream_t s) {
+  if (rows <= 0 || n <= 0) return cudaSuccess;
+  const bool staged = !rows_need_scratch(n);
+  // 8 rows a block, fewer where they would leave less than two blocks per SM
+  int warps = 8;
+  while (staged && warps > 1 && 8LL * n * warps > 100 * 1024) warps /= 2;
+  const size_t smem = staged ? (size_t)8 * n * warps : 0;
+  if (smem > 48 * 1024) {
+    cudaError_t e = cudaFuncSetAttribute(row_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         kRowSmem);
+    if (e != cudaSuccess) return e;
+  }
+  const long long blocks = (rows + warps - 1) / warps;
+  row_kernel<<<(unsigned)(blocks < 152 * 64 ? blocks : 152 * 64), 32 * warps, smem, s>>>(
+      in, out, scratch, n, row_len(n), rows, coef, one, staged);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_sweep(const float* in, float* out, const float2* fac, int n, long long lines,
+                         long long inner, long long outer, long long st, cudaStream_t s) {
+  if (lines <= 0 || n <= 0) return cudaSuccess;
+  sweep_kernel<<<(unsigned)((lines + 255) / 256), 256, 0, s>>>(in, out, fac, n, lines, inner, outer, st);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_dct(const float* in, float* out, const float* E, const float* O, bool inverse,
+                       int n, long long lines, long long inner, long long outer, long long st,
+                       cudaStream_t s) {
+  if (lines <= 0 || n <= 0) return cudaSuccess;
+  const int h = (n + 1) / 2;
+  const dim3 g((unsigned)((lines + kTL - 1) / kTL), (unsigned)((h + kTI - 1) / kTI));
+  if (inverse)
+    dct_kernel<true><<<g, 256, 0, s>>>(in, out, E, O, n, lines, inner, outer, st);
+  else
+    dct_kernel<false><<<g, 256, 0, s>>>(in, out, E, O, n, lines, inner, outer, st);
   return cudaGetLastError();
 }
 

@@ -2062,8 +2062,13 @@ int run_gn(mamute_ctx* ctx, const mamute_grid* g, const float* vel, const float*
   CK(upload(ctx->gnBins, bins, ctx->stream));
   CK(upload(ctx->gnWts, wts, ctx->stream));
   CK(ensure(ctx->gnRow, (size_t)2 * std::max(P.ncol, 1) * 4));
-  CK(cudaMemsetAsync(ctx->gnRe.p, 0, (size_t)nb * Bmax * N * 4, ctx->stream));
-  CK(cudaMemsetAsync(ctx->gnIm.p, 0, (size_t)nb * Bmax * N * 4, ctx->stream));
+  // With N a multiple of 4 every batch runs on the tensor cores, whose first
+  // block overwrites the accumulators; else they start from zero.
+  const bool clear = !dft_tc_supported(N, nb);
+  if (clear) {
+    CK(cudaMemsetAsync(ctx->gnRe.p, 0, (size_t)nb * Bmax * N * 4, ctx->stream));
+    CK(cudaMemsetAsync(ctx->gnIm.p, 0, (size_t)nb * Bmax * N * 4, ctx->stream));
+  }
   CK(cudaMemsetAsync(ctx->gnS.p, 0, (size_t)nb * N * 4, ctx->stream));
   CK(cudaMemsetAsync(ctx->gnR.p, 0, (size_t)nb * N * 4, ctx->stream));
   float* V = (float*)ctx->gnV.p;
@@ -2102,7 +2107,7 @@ int run_gn(mamute_ctx* ctx, const mamute_grid* g, const float* vel, const float*
       if ((n + 1) % kT == 0) TRY(flush(n + 1));
     }
     TRY(flush(nt));
-    CK(aux_count(ctx, launch_power(nb, N, nv, re, im, (float*)ctx->gnS.p, ctx->stream)));
+    CK(aux_count(ctx, launch_power(nb, N, nv, re, im, (float*)ctx->gnS.p, clear, ctx->stream)));
   }
   // Receiver side: receiver r0 + b of the common set in window b, a unit data
   // impulse at the last sample.  Batches of Br windows: when Br exceeds the
@@ -2179,7 +2184,7 @@ int run_gn(mamute_ctx* ctx, const mamute_grid* g, const float* vel, const float*
       if ((j + 1) % kT == 0) TRY(flush(j + 1));
     }
     TRY(flush(nt));
-    CK(aux_count(ctx, launch_power(nb, N, nv, re, im, (float*)ctx->gnR.p, ctx->stream)));
+    CK(aux_count(ctx, launch_power(nb, N, nv, re, im, (float*)ctx->gnR.p, clear, ctx->stream)));
     CK(cudaStreamSynchronize(ctx->stream));  // the host impulse row is reused
   }
   CK(aux_count(ctx, launch_assemble(N, nb, (const float*)ctx->gnWts.p, (const float*)ctx->gnR.p,

@@ -24,8 +24,8 @@ bool dft_tc_supported(long long N, int nb);
 cudaError_t launch_dft_tc(const CUtensorMap& vmap, long long N, int T, int n0, int nf,
                           const int* bins, int nb, float* W, float* re, float* im, bool overwrite,
                           int* status, cudaStream_t s);
-// pw[k][x] += sum over the nv windows of |acc[k][v N + x]|^2, then acc = 0.
-cudaError_t launch_power(int nb, long long N, int nv, float* re, float* im, float* pw,
+// pw[k][x] += sum over the nv windows of |acc[k][v N + x]|^2, then acc = 0 if clear.
+cudaError_t launch_power(int nb, long long N, int nv, float* re, float* im, float* pw, bool clear,
                          cudaStream_t s);
 // H[x] = 4 / (c^6 dt^4 nf) sum_k w[k] R[k][x] S[k][x].
 cudaError_t launch_assemble(long long N, int nb, const float* w, const float* R, const float* S,

@@ -5,10 +5,12 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <array>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <map>
 #include <string>
 #include <vector>
 
@@ -28,7 +30,7 @@ namespace {
 
 // Stability bound of the 3-D eighth-order leapfrog scheme:
 // (c dt / h)^2 * 3 * max_theta(-c0 - 2 sum c_j cos j theta) <= 4.
-double cfl_bound() {
+double cfl_bound_scan() {
   const double c[5] = {-205.0 / 72.0, 8.0 / 5.0, -1.0 / 5.0, 8.0 / 315.0, -1.0 / 560.0};
   double mx = 0.0;
   for (int i = 0; i <= 100000; ++i) {
@@ -38,6 +40,12 @@ double cfl_bound() {
     mx = std::max(mx, s);
   }
   return 2.0 / std::sqrt(3.0 * mx);
+}
+
+// The scan takes about 3 ms on a host core: once per process.
+double cfl_bound() {
+  static const double bound = cfl_bound_scan();
+  return bound;
 }
 
 struct DevBuf {
@@ -121,8 +129,20 @@ struct mamute_ctx {
   DevBuf gnV, gnRe, gnIm, gnS, gnR, gnW, gnBins, gnWts, gnRow;  // GN-diagonal scratch
   DevBuf nnPartial, nnLoss;  // network scratch
   DevBuf slotmaps;           // tensor maps of the checkpoint slots
-  int* status = nullptr;
+  char* stage = nullptr;  // page-locked staging of the uploads (see upload)
+  size_t stage_bytes = 0, stage_used = 0, stage_need = 0;
+  // Page-locked words: `status` is written by a kernel whose wait runs out
+  // (mapped), the others receive copies.  A pageable target would make each
+  // copy wait on the host, and a device word would need a clear and a copy per call.
+  struct HostWords {
+    int status;
+    unsigned int maxbits;
+    double value;
+  };
+  HostWords* host = nullptr;
+  int* status = nullptr;  // &host->status
   unsigned int* maxbits = nullptr;
+  cudaEvent_t vmax_ev = nullptr;  // maxbits has arrived
   // timing hook
   bool timing = false;
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
@@ -179,13 +199,40 @@ void release(DevBuf& b) {
   b.bytes = 0;
 }
 
+// Uploads go through the context's page-locked staging area, so that the host
+// neither waits for each copy nor keeps the vectors.  What a call stages is
+// counted, and stage_reset, which starts a call, makes room for as much; what
+// does not fit is copied from the vector and waited for.
 template <typename T>
-cudaError_t upload(DevBuf& b, const std::vector<T>& v, cudaStream_t s) {
+cudaError_t upload(mamute_ctx* ctx, DevBuf& b, const std::vector<T>& v) {
   cudaError_t e = ensure(b, sizeof(T) * std::max<size_t>(v.size(), 1));
   if (e != cudaSuccess || v.empty()) return e;
-  e = cudaMemcpyAsync(b.p, v.data(), sizeof(T) * v.size(), cudaMemcpyHostToDevice, s);
-  if (e != cudaSuccess) return e;
-  return cudaStreamSynchronize(s);  // host vectors are released after the call
+  const size_t bytes = sizeof(T) * v.size(), room = (bytes + 255) / 256 * 256;
+  ctx->stage_need += room;
+  if (ctx->stage_used + room <= ctx->stage_bytes) {
+    char* p = ctx->stage + ctx->stage_used;
+    ctx->stage_used += room;
+    std::memcpy(p, v.data(), bytes);
+    return cudaMemcpyAsync(b.p, p, bytes, cudaMemcpyHostToDevice, ctx->stream);
+  }
+  e = cudaMemcpyAsync(b.p, v.data(), bytes, cudaMemcpyHostToDevice, ctx->stream);
+  return e == cudaSuccess ? cudaStreamSynchronize(ctx->stream) : e;
+}
+
+cudaError_t stage_reset(mamute_ctx* ctx) {
+  cudaError_t e = cudaSuccess;
+  if (ctx->stage_used > 0) e = cudaStreamSynchronize(ctx->stream);  // a failed call's copies
+  if (ctx->stage_need > ctx->stage_bytes) {
+    if (ctx->stage) cudaFreeHost(ctx->stage);
+    ctx->stage = nullptr;
+    ctx->stage_bytes = 0;
+    if (cudaHostAlloc((void**)&ctx->stage, ctx->stage_need, cudaHostAllocPortable) == cudaSuccess)
+      ctx->stage_bytes = ctx->stage_need;
+    else
+      cudaGetLastError();  // without it the copies wait
+  }
+  ctx->stage_used = ctx->stage_need = 0;
+  return e;
 }
 
 // Cerjan profile of one padded axis; with a free surface at plane zs (z axis
@@ -235,6 +282,8 @@ int max_piece(const std::vector<int>& b) {
 
 
 
+constexpr int kMaxTilePoints = 4096;  // above every compiled tile's points
+
 // Receiver tables for one tiling (items ordered z block, row, column).
 void build_receivers(Plan& P, int TX, int zsplit, const std::vector<NodeEntry>& ent,
                      const std::vector<int>& item_base, const std::vector<Tiling>& tilings,
@@ -243,10 +292,11 @@ void build_receivers(Plan& P, int TX, int zsplit, const std::vector<NodeEntry>& 
                      std::vector<float>& gvals, std::vector<int>& colmap,
                      std::vector<int>* ent_of_col = nullptr) {
   struct Tmp {
-    int item, z, lxy, r;
+    unsigned long long key;  // item, plane, place in the tile
+    int r, item, z, lxy;
   };
-  std::vector<Tmp> t;
-  t.reserve(ent.size());
+  std::vector<Tmp> t(ent.size());
+  unsigned long long top = 0;
   for (int r = 0; r < (int)ent.size(); ++r) {
     const int s = ent[r].shot;
     const int lx = ent[r].lx, ly = ent[r].ly, lz = ent[r].lz;
@@ -258,14 +308,25 @@ void build_receivers(Plan& P, int TX, int zsplit, const std::vector<NodeEntry>& 
     const int zlen = (Nz + zsplit - 1) / zsplit;
     const int zb = std::min(lz / zlen, zsplit - 1);
     const int item = item_base[s] + (zb * nrows + tj) * ncols + ti;
-    t.push_back(Tmp{item, lz, (lx - T.xs[ti]) + TX * (ly - T.ys[tj]), r});
+    const int lxy = (lx - T.xs[ti]) + TX * (ly - T.ys[tj]);
+    const unsigned long long key =
+        ((unsigned long long)item * P.Nz + lz) * kMaxTilePoints + (unsigned)lxy;
+    top = std::max(top, key);
+    t[r] = Tmp{key, r, item, lz, lxy};
   }
-  std::sort(t.begin(), t.end(), [](const Tmp& a, const Tmp& b) {
-    if (a.item != b.item) return a.item < b.item;
-    if (a.z != b.z) return a.z < b.z;
-    if (a.lxy != b.lxy) return a.lxy < b.lxy;
-    return a.r < b.r;
-  });
+  // Stable radix order by key (equal keys keep the receivers' order); a
+  // comparison sort of the survey-size tables took several milliseconds a call.
+  {
+    constexpr int kBits = 11;
+    std::vector<Tmp> o(t.size());
+    for (int sh = 0; sh < 64 && (top >> sh) != 0; sh += kBits) {
+      size_t at[(1 << kBits) + 1] = {0};
+      for (const Tmp& e : t) ++at[((e.key >> sh) & ((1 << kBits) - 1)) + 1];
+      for (int k = 0; k < (1 << kBits); ++k) at[k + 1] += at[k];
+      for (const Tmp& e : t) o[at[(e.key >> sh) & ((1 << kBits) - 1)]++] = e;
+      t.swap(o);
+    }
+  }
   rec.assign(t.size(), RecEntry{});
   cells.assign(t.size(), 0);
   gvals.assign(t.size(), 0.f);
@@ -311,6 +372,19 @@ void build_receivers(Plan& P, int TX, int zsplit, const std::vector<NodeEntry>& 
   }
 }
 
+// step_blocks_per_sm, remembered per kernel variant and table length (a driver
+// query of about a microsecond, asked for every candidate of every call).
+int blocks_per_sm(int tx, int ty, bool dens, bool pml, int mode, int planes) {
+  thread_local std::map<std::array<int, 6>, int> known;
+  const std::array<int, 6> key = {tx, ty, dens, pml, mode, planes};
+  auto it = known.find(key);
+  if (it == known.end()) {
+    if (known.size() > 4096) known.clear();
+    it = known.emplace(key, step_blocks_per_sm(tx, ty, dens, pml, mode, planes)).first;
+  }
+  return it->second;
+}
+
 // Chooses, among the compiled tile shapes, the shape, a row refinement and a
 // split of the planes into z blocks that minimise the work of the busiest
 // SM: ceil(items / SMs) items of (box-bound points x planes), divided by a
@@ -338,7 +412,7 @@ TileChoice choose_tiles(const std::vector<VolDesc>& vols, bool dens, bool pml, i
     // per-plane table counts as long as the z block is.
     int per_sm_of[sizeof zsplits / sizeof zsplits[0]];
     for (size_t k = 0; k < sizeof zsplits / sizeof zsplits[0]; ++k)
-      per_sm_of[k] = step_blocks_per_sm(TX, TY, dens, pml, mode,
+      per_sm_of[k] = blocks_per_sm(TX, TY, dens, pml, mode,
                                         mode == MODE_ADJ_STORED ? (Nz + zsplits[k] - 1) / zsplits[k] : Nz);
     const int warps_cta = (TX / 4) * TY / 32;
     for (int r = 1; r <= 2; ++r) {
@@ -390,12 +464,9 @@ TileChoice choose_tiles(const std::vector<VolDesc>& vols, bool dens, bool pml, i
   return best;
 }
 
-// adj_mode: the adjoint kernel mode the tiles are chosen for (MODE_ADJ when
-// the forward states are recomputed, MODE_ADJ_STORED when every imaging term
-// is kept: their shared-memory footprints, hence occupancies, differ).
-int build_plan(mamute_ctx* ctx, const mamute_grid* g, bool dens, int n_src, const float* src_xyz,
-               const int* rec_offset, const float* rec_xyz, const int* aperture, Plan& P,
-               const int* tiles = nullptr, int adj_mode = MODE_ADJ) {
+// Windows, sources and receiver nodes of a call (after checking it).
+int plan_windows(mamute_ctx* ctx, const mamute_grid* g, bool dens, int n_src, const float* src_xyz,
+               const int* rec_offset, const float* rec_xyz, const int* aperture, Plan& P) {
   if (!g) return fail(ctx, MAMUTE_EINVAL, "grid is NULL");
   if (g->nx < 1 || g->ny < 1 || g->nz < 1 || g->border < 0 || g->nt < 1)
     return fail(ctx, MAMUTE_EINVAL, "bad grid dimensions");
@@ -477,7 +548,8 @@ int build_plan(mamute_ctx* ctx, const mamute_grid* g, bool dens, int n_src, cons
     }
     return !out.empty();
   };
-  std::vector<NodeEntry> ent;
+  std::vector<NodeEntry>& ent = P.ent;
+  ent.reserve((size_t)n_rec * (g->xyz_interp ? 8 : 1));
   std::vector<int> rcount(n_rec, 0);
   std::vector<Corner> cs;
   long long off = 0, toff = 0;
@@ -544,7 +616,17 @@ int build_plan(mamute_ctx* ctx, const mamute_grid* g, bool dens, int n_src, cons
   P.nrec = n_rec;
   P.one_node = true;
   for (int r = 0; r < n_rec; ++r) P.one_node = P.one_node && rcount[r] == 1;
-  // Work items: one per tile, all planes, for the forward and adjoint kernels.
+  return MAMUTE_OK;
+}
+
+// Work items and receiver tables of planned windows: the forward kernels', and
+// with adj_mode >= 0 the adjoint kernels' for that mode (MODE_ADJ when the
+// forward states are recomputed, MODE_ADJ_STORED when every imaging term is
+// kept: their shared-memory footprints, hence occupancies, differ).
+int plan_tiles(mamute_ctx* ctx, Plan& P, const int* tiles, int adj_mode) {
+  const int n_src = (int)P.vols.size(), n_rec = P.nrec;
+  const bool dens = P.dens;
+  const std::vector<NodeEntry>& ent = P.ent;
   int n_sm = 0;
   cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, ctx->device);
   if (n_sm < 1) n_sm = 1;
@@ -552,8 +634,11 @@ int build_plan(mamute_ctx* ctx, const mamute_grid* g, bool dens, int n_src, cons
   auto pick = [&](int i, const char* env) { return (tiles && tiles[i] > 0) ? tiles[i] : env_int(env, 0); };
   TileChoice fc = choose_tiles(P.vols, dens, P.pml, fmode, n_sm, pick(0, "MAMUTE_TX"), pick(1, "MAMUTE_TY"),
                                pick(2, "MAMUTE_ZSPLIT"));
-  TileChoice ac = choose_tiles(P.vols, dens, P.pml, P.pml ? MODE_ADJ_STORED : adj_mode, n_sm, pick(3, "MAMUTE_ADJ_TX"),
-                               pick(4, "MAMUTE_ADJ_TY"), pick(5, "MAMUTE_ADJ_ZSPLIT"));
+  const int ax = pick(3, "MAMUTE_ADJ_TX"), ay = pick(4, "MAMUTE_ADJ_TY"), az = pick(5, "MAMUTE_ADJ_ZSPLIT");
+  TileChoice ac = fc;
+  if (adj_mode >= 0 || ax > 0 || ay > 0 || az > 0)  // (a shape asked for is checked in any call)
+    ac = choose_tiles(P.vols, dens, P.pml, P.pml ? MODE_ADJ_STORED : std::max(adj_mode, (int)MODE_ADJ), n_sm,
+                      ax, ay, az);
   if (fc.tilings.empty() || ac.tilings.empty())
     return fail(ctx, MAMUTE_EINVAL, "unsupported tile shape");
   P.tx = fc.tx; P.ty = fc.ty; P.atx = ac.tx; P.aty = ac.ty;
@@ -581,7 +666,6 @@ int build_plan(mamute_ctx* ctx, const mamute_grid* g, bool dens, int n_src, cons
                   P.rec_cell, P.rec_g, P.colmap, &ent_of_col);
   P.fwd_col_of_ent.assign(ent.size(), 0);
   for (size_t c = 0; c < ent_of_col.size(); ++c) P.fwd_col_of_ent[ent_of_col[c]] = (int)c;
-  P.ent = ent;
   // receiver -> internal columns of the forward tables, ascending
   P.rcol_ptr.assign(n_rec + 1, 0);
   for (int c = 0; c < P.ncol; ++c) ++P.rcol_ptr[P.colmap[c] + 1];
@@ -591,6 +675,7 @@ int build_plan(mamute_ctx* ctx, const mamute_grid* g, bool dens, int n_src, cons
     std::vector<int> fill(P.rcol_ptr.begin(), P.rcol_ptr.end() - 1);
     for (int c = 0; c < P.ncol; ++c) P.rcols[fill[P.colmap[c]]++] = c;
   }
+  if (adj_mode < 0) return MAMUTE_OK;
   make_items(ac, P.aitems, base);
   build_receivers(P, P.atx, ac.zsplit, ent, base, ac.tilings, P.aitems, P.arec_ptr, P.arec,
                   P.arec_cell, P.arec_g, P.acolmap);
@@ -622,14 +707,11 @@ cudaError_t aux_count(mamute_ctx* ctx, cudaError_t e) {
   return e;
 }
 
-int check_cfl(mamute_ctx* ctx, Plan& P, const float* vel) {
-  CK(cudaMemsetAsync(ctx->maxbits, 0, sizeof(unsigned int), ctx->stream));
-  CK(aux_count(ctx, launch_max(vel, (long long)P.nx * P.ny * P.nz, ctx->maxbits, ctx->stream)));
-  unsigned int bits = 0;
-  CK(cudaMemcpyAsync(&bits, ctx->maxbits, sizeof bits, cudaMemcpyDeviceToHost, ctx->stream));
-  CK(cudaStreamSynchronize(ctx->stream));
+// The CFL check on the maximum that start_coef reads back.
+int check_cfl(mamute_ctx* ctx, Plan& P) {
+  CK(cudaEventSynchronize(ctx->vmax_ev));
   float vmax;
-  std::memcpy(&vmax, &bits, sizeof vmax);
+  std::memcpy(&vmax, &ctx->host->maxbits, sizeof vmax);
   P.vmax = vmax;
   const double courant = (double)vmax * P.dt / P.h;
   if (!(courant <= cfl_bound()))
@@ -638,9 +720,14 @@ int check_cfl(mamute_ctx* ctx, Plan& P, const float* vel) {
   return MAMUTE_OK;
 }
 
-// Coefficients, geometry tables, pools and maps.
-int setup(mamute_ctx* ctx, Plan& P, const float* vel, const float* rho, bool need_psi,
-          bool need_acc) {
+// Issues the maximum velocity and the coefficient preparation, which run while
+// the host plans the tiles and receiver tables.
+int start_coef(mamute_ctx* ctx, const Plan& P, const float* vel, const float* rho) {
+  CK(cudaMemsetAsync(ctx->maxbits, 0, sizeof(unsigned int), ctx->stream));
+  CK(aux_count(ctx, launch_max(vel, (long long)P.nx * P.ny * P.nz, ctx->maxbits, ctx->stream)));
+  CK(cudaMemcpyAsync(&ctx->host->maxbits, ctx->maxbits, sizeof(unsigned int), cudaMemcpyDeviceToHost,
+                     ctx->stream));
+  CK(cudaEventRecord(ctx->vmax_ev, ctx->stream));
   const size_t nG = (size_t)P.Nz * P.Ny * P.pitchG;
   CK(ensure(ctx->coefA, nG * 4));
   if (P.dens) CK(ensure(ctx->coefM, nG * 4));
@@ -649,37 +736,45 @@ int setup(mamute_ctx* ctx, Plan& P, const float* vel, const float* rho, bool nee
                   (float*)ctx->coefA.p, P.dens ? (float*)ctx->coefM.p : nullptr,
                   P.dens ? (double*)ctx->srho.p : nullptr};
   CK(aux_count(ctx, launch_prep_coef(ca, ctx->stream)));
+  return MAMUTE_OK;
+}
+
+// Geometry tables, pools and maps (need_psi: of the adjoint too).
+int setup(mamute_ctx* ctx, Plan& P, const float* vel, const float* rho, bool need_psi,
+          bool need_acc) {
   const size_t pool = (size_t)P.pool_elems * 4;
   for (int i = 0; i < 2; ++i) CK(ensure(ctx->pool[i], pool));
   if (need_psi)
     for (int i = 0; i < 2; ++i) CK(ensure(ctx->psi[i], pool));
   if (need_acc) CK(ensure(ctx->acc, pool));
-  CK(upload(ctx->vols, P.vols, ctx->stream));
-  CK(upload(ctx->items, P.items, ctx->stream));
-  CK(upload(ctx->recptr, P.rec_ptr, ctx->stream));
-  CK(upload(ctx->rec, P.rec, ctx->stream));
-  CK(upload(ctx->colmap, P.colmap, ctx->stream));
-  CK(upload(ctx->cells, P.rec_cell, ctx->stream));
-  CK(upload(ctx->gvals, P.rec_g, ctx->stream));
-  CK(upload(ctx->aitems, P.aitems, ctx->stream));
-  CK(upload(ctx->arecptr, P.arec_ptr, ctx->stream));
-  CK(upload(ctx->arec, P.arec, ctx->stream));
-  CK(upload(ctx->acolmap, P.acolmap, ctx->stream));
-  CK(upload(ctx->acells, P.arec_cell, ctx->stream));
-  CK(upload(ctx->agvals, P.arec_g, ctx->stream));
-  CK(upload(ctx->srccell, P.src_cell, ctx->stream));
-  CK(upload(ctx->srcw, P.src_w, ctx->stream));
+  CK(upload(ctx, ctx->vols, P.vols));
+  CK(upload(ctx, ctx->items, P.items));
+  CK(upload(ctx, ctx->recptr, P.rec_ptr));
+  CK(upload(ctx, ctx->rec, P.rec));
+  CK(upload(ctx, ctx->colmap, P.colmap));
+  CK(upload(ctx, ctx->cells, P.rec_cell));
+  CK(upload(ctx, ctx->gvals, P.rec_g));
+  if (need_psi) {
+    CK(upload(ctx, ctx->aitems, P.aitems));
+    CK(upload(ctx, ctx->arecptr, P.arec_ptr));
+    CK(upload(ctx, ctx->arec, P.arec));
+    CK(upload(ctx, ctx->acolmap, P.acolmap));
+    CK(upload(ctx, ctx->acells, P.arec_cell));
+    CK(upload(ctx, ctx->agvals, P.arec_g));
+  }
+  CK(upload(ctx, ctx->srccell, P.src_cell));
+  CK(upload(ctx, ctx->srcw, P.src_w));
   if (!P.one_node) {
     std::vector<int> iota(P.ncol);
     for (int c = 0; c < P.ncol; ++c) iota[c] = c;
-    CK(upload(ctx->ident, iota, ctx->stream));
-    CK(upload(ctx->rcolptr, P.rcol_ptr, ctx->stream));
-    CK(upload(ctx->rcols, P.rcols, ctx->stream));
+    CK(upload(ctx, ctx->ident, iota));
+    CK(upload(ctx, ctx->rcolptr, P.rcol_ptr));
+    CK(upload(ctx, ctx->rcols, P.rcols));
     CK(ensure(ctx->ecol, (size_t)P.ncol * P.nt * 4));
   }
-  CK(upload(ctx->gx, P.gx, ctx->stream));
-  CK(upload(ctx->gy, P.gy, ctx->stream));
-  CK(upload(ctx->gz, P.gz, ctx->stream));
+  CK(upload(ctx, ctx->gx, P.gx));
+  CK(upload(ctx, ctx->gy, P.gy));
+  CK(upload(ctx, ctx->gz, P.gz));
   // Scales at receivers (both tables) and sources.
   GeomArgs ga{vel, rho, (int)P.rec.size(), (int)P.vols.size(), (const long long*)ctx->cells.p,
               (const float*)ctx->gvals.p, (RecEntry*)ctx->rec.p, (const long long*)ctx->srccell.p,
@@ -688,7 +783,7 @@ int setup(mamute_ctx* ctx, Plan& P, const float* vel, const float* rho, bool nee
   GeomArgs gb{vel, rho, (int)P.arec.size(), 0, (const long long*)ctx->acells.p,
               (const float*)ctx->agvals.p, (RecEntry*)ctx->arec.p, nullptr, nullptr, nullptr,
               P.h, P.dt};
-  CK(aux_count(ctx, launch_geometry(gb, ctx->stream)));
+  if (need_psi) CK(aux_count(ctx, launch_geometry(gb, ctx->stream)));
   // Tensor maps (layout in ShotMaps).
   std::vector<ShotMaps> maps(P.vols.size());
   for (size_t s = 0; s < P.vols.size(); ++s) {
@@ -717,7 +812,7 @@ int setup(mamute_ctx* ctx, Plan& P, const float* vel, const float* rho, bool nee
     }
     if (!ok) return fail(ctx, MAMUTE_ECUDA, "cuTensorMapEncodeTiled failed (shot %d)", (int)s);
   }
-  CK(upload(ctx->maps, maps, ctx->stream));
+  CK(upload(ctx, ctx->maps, maps));
   ctx->hmaps = maps;
   std::vector<CoefMaps> cm(2);  // [0]: forward tile boxes, [1]: adjoint tile boxes
   for (int v = 0; v < 2; ++v) {
@@ -728,7 +823,7 @@ int setup(mamute_ctx* ctx, Plan& P, const float* vel, const float* rho, bool nee
         encode3d(ctx, &cm[v].m[1], (const float*)ctx->coefM.p, P.Nx, P.Ny, P.Nz, P.pitchG, bx, by))
       return fail(ctx, MAMUTE_ECUDA, "cuTensorMapEncodeTiled failed (M)");
   }
-  CK(upload(ctx->cmaps, cm, ctx->stream));
+  CK(upload(ctx, ctx->cmaps, cm));
   return MAMUTE_OK;
 }
 
@@ -827,9 +922,8 @@ StepArgs fwd_args(mamute_ctx* ctx, const Plan& P, int n, const float* wavelet, f
 }
 
 int finish(mamute_ctx* ctx) {
-  int st = 0;
-  CK(cudaMemcpyAsync(&st, ctx->status, sizeof st, cudaMemcpyDeviceToHost, ctx->stream));
   CK(cudaStreamSynchronize(ctx->stream));
+  const int st = *(volatile int*)ctx->status;
   if (ctx->timing && ctx->ev0_set) {
     float ms = 0.f;
     CK(cudaEventElapsedTime(&ms, ctx->ev0, ctx->ev1));
@@ -848,7 +942,8 @@ int check_common(mamute_ctx* ctx, const mamute_grid* g, const float* vel, const 
   ctx->launches = 0;
   if (!vel || !wavelet || !g) return fail(ctx, MAMUTE_EINVAL, "NULL vel, wavelet or grid");
   CK(cudaSetDevice(ctx->device));
-  CK(cudaMemsetAsync(ctx->status, 0, sizeof(int), ctx->stream));
+  CK(stage_reset(ctx));
+  *ctx->status = 0;  // no kernel of an earlier call is in flight
   return MAMUTE_OK;
 }
 
@@ -857,6 +952,15 @@ int check_common(mamute_ctx* ctx, const mamute_grid* g, const float* vel, const 
     int rc_ = (x);           \
     if (rc_ != MAMUTE_OK) return rc_; \
   } while (0)
+
+// A call that fails after it has launched work leaves none in flight: the
+// caller's arrays may go when it returns.  (A call that succeeds has
+// synchronised already, and the wait returns at once.)
+struct InFlight {
+  mamute_ctx* ctx;
+  explicit InFlight(mamute_ctx* c) : ctx(c) {}
+  ~InFlight() { cudaStreamSynchronize(ctx->stream); }
+};
 
 // Two-level forward launches (stencil_pair.cu), on request (time_blocking =
 // 2, or MAMUTE_PAIRS=1): one shot, no free surface, every tile resident at
@@ -929,12 +1033,12 @@ bool plan_pairs(mamute_ctx* ctx, Plan& P, const mamute_opts* opts) {
 
 // Tables, tensor maps and progress flags of the two-level launches.
 int setup_pairs(mamute_ctx* ctx, const Plan& P, const float* vel, const float* rho) {
-  CK(upload(ctx->pitems, P.pitems, ctx->stream));
-  CK(upload(ctx->pnbr, P.pnbr, ctx->stream));
-  CK(upload(ctx->precptr, P.prec_ptr, ctx->stream));
-  CK(upload(ctx->prec, P.prec, ctx->stream));
-  CK(upload(ctx->pcells, P.prec_cell, ctx->stream));
-  CK(upload(ctx->pgvals, P.prec_g, ctx->stream));
+  CK(upload(ctx, ctx->pitems, P.pitems));
+  CK(upload(ctx, ctx->pnbr, P.pnbr));
+  CK(upload(ctx, ctx->precptr, P.prec_ptr));
+  CK(upload(ctx, ctx->prec, P.prec));
+  CK(upload(ctx, ctx->pcells, P.prec_cell));
+  CK(upload(ctx, ctx->pgvals, P.prec_g));
   GeomArgs ga{vel, rho, (int)P.prec.size(), 0, (const long long*)ctx->pcells.p,
               (const float*)ctx->pgvals.p, (RecEntry*)ctx->prec.p, nullptr, nullptr, nullptr,
               P.h, P.dt};
@@ -957,7 +1061,7 @@ int setup_pairs(mamute_ctx* ctx, const Plan& P, const float* vel, const float* r
   else
     pm[0].m[5] = pm[0].m[4];
   if (!ok) return fail(ctx, MAMUTE_ECUDA, "cuTensorMapEncodeTiled failed (two-level maps)");
-  CK(upload(ctx->pmaps, pm, ctx->stream));
+  CK(upload(ctx, ctx->pmaps, pm));
   CK(ensure(ctx->pflags, P.pitems.size() * 4));
   return MAMUTE_OK;
 }
@@ -1020,7 +1124,7 @@ int do_smooth(mamute_ctx* ctx, int nx, int ny, int nz, double h, int mode, const
         }
       }
     }
-    CK(upload(ctx->smMat, tab, ctx->stream));
+    CK(upload(ctx, ctx->smMat, tab));
     if (bessel) {
       CK(ensure(ctx->smLam, sizeof(RowCoef) * (size_t)ny * nz));
       ++ctx->launches;
@@ -1158,9 +1262,9 @@ int do_resample(mamute_ctx* ctx, int ntr, int nt_in, double dt_in, int nt_out, d
     std::vector<float> wb((size_t)K * rows, 0.0f);
     for (int m = 0; m < rows; ++m)
       for (int k = ptr[m]; k < ptr[m + 1]; ++k) wb[(size_t)(col[k] - c0[m]) * rows + m] = w[k];
-    CK(upload(ctx->rsPtr, c0, ctx->stream));
-    CK(upload(ctx->rsCol, len, ctx->stream));
-    CK(upload(ctx->rsW, wb, ctx->stream));
+    CK(upload(ctx, ctx->rsPtr, c0));
+    CK(upload(ctx, ctx->rsCol, len));
+    CK(upload(ctx, ctx->rsW, wb));
     ctx->rsKey = key;
   }
   ++ctx->launches;
@@ -1315,8 +1419,8 @@ int cpml_setup(mamute_ctx* ctx, const Plan& P, std::vector<CpmlVol>& cv, int n_a
   }
   const size_t nb = b.size();
   b.insert(b.end(), c.begin(), c.end());
-  CK(upload(ctx->cprof, b, ctx->stream));
-  CK(upload(ctx->cvols, W, ctx->stream));
+  CK(upload(ctx, ctx->cprof, b));
+  CK(upload(ctx, ctx->cvols, W));
   const size_t mem = (size_t)n_arrays * T.elems * 4, pool = (size_t)P.pool_elems * 4;
   CK(ensure(ctx->cpml, mem));
   CK(ensure(ctx->cext, pool));
@@ -1358,12 +1462,15 @@ int run_model(mamute_ctx* ctx, const mamute_grid* g, const float* vel, const flo
               float* host_seis = nullptr) {
   TRY(check_common(ctx, g, vel, wavelet));
   Plan P;
-  TRY(build_plan(ctx, g, rho != nullptr, n_src, src_xyz, rec_offset, rec_xyz,
-                 opts ? opts->aperture : nullptr, P, opts ? opts->tiles : nullptr));
+  TRY(plan_windows(ctx, g, rho != nullptr, n_src, src_xyz, rec_offset, rec_xyz,
+                   opts ? opts->aperture : nullptr, P));
   if (P.ncol > 0 && !seis) return fail(ctx, MAMUTE_EINVAL, "seis is NULL");
   int ti = 0, ntd = P.nt;
   TRY(check_interp(ctx, g, opts, &ti, &ntd));
-  TRY(check_cfl(ctx, P, vel));
+  InFlight guard(ctx);
+  TRY(start_coef(ctx, P, vel, rho));
+  TRY(plan_tiles(ctx, P, opts ? opts->tiles : nullptr, -1));
+  TRY(check_cfl(ctx, P));
   const bool ph = opts && opts->phess;
   if (P.pml && ph) return fail(ctx, MAMUTE_EINVAL, "phess is not available with pml");
   PmlTables T;
@@ -1595,14 +1702,14 @@ int run_gradient(mamute_ctx* ctx, const mamute_grid* g, const float* vel, const 
   TRY(check_common(ctx, g, vel, wavelet));
   if (!grad) return fail(ctx, MAMUTE_EINVAL, "grad is NULL");
   Plan P;
-  TRY(build_plan(ctx, g, rho != nullptr, n_src, src_xyz, rec_offset, rec_xyz,
-                 opts ? opts->aperture : nullptr, P, opts ? opts->tiles : nullptr));
+  TRY(plan_windows(ctx, g, rho != nullptr, n_src, src_xyz, rec_offset, rec_xyz,
+                   opts ? opts->aperture : nullptr, P));
   if (P.ncol > 0 && !d_in) return fail(ctx, MAMUTE_EINVAL, "data is NULL");
   int ti = 0, ntd = P.nt;
   TRY(check_interp(ctx, g, opts, &ti, &ntd));
   const int smode = opts ? opts->smooth_mode : 0;
   if (smode < 0 || smode > 2) return fail(ctx, MAMUTE_EINVAL, "smooth_mode must be 0, 1 or 2");
-  TRY(check_cfl(ctx, P, vel));
+  InFlight guard(ctx);
   {
     // When every step's imaging term will be kept (the storage decision
     // below, made here ahead of it on the same figures), choose the adjoint
@@ -1616,14 +1723,9 @@ int run_gradient(mamute_ctx* ctx, const mamute_grid* g, const float* vel, const 
       const double need = (double)P.nt * P.term_elems * 4;
       keep_all = need <= fr_ * ((double)fr + (double)ctx->tstore.bytes + (double)ctx->slots.bytes);
     }
-    if (keep_all) {
-      Plan Q;
-      TRY(build_plan(ctx, g, rho != nullptr, n_src, src_xyz, rec_offset, rec_xyz,
-                     opts ? opts->aperture : nullptr, Q, opts ? opts->tiles : nullptr,
-                     MODE_ADJ_STORED));
-      Q.vmax = P.vmax;
-      P = std::move(Q);
-        }
+    TRY(start_coef(ctx, P, vel, rho));
+    TRY(plan_tiles(ctx, P, opts ? opts->tiles : nullptr, keep_all ? MODE_ADJ_STORED : MODE_ADJ));
+    TRY(check_cfl(ctx, P));
   }
   const bool ph = opts && opts->phess;
   if (P.pml && ph) return fail(ctx, MAMUTE_EINVAL, "phess is not available with pml");
@@ -1692,7 +1794,7 @@ int run_gradient(mamute_ctx* ctx, const mamute_grid* g, const float* vel, const 
                       CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE))
         return fail(ctx, MAMUTE_ECUDA, "cuTensorMapEncodeTiled failed (term store)");
     }
-    CK(upload(ctx->maps, ctx->hmaps, ctx->stream));
+    CK(upload(ctx, ctx->maps, ctx->hmaps));
   } else if (nsnap > 0) {
     slots = std::min(nsnap, P.nt);
   } else {
@@ -1733,7 +1835,7 @@ int run_gradient(mamute_ctx* ctx, const mamute_grid* g, const float* vel, const 
               encode3d(ctx, m + 2, base, V.Nx, V.Ny, V.Nz, V.pitch, P.atx + 8, P.aty + 8))
             return fail(ctx, MAMUTE_ECUDA, "cuTensorMapEncodeTiled failed (checkpoint slot)");
         }
-    CK(upload(ctx->slotmaps, sm, ctx->stream));
+    CK(upload(ctx, ctx->slotmaps, sm));
   }
   auto buf_ptr = [&](Buf b) -> char* {
     return b.slot < 0 ? (char*)ctx->pool[b.part].p
@@ -1930,10 +2032,10 @@ int run_gradient(mamute_ctx* ctx, const mamute_grid* g, const float* vel, const 
       CK(cudaMemsetAsync(grad, 0, (size_t)ztop * P.nx * P.ny * 4, ctx->stream));
   }
   if (misfit) {
-    double J = 0.0;
-    CK(cudaMemcpyAsync(&J, ctx->misfit.p, sizeof J, cudaMemcpyDeviceToHost, ctx->stream));
+    CK(cudaMemcpyAsync(&ctx->host->value, ctx->misfit.p, sizeof(double), cudaMemcpyDeviceToHost,
+                       ctx->stream));
     TRY(finish(ctx));
-    *misfit = J;
+    *misfit = ctx->host->value;
     return MAMUTE_OK;
   }
   return finish(ctx);
@@ -1959,11 +2061,14 @@ int run_gn(mamute_ctx* ctx, const mamute_grid* g, const float* vel, const float*
           return fail(ctx, MAMUTE_EINVAL, "every shot must record at the same receivers");
   }
   Plan P;
-  TRY(build_plan(ctx, g, rho != nullptr, n_src, src_xyz, rec_offset, rec_xyz, nullptr, P));
+  TRY(plan_windows(ctx, g, rho != nullptr, n_src, src_xyz, rec_offset, rec_xyz, nullptr, P));
   if (P.pml) return fail(ctx, MAMUTE_EINVAL, "the GN diagonal uses the sponge boundary (pml = 0)");
   if (!P.one_node)
     return fail(ctx, MAMUTE_EINVAL, "the Gauss-Newton diagonal needs receivers on grid nodes");
-  TRY(check_cfl(ctx, P, vel));
+  InFlight guard(ctx);
+  TRY(start_coef(ctx, P, vel, rho));
+  TRY(plan_tiles(ctx, P, nullptr, MODE_ADJ));
+  TRY(check_cfl(ctx, P));
   // Compact interior term layout: slot k of the ring is [nz][ny][nx].
   auto compact_terms = [](Plan& Q) {
     long long toff = 0;
@@ -2059,8 +2164,8 @@ int run_gn(mamute_ctx* ctx, const mamute_grid* g, const float* vel, const float*
   CK(ensure(ctx->gnS, (size_t)nb * N * 4));
   CK(ensure(ctx->gnR, (size_t)nb * N * 4));
   CK(ensure(ctx->gnW, std::max((size_t)kT * dft_max_bins() * 8, dft_tc_image_bytes(kT, nb))));
-  CK(upload(ctx->gnBins, bins, ctx->stream));
-  CK(upload(ctx->gnWts, wts, ctx->stream));
+  CK(upload(ctx, ctx->gnBins, bins));
+  CK(upload(ctx, ctx->gnWts, wts));
   CK(ensure(ctx->gnRow, (size_t)2 * std::max(P.ncol, 1) * 4));
   // With N a multiple of 4 every batch runs on the tensor cores, whose first
   // block overwrites the accumulators; else they start from zero.
@@ -2124,7 +2229,8 @@ int run_gn(mamute_ctx* ctx, const mamute_grid* g, const float* vel, const float*
       std::copy(rec_xyz, rec_xyz + 3 * (size_t)nr0, rxyz.begin() + 3 * (size_t)b * nr0);
       roff[b + 1] = (b + 1) * nr0;
     }
-    TRY(build_plan(ctx, g, rho != nullptr, Br, sxyz.data(), roff.data(), rxyz.data(), nullptr, Pr));
+    TRY(plan_windows(ctx, g, rho != nullptr, Br, sxyz.data(), roff.data(), rxyz.data(), nullptr, Pr));
+    TRY(plan_tiles(ctx, Pr, nullptr, MODE_ADJ));
     if (!Pr.one_node || Pr.Nz != P.Nz)
       return fail(ctx, MAMUTE_ECUDA, "receiver plan differs from the shot plan");
     Pr.vmax = P.vmax;
@@ -2269,8 +2375,12 @@ int mamute_ctx_create(mamute_ctx** out, int device, void* stream) {
     return MAMUTE_ECUDA;
   }
   ctx->encode = (PFN_cuTensorMapEncodeTiled_v12000)fn;
-  if (cudaMalloc(&ctx->status, 256) != cudaSuccess || cudaMalloc(&ctx->maxbits, 256) != cudaSuccess ||
-      ensure(ctx->misfit, 256) != cudaSuccess) {
+  if (cudaHostAlloc((void**)&ctx->host, sizeof(*ctx->host), cudaHostAllocMapped | cudaHostAllocPortable) ==
+      cudaSuccess)
+    ctx->status = &ctx->host->status;
+  if (!ctx->host || cudaMalloc(&ctx->maxbits, 256) != cudaSuccess ||
+      ensure(ctx->misfit, 256) != cudaSuccess ||
+      cudaEventCreateWithFlags(&ctx->vmax_ev, cudaEventDisableTiming) != cudaSuccess) {
     mamute_ctx_destroy(ctx);
     return MAMUTE_ENOMEM;
   }
@@ -2298,7 +2408,9 @@ void mamute_ctx_destroy(mamute_ctx* ctx) {
                    &ctx->prec, &ctx->pcells, &ctx->pgvals, &ctx->pmaps, &ctx->pflags,
                    &ctx->cpml, &ctx->cext, &ctx->cprof, &ctx->cvols};
   for (DevBuf* b : all) release(*b);
-  if (ctx->status) cudaFree(ctx->status);
+  if (ctx->host) cudaFreeHost(ctx->host);
+  if (ctx->stage) cudaFreeHost(ctx->stage);
+  if (ctx->vmax_ev) cudaEventDestroy(ctx->vmax_ev);
   if (ctx->maxbits) cudaFree(ctx->maxbits);
   for (cudaEvent_t ev : ctx->dft_ev) cudaEventDestroy(ev);
   if (ctx->ev0) cudaEventDestroy(ctx->ev0);
@@ -2409,6 +2521,7 @@ static int nn_begin(mamute_ctx* ctx) {
   if (!ctx) return MAMUTE_EINVAL;
   ctx->err.clear();
   CK(cudaSetDevice(ctx->device));
+  CK(stage_reset(ctx));
   return MAMUTE_OK;
 }
 
@@ -2432,10 +2545,8 @@ static CUresult encode_act(mamute_ctx* ctx, CUtensorMap* m, const void* p, int D
 
 // As nn_end, for kernels with bounded device-side waits.
 static int nn_end_status(mamute_ctx* ctx) {
-  int st = 0;
-  CK(cudaMemcpyAsync(&st, ctx->status, sizeof st, cudaMemcpyDeviceToHost, ctx->stream));
   CK(cudaStreamSynchronize(ctx->stream));
-  if (st & kErrTimeout) return fail(ctx, MAMUTE_ETIMEOUT, "a device-side wait ran out");
+  if (*(volatile int*)ctx->status & kErrTimeout) return fail(ctx, MAMUTE_ETIMEOUT, "a device-side wait ran out");
   return MAMUTE_OK;
 }
 
@@ -2465,7 +2576,7 @@ int mamute_conv3d(mamute_ctx* ctx, int D, int H, int W, const unsigned short* x,
                     CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE))
       return fail(ctx, MAMUTE_ECUDA, "conv3d: cuTensorMapEncodeTiled failed");
   }
-  CK(cudaMemsetAsync(ctx->status, 0, sizeof(int), ctx->stream));
+  *ctx->status = 0;
   CK(launch_conv(a, xmap, ctx->status, ctx->stream));
   return nn_end_status(ctx);
 }
@@ -2485,7 +2596,7 @@ int mamute_conv3d_wgrad(mamute_ctx* ctx, int D, int H, int W, const unsigned sho
   conv_gy_box(gbox);
   if (encode_act(ctx, &xmap, x, D, H, W, hbox) || encode_act(ctx, &gmap, gy, D, H, W, gbox))
     return fail(ctx, MAMUTE_ECUDA, "conv3d_wgrad: cuTensorMapEncodeTiled failed");
-  CK(cudaMemsetAsync(ctx->status, 0, sizeof(int), ctx->stream));
+  *ctx->status = 0;
   CK(launch_wgrad(a, xmap, gmap, ctx->status, gw, gb, ctx->stream));
   return nn_end_status(ctx);
 }

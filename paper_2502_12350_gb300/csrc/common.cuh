@@ -121,12 +121,19 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
   return ok != 0;
 }
 
+// The status word lies in mapped host memory; kErrTimeout is its only flag, so
+// a plain store does.
+__device__ __forceinline__ void report_timeout(int* status) {
+  *reinterpret_cast<volatile int*>(status) = kErrTimeout;
+  __threadfence_system();
+}
+
 // Bounded wait: returns false (and records a timeout) if the phase does not
 // complete within kSpinLimit polls.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* status) {
   for (long long i = 0; i < kSpinLimit; ++i)
     if (mbar_try_wait(bar, parity)) return true;
-  atomicOr(status, kErrTimeout);
+  report_timeout(status);
   return false;
 }
 

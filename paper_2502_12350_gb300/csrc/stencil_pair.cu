@@ -366,7 +366,7 @@ __global__ void __launch_bounds__((TX / 4) * (TY / 2) + 32, 1) pair_kernel(const
             return true;
           }
         }
-        atomicOr(a.status, kErrTimeout);
+        report_timeout(a.status);
         return false;
       };
       for (int z = 0; z < Nz; ++z) {

@@ -127,7 +127,7 @@ __device__ __forceinline__ bool tc_wait(uint64_t* bar, uint32_t parity, int* sta
     if (mbar_try_wait(bar, parity)) return true;
     if ((i & 255) == 255 && *abort_flag) return false;
   }
-  atomicOr(status, kErrTimeout);
+  report_timeout(status);
   *abort_flag = 1;
   return false;
 }

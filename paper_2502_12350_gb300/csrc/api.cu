@@ -1579,6 +1579,7 @@ int run_model(mamute_ctx* ctx, const mamute_grid* g, const float* vel, const flo
       } else {
         if (P.pml) TRY(cpml_step(ctx, T, false, n, (const float*)ctx->pool[n & 1].p));
         StepArgs a = fwd_args(ctx, P, n, wavelet, drow, mode);
+        a.chained = !P.pml && !pairs && n > t0;
         CK(step_launch(ctx, P, a, (int)P.items.size(), P.planes, P.tx, P.ty, mode));
         n += 1;
       }
@@ -1853,6 +1854,7 @@ int run_gradient(mamute_ctx* ctx, const mamute_grid* g, const float* vel, const 
     }
   };
   Buf cur{-1, 0}, prev{-1, 1};  // u^0 and u^{-1}
+  bool chained = false;         // the last operation issued is a step launch
   int sn = 0;                   // time level held in cur
   int recorded = 0;             // steps whose data sample is recorded
   auto fwd_step = [&](int n, bool first_sweep) -> int {
@@ -1868,6 +1870,8 @@ int run_gradient(mamute_ctx* ctx, const mamute_grid* g, const float* vel, const 
     a.sU = a.sF;
     a.fout = (float*)buf_ptr(out);
     if (P.pml) TRY(cpml_step(ctx, T, false, n, (const float*)buf_ptr(cur)));
+    a.chained = chained && !P.pml;
+    chained = true;
     CK(step_launch(ctx, P, a, (int)P.items.size(), P.planes, P.tx, P.ty, mode));
     if (rec) recorded = n + 1;
     prev = cur;
@@ -1958,10 +1962,13 @@ int run_gradient(mamute_ctx* ctx, const mamute_grid* g, const float* vel, const 
     a.zs = P.zs;
     if (P.pml)  // memory-variable multipliers and E from psi^{k+1}
       TRY(cpml_step(ctx, T, true, i, (const float*)ctx->psi[(k + 1) & 1].p));
+    a.chained = chained && !P.pml;
+    chained = true;
     CK(step_launch(ctx, P, a, (int)P.aitems.size(), P.aplanes, P.atx, P.aty, mode));
     return MAMUTE_OK;
   };
   auto begin_adjoint = [&]() -> int {
+    chained = false;
     TRY(make_residual());
     if (P.pml)  // the memory variables' multipliers start at zero
       CK(cudaMemsetAsync(ctx->cpml.p, 0, (size_t)kPmlArraysGradient * T.elems * 4, ctx->stream));
@@ -1989,6 +1996,7 @@ int run_gradient(mamute_ctx* ctx, const mamute_grid* g, const float* vel, const 
           break;
         case REV_STORE: {  // slot half (m & 1) holds u^m
           const Buf dc{A.a, sn & 1}, dp{A.a, (sn + 1) & 1};
+          chained = false;
           if (!(dc == cur))
             CK(cudaMemcpyAsync(buf_ptr(dc), buf_ptr(cur), pool, cudaMemcpyDeviceToDevice, ctx->stream));
           if (!(dp == prev))
@@ -1997,6 +2005,7 @@ int run_gradient(mamute_ctx* ctx, const mamute_grid* g, const float* vel, const 
         }
         case REV_RESTORE:
           if (A.a < 0) {
+            chained = false;
             CK(cudaMemsetAsync(ctx->pool[0].p, 0, pool, ctx->stream));
             CK(cudaMemsetAsync(ctx->pool[1].p, 0, pool, ctx->stream));
             cur = Buf{-1, 0};
@@ -2208,6 +2217,7 @@ int run_gn(mamute_ctx* ctx, const mamute_grid* g, const float* vel, const float*
       StepArgs a = fwd_args(ctx, P, n, wavelet, nullptr, MODE_FWD_STORE);
       a.items = (const WorkItem*)ctx->items.p + ib;
       a.tstore = V + (size_t)(n % kT) * Nb - (size_t)s0 * N;
+      a.chained = n % kT != 0;
       CK(step_launch(ctx, P, a, ie - ib, P.planes, P.tx, P.ty, MODE_FWD_STORE));
       if ((n + 1) % kT == 0) TRY(flush(n + 1));
     }
@@ -2284,6 +2294,7 @@ int run_gn(mamute_ctx* ctx, const mamute_grid* g, const float* vel, const float*
       a.rec_ptr = (const int*)ctx->arecptr.p;
       a.rec = (const RecEntry*)ctx->arec.p;
       a.rin = (j == 0) ? imp_row : zero_row;
+      a.chained = j % kT != 0;
       a.status = ctx->status;
       a.zs = R->zs;
       CK(step_launch(ctx, *R, a, ie - ib, R->aplanes, R->atx, R->aty, MODE_ADJ_TERM));

@@ -47,6 +47,9 @@ struct StepArgs {
   const float* rin;       // adjoint: residual row injected at this step
   int* status;            // error flags
   int zs;                 // padded plane of a free surface (odd image above it), -1 if none
+  // The previous operation on the stream is a step launch: this one may start
+  // beside its tail (programmatic dependent launch).
+  bool chained;
 };
 
 // Tensor maps of one shot for the two-level kernel (boxes of its tile):

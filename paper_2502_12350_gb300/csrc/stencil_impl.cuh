@@ -235,6 +235,11 @@ __global__ void __launch_bounds__((TX / 4) * TY + 32, (MinBlocks<TX, TY, MODE>::
     fence_barrier_init();
   }
   __syncthreads();
+  // A chained launch (StepArgs::chained) may start while the previous step
+  // ends: everything above reads tables that no step writes.  The producer
+  // waits for the previous step before its first load; the other threads act
+  // on its loads alone, so the wait covers their stores too.  (500 steps of 96^3:
+  // 5.58 -> 4.98 ms; 800 launches of a 320^3 gradient: 88.5 -> 85.7 ms.)
 
   // Maps of the buffers this launch reads (chosen by the host per step).
   const CUtensorMap* mapF = a.mF + (long long)it.vol * a.sF;
@@ -257,6 +262,7 @@ __global__ void __launch_bounds__((TX / 4) * TY + 32, (MinBlocks<TX, TY, MODE>::
       if (ACC) tmap_acquire(mapAcc);
       if (TERM) tmap_acquire(mapT);
       if (PML) tmap_acquire(mapE);
+      dependency_wait();
       const int nu = npl + 2 * kHalo;
       const int cx = V.cx0 + x0, cy = V.cy0 + y0;
       int nF = 0, nC = 0;  // loads issued into the halo and centre rings
@@ -308,6 +314,7 @@ __global__ void __launch_bounds__((TX / 4) * TY + 32, (MinBlocks<TX, TY, MODE>::
           ++nC;
         }
       }
+      launch_dependents();  // every load is issued: the last planes remain
     }
     return;
   }
@@ -548,8 +555,17 @@ static cudaError_t launch_one(const StepArgs& a, int n_items, int max_planes, cu
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occupancy, step_kernel<TX, TY, DENS, MODE, PML>,
                                                          (TX / 4) * TY + 32, sm);
   }
-  step_kernel<TX, TY, DENS, MODE, PML><<<n_items, (TX / 4) * TY + 32, sm, s>>>(a);
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)n_items);
+  cfg.blockDim = dim3((TX / 4) * TY + 32);
+  cfg.dynamicSmemBytes = sm;
+  cfg.stream = s;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = a.chained ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, step_kernel<TX, TY, DENS, MODE, PML>, a);
 }
 
 template <int TX, int TY, int MODE, bool PML = false>

@@ -441,7 +441,10 @@ TileChoice choose_tiles(const std::vector<VolDesc>& vols, bool dens, bool pml, i
         if (force_z > 0 && zs != force_z) continue;
         if (force_z <= 0 && zs > 1 && Nz / zs < 8) break;
         if (per_sm < 1) continue;
-        const long long items = tiles * zs;
+        // blocks of ceil(Nz / zs) planes: fewer than zs where the last ones
+        // would be empty (34 planes in 16 blocks are 12 of 3 planes)
+        const int blocks = (Nz + (Nz + zs - 1) / zs - 1) / ((Nz + zs - 1) / zs);
+        const long long items = tiles * blocks;
         const long long per = (items + n_sm - 1) / n_sm;  // items on the busiest SM
         const double warps = (double)std::min<long long>(per_sm, per) * warps_cta;
         const double occ = std::min(1.0, warps / 16.0);
@@ -455,7 +458,7 @@ TileChoice choose_tiles(const std::vector<VolDesc>& vols, bool dens, bool pml, i
           best_cost = cost;
           best.tx = TX;
           best.ty = TY;
-          best.zsplit = zs;
+          best.zsplit = blocks;
           best.tilings = tl;
         }
       }

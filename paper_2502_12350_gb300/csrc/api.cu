@@ -386,11 +386,25 @@ int blocks_per_sm(int tx, int ty, bool dens, bool pml, int mode, int planes) {
 }
 
 // Chooses, among the compiled tile shapes, the shape, a row refinement and a
-// split of the planes into z blocks that minimise the work of the busiest
-// SM: ceil(items / SMs) items of (box-bound points x planes), divided by a
-// factor for the resident warps (per-SM bandwidth falls off below about
-// 16 warps).  Items beyond the resident slots run in later waves, which the
-// same count captures.  MAMUTE_TX / MAMUTE_TY force a shape.
+// split of the planes into z blocks with the least modelled time of the
+// busiest SM, which has ceil(items / SMs) items:
+//   throughput  items x points per plane x planes at kRate points per us (kRateL2
+//               where all arrays fit in L2).  A CTA loads and computes its
+//               whole box, so the points are the mean of the largest tile's
+//               and the box's, the box weighted by its halo loads; z blocks
+//               prime with 8 halo planes of one of ~4 arrays (2 planes' worth);
+//               divided by a factor for the resident warps (per-SM bandwidth
+//               falls off below about 16 warps).
+//   latency     each wave of resident items: start-up and priming, and the
+//               dependent chain of a plane, kPlane us.
+// Fitted to measured sweeps: 96^3 at 16 B per point (48x16 in 24 blocks 6.0 us
+// a step, 48x16 in 12 8.4, 64x16 in 12 10.4), 20 windows of 136x120x104 (72x16
+// in 4 139 us, 64x16 in 4 160, 128x8 in 1 190), the recomputing adjoint of
+// 213x202x163 (32x16 in 3 54 us, 72x16 in 3 58, 32x8 in 4 72).
+// MAMUTE_TX / MAMUTE_TY force a shape.
+constexpr double kRate = 2300.0, kRateL2 = 4500.0, kL2Bytes = 100e6;
+constexpr double kStart = 3.2, kPlane = 0.4;
+
 struct TileChoice {
   int tx = 64, ty = 16, zsplit = 1;
   std::vector<Tiling> tilings;
@@ -400,10 +414,13 @@ TileChoice choose_tiles(const std::vector<VolDesc>& vols, bool dens, bool pml, i
                         int force_tx, int force_ty, int force_z) {
   static const int shapes[][2] = {{64, 16}, {72, 16}, {48, 16}, {96, 8}, {64, 8},
                                   {128, 8}, {32, 16}, {32, 8}};
-  static const int zsplits[] = {1, 2, 3, 4, 6, 8, 12, 16};
+  static const int zsplits[] = {1, 2, 3, 4, 5, 6, 7, 8, 10, 12, 14, 16, 20, 24, 32, 48};
   TileChoice best;
   double best_cost = -1.0;
   const int Nz = vols.empty() ? 1 : vols[0].Nz;
+  double bytes = 0.0;  // of about five arrays
+  for (const VolDesc& V : vols) bytes += 20.0 * V.pitch * V.Ny * V.Nz;
+  const double rate = bytes < kL2Bytes ? kRateL2 : kRate;
   for (const auto& sh : shapes) {
     const int TX = sh[0], TY = sh[1];
     if (force_tx > 0 && (TX != force_tx || TY != force_ty)) continue;
@@ -430,16 +447,17 @@ TileChoice choose_tiles(const std::vector<VolDesc>& vols, bool dens, bool pml, i
         // rows refined only while tiles stay at least half full
         if (r > 1 && 2 * (V.Ny / nrows) < TY) { ok = false; break; }
         tiles += (long long)(T.xs.size() - 1) * (T.ys.size() - 1);
-        // a CTA computes its whole box even when the tile is smaller
-        maxpts = std::max(maxpts, std::max((double)max_piece(T.xs) * max_piece(T.ys),
-                                           0.6 * TX * TY));
+        maxpts = std::max(maxpts, (double)max_piece(T.xs) * max_piece(T.ys));
         tl.push_back(std::move(T));
       }
       if (!ok || tiles <= 0) continue;
+      // 1.69: halo box over tile of 64 x 16
+      const double halo = (double)(TX + 8) * (TY + 8) / (TX * TY) / 1.69;
+      const double pts = 0.5 * maxpts + 0.5 * TX * TY * (0.6 + 0.4 * halo);
       for (size_t k = 0; k < sizeof zsplits / sizeof zsplits[0]; ++k) {
         const int zs = zsplits[k], per_sm = per_sm_of[k];
         if (force_z > 0 && zs != force_z) continue;
-        if (force_z <= 0 && zs > 1 && Nz / zs < 8) break;
+        if (force_z <= 0 && zs > 1 && Nz / zs < 4) break;
         if (per_sm < 1) continue;
         // blocks of ceil(Nz / zs) planes: fewer than zs where the last ones
         // would be empty (34 planes in 16 blocks are 12 of 3 planes)
@@ -448,11 +466,12 @@ TileChoice choose_tiles(const std::vector<VolDesc>& vols, bool dens, bool pml, i
         const long long per = (items + n_sm - 1) / n_sm;  // items on the busiest SM
         const double warps = (double)std::min<long long>(per_sm, per) * warps_cta;
         const double occ = std::min(1.0, warps / 16.0);
-        // z-block priming reads 8 extra halo planes of one of ~4 arrays
-        const double planes = (double)((Nz + zs - 1) / zs) + (zs > 1 ? 2.0 : 0.0);
-        const double cost = (double)per * maxpts * planes / occ;
+        const double planes = (double)((Nz + zs - 1) / zs);
+        const double waves = (double)((per + per_sm - 1) / per_sm);
+        const double cost = (double)per * pts * (planes + (zs > 1 ? 2.0 : 0.0)) / (rate * occ) +
+                            waves * (kStart + kPlane * planes);
         if (env_int("MAMUTE_VERBOSE", 0) >= 2)
-          fprintf(stderr, "mamute tiles: mode %d %dx%d rows x%d z%d: %d per SM, cost %.0f\n", mode, TX,
+          fprintf(stderr, "mamute tiles: mode %d %dx%d rows x%d z%d: %d per SM, cost %.1f us\n", mode, TX,
                   TY, r, zs, per_sm, cost);
         if (best_cost < 0 || cost < best_cost * (1.0 - 1e-3)) {
           best_cost = cost;

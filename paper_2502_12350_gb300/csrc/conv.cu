@@ -63,29 +63,39 @@ __device__ __forceinline__ int swz(int v, int half) { return 2 * v + (half ^ ((v
 
 // Weight gradient: per CTA partial sums over its tiles of
 // gw[tap][o][i] = sum_p gy[p][o] x[p + tap - 1][i] and gb[o] = sum_p gy[p][o].
-// Persistent like the forward kernel: per 16 x 8 x 4 tile one TMA load
-// brings the 18 x 10 x 6 halo of x and one the 16 x 8 x 4 tile of gy (both
-// with the 32-byte swizzle) into a double buffer.  Warp w accumulates taps
-// w, w + 8, w + 16, w + 24; per output row the A fragment is gy^T (16 out
-// channels x 16 voxels) and the B fragment the shifted x row.  Warp 0 also
-// sums gy for the bias from its A fragments.
+// Persistent, one CTA per SM: per 16 x 8 x 4 tile one TMA load brings the
+// 18 x 10 x 6 halo of x and one the 16 x 8 x 4 tile of gy (both with the
+// 32-byte swizzle) into a ring of kWStages stages.  Warp (dx, zz) takes output
+// plane zz and the 9 taps of one dx: the 8 rows' A fragments gy^T (16 out
+// channels x 16 voxels) stay in registers for the whole plane, and each
+// fragment B of a shifted halo row is used for the three rows (dy) that it
+// feeds, so a plane costs 38 ldmatrix per warp for 144 products.  (Taps dealt
+// to warps, A and B loaded per tap and row, took 2.5 times the shared-memory
+// reads, the bound of that form: 114 us for 80x160x160, now 71.)  The dx = 0 warps
+// also sum gy for the bias from their A fragments.  The four planes' sums are
+// added in order at the end.
 constexpr int kGTile = kFZ * kTY * kTX * kC * 2;  // bytes of a gy tile
 static_assert(kGTile % 256 == 0, "gy tiles must stay 256-byte aligned");
 constexpr int kWStage = kFHalo + kGTile;
+constexpr int kWStages = 4;
+constexpr int kWThreads = 32 * 3 * kFZ;
+static_assert(kWStage % 256 == 0, "stages must stay 256-byte aligned");
+static_assert(kFZ * (kTaps * kC * kC + kC) * 4 <= kWStages * kWStage, "the planes' sums reuse the stages");
 
 __device__ __forceinline__ float2 bf2x2(uint32_t v) {
   return make_float2(__uint_as_float(v << 16), __uint_as_float(v & 0xffff0000u));
 }
 
-__global__ void __launch_bounds__(256, 2)
+__global__ void __launch_bounds__(kWThreads, 1)
     conv_wgrad_kernel(const __grid_constant__ CUtensorMap xmap,
                       const __grid_constant__ CUtensorMap gmap, WgradArgs a, int* status) {
   extern __shared__ unsigned char wsm_raw[];
   unsigned char* dsm = wsm_raw + ((256 - (smem_u32(wsm_raw) & 255)) & 255);
-  __shared__ uint64_t bar[2];
+  __shared__ uint64_t bar[kWStages];
   __shared__ int abort_flag;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int mat = lane >> 3, r = lane & 7;
+  const int dx = warp % 3, zz = warp / 3;
   const int tiles_x = (a.W + kTX - 1) / kTX, tiles_y = (a.H + kTY - 1) / kTY;
   const int tiles_z = (a.D + kFZ - 1) / kFZ;
   const long long n_tiles = (long long)tiles_x * tiles_y * tiles_z;
@@ -99,69 +109,78 @@ __global__ void __launch_bounds__(256, 2)
     tma_load_4d(st + kFHalo, &gmap, 0, x0, y0, z0, &bar[b]);
   };
   if (threadIdx.x == 0) {
-    mbar_init(&bar[0], 1);
-    mbar_init(&bar[1], 1);
+    for (int b = 0; b < kWStages; ++b) mbar_init(&bar[b], 1);
     fence_barrier_init();
     abort_flag = 0;
   }
   __syncthreads();
-  if (threadIdx.x == 0 && (long long)blockIdx.x < n_tiles) issue(0, blockIdx.x);
-  float acc[4][2][4];
+  int issued = 0;  // tiles of this CTA whose loads are issued (thread 0)
+  auto issue_to = [&](int n) {
+    for (; issued < n && blockIdx.x + (long long)issued * gridDim.x < n_tiles; ++issued)
+      issue(issued % kWStages, blockIdx.x + (long long)issued * gridDim.x);
+  };
+  float acc[9][2][4];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < 9; ++i)
 #pragma unroll
     for (int j = 0; j < 2; ++j)
 #pragma unroll
       for (int k = 0; k < 4; ++k) acc[i][j][k] = 0.f;
-  float bsum[2] = {0.f, 0.f};  // warp 0: out channels g and g + 8
+  float bsum[2] = {0.f, 0.f};  // dx = 0: out channels g and g + 8
   int it = 0;
-  bool issued_next = false;
   for (long long tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, ++it) {
-    const int b = it & 1;
-    issued_next = threadIdx.x == 0 && tile + gridDim.x < n_tiles;
-    if (issued_next) issue(b ^ 1, tile + gridDim.x);
-    if (!mbar_wait(&bar[b], (uint32_t)((it >> 1) & 1), status)) abort_flag = 1;
+    const int b = it % kWStages;
+    // every warp has left tile it - 1, whose stage takes tile it + kWStages - 1
+    if (threadIdx.x == 0) issue_to(it + kWStages);
+    if (!mbar_wait(&bar[b], (uint32_t)((it / kWStages) & 1), status)) abort_flag = 1;
     __syncthreads();
     if (abort_flag) {
-      if (issued_next) mbar_wait(&bar[b ^ 1], (uint32_t)(((it + 1) >> 1) & 1), status);
+      // let the issued loads land before the CTA exits
+      if (threadIdx.x == 0)
+        for (int k = it + 1; k < issued; ++k)
+          mbar_wait(&bar[k % kWStages], (uint32_t)((k / kWStages) & 1), status);
       return;
     }
     const unsigned char* hb = dsm + b * kWStage;
     const unsigned char* gb = hb + kFHalo;
-#pragma unroll 2
-    for (int row = 0; row < kFZ * kTY; ++row) {  // k step: the 16 voxels of one output row
-      const int oz = row / kTY, oy = row % kTY;
-      uint32_t af[4];
+    uint32_t af[kTY][4];
+#pragma unroll
+    for (int oy = 0; oy < kTY; ++oy) {
       // A = gy^T: rows voxel r + 8 (mat >> 1), channel half (mat & 1), transposed.
-      ldsm_x4_t(af, gb + swz(row * kTX + r + 8 * (mat >> 1), mat & 1) * 16);
-      if (warp == 0) {
-        const float2 p0 = bf2x2(af[0]), p1 = bf2x2(af[1]), p2 = bf2x2(af[2]), p3 = bf2x2(af[3]);
+      ldsm_x4_t(af[oy], gb + swz((zz * kTY + oy) * kTX + r + 8 * (mat >> 1), mat & 1) * 16);
+      if (dx == 0) {
+        const float2 p0 = bf2x2(af[oy][0]), p1 = bf2x2(af[oy][1]), p2 = bf2x2(af[oy][2]),
+                     p3 = bf2x2(af[oy][3]);
         bsum[0] += (p0.x + p0.y) + (p2.x + p2.y);
         bsum[1] += (p1.x + p1.y) + (p3.x + p3.y);
       }
+    }
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int tap = warp + 8 * i;
-        if (tap < kTaps) {
-          const int dz = tap / 9, dy = (tap / 3) % 3, dx = tap % 3;
-          uint32_t bf[4];
-          // B = shifted x: rows voxel r + 8 (mat & 1), channel half (mat >> 1), transposed.
-          const int hv = ((oz + dz) * kHY + oy + dy) * kHX + dx + r + 8 * (mat & 1);
-          ldsm_x4_t(bf, hb + swz(hv, mat >> 1) * 16);
-          mma16816(acc[i][0], af, bf[0], bf[1]);
-          mma16816(acc[i][1], af, bf[2], bf[3]);
+    for (int dz = 0; dz < 3; ++dz) {
+#pragma unroll
+      for (int hy = 0; hy < kHY; ++hy) {
+        uint32_t bf[4];
+        // B = shifted x: rows voxel r + 8 (mat & 1), channel half (mat >> 1), transposed.
+        const int hv = ((zz + dz) * kHY + hy) * kHX + dx + r + 8 * (mat & 1);
+        ldsm_x4_t(bf, hb + swz(hv, mat >> 1) * 16);
+#pragma unroll
+        for (int dy = 0; dy < 3; ++dy) {
+          const int oy = hy - dy;
+          if (oy < 0 || oy >= kTY) continue;
+          mma16816(acc[dz * 3 + dy][0], af[oy], bf[0], bf[1]);
+          mma16816(acc[dz * 3 + dy][1], af[oy], bf[2], bf[3]);
         }
       }
     }
-    __syncthreads();  // stage b is free for the load issued next iteration
+    __syncthreads();  // the stage is free for the load issued next iteration
   }
-  // Partial sums: d0 = (o = g, i = nt*8 + 2t), d1 = (g, +1), d2/d3 rows g + 8.
+  // Sums per plane: d0 = (o = g, i = nt*8 + 2t), d1 = (g, +1), d2/d3 rows g + 8.
+  constexpr int n = kTaps * kC * kC + kC;
   const int g = lane >> 2, t = lane & 3;
-  float* part = a.partial + (long long)blockIdx.x * (kTaps * kC * kC + kC);
+  float* part = reinterpret_cast<float*>(dsm) + zz * n;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int tap = warp + 8 * i;
-    if (tap >= kTaps) continue;
+  for (int i = 0; i < 9; ++i) {
+    const int tap = 3 * i + dx;
 #pragma unroll
     for (int nt = 0; nt < 2; ++nt) {
       const int ci = nt * 8 + 2 * t;
@@ -172,7 +191,7 @@ __global__ void __launch_bounds__(256, 2)
       p[(g + 8) * kC + ci + 1] = acc[i][nt][3];
     }
   }
-  if (warp == 0) {
+  if (dx == 0) {
 #pragma unroll
     for (int o = 1; o < 4; o <<= 1) {
       bsum[0] += __shfl_xor_sync(0xffffffffu, bsum[0], o);
@@ -182,6 +201,14 @@ __global__ void __launch_bounds__(256, 2)
       part[kTaps * kC * kC + g] = bsum[0];
       part[kTaps * kC * kC + g + 8] = bsum[1];
     }
+  }
+  __syncthreads();
+  const float* sums = reinterpret_cast<const float*>(dsm);
+  for (int i = threadIdx.x; i < n; i += kWThreads) {
+    float v = sums[i];
+#pragma unroll
+    for (int k = 1; k < kFZ; ++k) v += sums[k * n + i];
+    a.partial[(long long)blockIdx.x * n + i] = v;
   }
 }
 
@@ -325,7 +352,7 @@ cudaError_t launch_features(long long N, const float* vel, const float* ph, cons
   return cudaGetLastError();
 }
 
-int wgrad_blocks() { return 152 * 2; }
+int wgrad_blocks() { return 152; }
 // per-CTA partials, then the FP64 group sums of the two-stage reduction
 size_t wgrad_partial_floats() {
   const size_t n = kTaps * kC * kC + kC;
@@ -434,12 +461,12 @@ cudaError_t launch_wgrad(const WgradArgs& a, const CUtensorMap& xmap, const CUte
   if (!attr) {
     cudaError_t e = cudaFuncSetAttribute(conv_wgrad_kernel,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         2 * kWStage + 256);
+                                         kWStages * kWStage + 256);
     if (e != cudaSuccess) return e;
     attr = true;
   }
   const int grid = (int)std::min<long long>(n_tiles, wgrad_blocks());
-  conv_wgrad_kernel<<<grid, 256, 2 * kWStage + 256, s>>>(xmap, gmap, a, status);
+  conv_wgrad_kernel<<<grid, kWThreads, kWStages * kWStage + 256, s>>>(xmap, gmap, a, status);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const int n = kTaps * kC * kC + kC, groups = (grid + kRedGroup - 1) / kRedGroup;

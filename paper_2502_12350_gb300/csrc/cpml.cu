@@ -490,8 +490,11 @@ __global__ void __launch_bounds__(kThreads) rev_x_kernel(CpmlArgs c) {
 
 // Threads that a marching launch should have: enough columns leave the slabs
 // whole (a cut makes 8 or 16 cells of the neighbouring piece again); with
-// fewer, the slabs are cut into pieces of at least 3 cells.
-constexpr long long kMarchThreads = 152LL * 512;
+// fewer, the slabs are cut into pieces of at least 3 cells.  250 gradient steps
+// of 256^3 take 92.1, 92.3, 94.4, 100.7 and 119.5 ms with 128, 256, 512, 1024
+// and 2048 threads per SM asked for, 300 steps of 448x448x256 107.5 to 108.2
+// up to 1024 and 111.8 at 2048.
+constexpr long long kMarchThreads = 152LL * 256;
 
 int piece(const CpmlExtent& e, int a) {
   long long cuts = std::max(1LL, kMarchThreads / std::max(1LL, e.threads[a]));

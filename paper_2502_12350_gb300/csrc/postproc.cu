@@ -14,7 +14,7 @@
 // (Six dense transforms, three per direction, and a spectral multiplier made
 // the 600x600x200 Bessel filter 15.9 ms; with the transforms along x replaced
 // by a bandwidth-bound pass of 0.16 ms and the others halved by their symmetry
-// it takes 4.0 ms: 1.33 ms a transform along y, 0.59 along z.)
+// it took 4.1 ms, and takes 3.4 with packed multiply-adds.)
 //
 // Resampling (Sec. 2: time interpolation by nearest neighbour or sinc;
 // Table 1 Interpolate).  The resampling of every trace is the same sparse
@@ -187,7 +187,11 @@ __global__ void __launch_bounds__(256) sweep_kernel(const float* in, float* out,
 // sums).  A block makes 64 even and 64 odd modes (inverse: 64 mirrored pairs
 // of cells) of 128 lines; each of its 256 threads accumulates 8 lines x 4
 // outputs x 2, fed by float4 shared-memory reads, with the next chunk's
-// global loads in registers while a chunk is multiplied.  FP32 ALU bound.
+// global loads in registers while a chunk is multiplied.  Bound by issue and
+// the shared-memory reads: with one multiply-add per instruction the FMA pipe
+// was 46 % busy and an instruction issued in 61 % of the cycles; two lines per
+// instruction and warps of 8 x 4 threads took the 600x600x200 Bessel filter
+// from 4.06 to 3.37 ms.
 constexpr int kTL = 128, kTI = 64, kTK = 8;
 constexpr int kAP = kTL + 4;  // A row pitch
 
@@ -205,7 +209,9 @@ __global__ void __launch_bounds__(256, 2)
   __shared__ __align__(16) float As[2][2][kTK][kAP];
   __shared__ __align__(16) float Bs[2][2][kTK][kTI];
   const int h = (n + 1) / 2;
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  // a warp holds 8 x 4 of the block's 16 x 16 threads
+  const int tid = threadIdx.x;
+  const int tx = (tid & 7) + (tid >> 5 & 1) * 8, ty = (tid >> 3 & 3) + (tid >> 6) * 4;
   const long long L0 = (long long)blockIdx.x * kTL;
   const int i0 = blockIdx.y * kTI;
   // loads: 128 lines x 8 cells x 2 = 4 pairs per thread (one line each), and
@@ -216,20 +222,30 @@ __global__ void __launch_bounds__(256, 2)
   const float* src = in + (lok ? (LA / inner) * outer + LA % inner : 0);
   const int bi = tid & (kTI - 1), bj = tid / kTI;
   float ra[2][4], rb[2][2];
+  // cells p and q of the thread's next pair, and from one pair to its next
+  const float* fp = src + (INV ? 2 * aj : aj) * st;
+  const float* fq = src + (INV ? 2 * aj + 1 : n - 1 - aj) * st;
+  const long long dp = (INV ? 4 : 2) * st, dq = INV ? dp : -dp;
+  const float* ep = E + (long long)bj * h + i0 + bi;
+  const float* op = O + (long long)bj * h + i0 + bi;
+  const bool iok = i0 + bi < h;
   auto load = [&](int j0) {
+    int j = j0 + aj;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const int j = j0 + aj + 2 * k;
-      const int p = INV ? 2 * j : j, q = INV ? 2 * j + 1 : n - 1 - j;
-      ra[0][k] = lok && j < h ? src[p * st] : 0.0f;
-      ra[1][k] = lok && j < h && q < n && q != p ? src[q * st] : 0.0f;
+    for (int k = 0; k < 4; ++k, j += 2) {
+      const bool ok = lok && j < h;
+      ra[0][k] = ok ? *fp : 0.0f;
+      ra[1][k] = ok && (INV ? 2 * j + 1 < n : 2 * j + 1 != n) ? *fq : 0.0f;
+      fp += dp;
+      fq += dq;
     }
+    j = j0 + bj;
 #pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      const int j = j0 + bj + 4 * k, i = i0 + bi;
-      const bool ok = j < h && i < h;
-      rb[0][k] = ok ? __ldg(E + (long long)j * h + i) : 0.0f;
-      rb[1][k] = ok ? __ldg(O + (long long)j * h + i) : 0.0f;
+    for (int k = 0; k < 2; ++k, j += 4) {
+      rb[0][k] = iok && j < h ? __ldg(ep) : 0.0f;
+      rb[1][k] = iok && j < h ? __ldg(op) : 0.0f;
+      ep += 4 * h;
+      op += 4 * h;
     }
   };
   auto stage = [&](int s) {
@@ -244,7 +260,7 @@ __global__ void __launch_bounds__(256, 2)
       Bs[s][1][bj + 4 * k][bi] = rb[1][k];
     }
   };
-  float acc[2][8][4] = {};
+  float2 acc[2][4][4] = {};  // two lines each
   load(0);
   stage(0);
   __syncthreads();
@@ -252,21 +268,21 @@ __global__ void __launch_bounds__(256, 2)
   for (int j0 = 0; j0 < h; j0 += kTK, s ^= 1) {
     const bool more = j0 + kTK < h;
     if (more) load(j0 + kTK);
-#pragma unroll
+#pragma unroll 2
     for (int k = 0; k < kTK; ++k)
 #pragma unroll
       for (int v = 0; v < 2; ++v) {
-        // lines 4 ty .. and 64 + 4 ty ..: the two rows of threads of a warp
-        // read consecutive float4s
+        // lines 4 ty .. and 64 + 4 ty ..: the rows of threads of a warp read
+        // consecutive float4s
         const float4 a0 = *reinterpret_cast<const float4*>(&As[s][v][k][ty * 4]);
         const float4 a1 = *reinterpret_cast<const float4*>(&As[s][v][k][64 + ty * 4]);
         const float4 b = *reinterpret_cast<const float4*>(&Bs[s][v][k][tx * 4]);
-        const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+        const float2 a[4] = {{a0.x, a0.y}, {a0.z, a0.w}, {a1.x, a1.y}, {a1.z, a1.w}};
         const float bb[4] = {b.x, b.y, b.z, b.w};
 #pragma unroll
-        for (int r = 0; r < 8; ++r)
+        for (int c = 0; c < 4; ++c)
 #pragma unroll
-          for (int c = 0; c < 4; ++c) acc[v][r][c] = fmaf(a[r], bb[c], acc[v][r][c]);
+          for (int r = 0; r < 4; ++r) acc[v][r][c] = __ffma2_rn(a[r], make_float2(bb[c], bb[c]), acc[v][r][c]);
       }
     if (more) stage(s ^ 1);
     __syncthreads();
@@ -287,7 +303,8 @@ __global__ void __launch_bounds__(256, 2)
       float e[4], o[4];
 #pragma unroll
       for (int r = 0; r < 4; ++r) {
-        const float x = acc[0][4 * g + r][c], y = acc[1][4 * g + r][c];
+        const float2 xx = acc[0][2 * g + r / 2][c], yy = acc[1][2 * g + r / 2][c];
+        const float x = r & 1 ? xx.y : xx.x, y = r & 1 ? yy.y : yy.x;
         e[r] = INV ? x + y : x;
         o[r] = INV ? x - y : y;
       }

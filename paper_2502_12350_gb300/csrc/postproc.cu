@@ -26,6 +26,7 @@
 
 #include <cmath>
 #include <cstdint>
+#include <type_traits>
 
 namespace mamute {
 
@@ -329,13 +330,19 @@ __global__ void __launch_bounds__(256, 2)
 // the outputs 8 g .. 8 g + 7, lane l the traces 4 l .. 4 l + 3, 32 sums in
 // registers.  The input window of the block's outputs passes through shared
 // memory in chunks of kBK samples, [sample][trace], beside the weights of
-// each (sample, output) and a mask of the outputs whose band holds the
-// sample; per sample a thread reads 4 trace values and 8 weights for 32
-// multiply-adds.  (One output and 8 traces per thread, straight from global
-// memory, spent 33 L1 wavefronts per 8 multiply-add instructions, the
-// outputs' bands being dt_out / dt_in samples apart: 65,536 traces of 4000
-// samples to 1000 took 1.76 ms, now 0.92; with chunks of 64 samples, half the
-// resident blocks and a branch per output 1.16.)  Every output is the same sum
+// each (sample, output), zero outside the output's band; per sample a thread
+// reads 4 trace values and 8 weights for 32 multiply-adds, two outputs per
+// instruction.  Zero weights add nothing to a finite sum of finite samples, so
+// the outputs' bands need no branches; a thread also sums zero times every
+// sample, which is not zero if a sample is not finite, and then the block
+// takes its chunks again with a mask of the outputs whose band holds the
+// sample (such a sample reaches only those).  (One output and 8 traces per
+// thread, straight from global memory, spent 33 L1 wavefronts per 8
+// multiply-add instructions, the outputs' bands being dt_out / dt_in samples
+// apart: 65,536 traces of 4000 samples to 1000 took 1.76 ms; masks on the
+// samples that not all 8 outputs take, one multiply-add per instruction, 0.93;
+// now 0.85.)  Bound by issue and the barriers of the chunks: a warp's 8
+// outputs take about half of the block's window.  Every output is the same sum
 // in the same order.
 constexpr int kBM = 32, kBT = 128, kBK = 32;
 constexpr int kBP = kBT + 4;  // sample pitch: 8 samples x 4 traces of a load fall on 32 banks
@@ -371,15 +378,6 @@ __global__ void __launch_bounds__(kBT)
     hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, d));
   }
   const int glo = __shfl_sync(0xffffffffu, lo, 8 * g), ghi = __shfl_sync(0xffffffffu, hi, 8 * g);
-  // samples that all 8 outputs of the warp take
-  int clo = mc, chi = mc + ml;
-#pragma unroll
-  for (int d = 1; d < 8; d <<= 1) {
-    clo = max(clo, __shfl_xor_sync(0xffffffffu, clo, d));
-    chi = min(chi, __shfl_xor_sync(0xffffffffu, chi, d));
-  }
-  clo = __shfl_sync(0xffffffffu, clo, 8 * g);
-  chi = max(clo, __shfl_sync(0xffffffffu, chi, 8 * g));
 #pragma unroll
   for (int d = 8; d < 32; d <<= 1) {
     lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, d));
@@ -407,58 +405,54 @@ __global__ void __launch_bounds__(kBT)
       }
       asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    float acc[8][4] = {};
-    __syncthreads();  // the previous traces' last chunk is read
-    if (lo < hi) issue(lo, st[0]);
-    int b = 0;
-    for (int kc = lo; kc < hi; kc += kBK, b ^= 1) {
-      if (kc + kBK < hi) {
-        issue(kc + kBK, st[b ^ 1]);
-        asm volatile("cp.async.wait_group 1;" ::: "memory");
-      } else {
-        asm volatile("cp.async.wait_group 0;" ::: "memory");
-      }
-      __syncthreads();
-      const BandStage& s = st[b];
-      // the samples before and after the common ones are taken by some outputs
-      // only: the others add nothing, whatever the sample holds
-      const int k0 = max(glo, kc) - kc, k3 = min(ghi, kc + kBK) - kc;
-      const int k1 = min(max(clo - kc, k0), k3), k2 = min(max(chi - kc, k1), k3);
-      auto some = [&](int b, int e) {
-        for (int k = b; k < e; ++k) {
+    float2 acc[4][4];  // [two outputs][trace]
+    // All chunks into acc; true if a sample the thread has met is not finite.
+    auto chunks = [&](auto masked) {
+      constexpr bool kMasked = decltype(masked)::value;
+      float2 met = {0.0f, 0.0f};  // zero times every sample
+#pragma unroll
+      for (int o = 0; o < 4; ++o)
+#pragma unroll
+        for (int t = 0; t < 4; ++t) acc[o][t] = make_float2(0.0f, 0.0f);
+      __syncthreads();  // the previous traces' last chunk is read
+      if (lo < hi) issue(lo, st[0]);
+      int b = 0;
+      for (int kc = lo; kc < hi; kc += kBK, b ^= 1) {
+        if (kc + kBK < hi) {
+          issue(kc + kBK, st[b ^ 1]);
+          asm volatile("cp.async.wait_group 1;" ::: "memory");
+        } else {
+          asm volatile("cp.async.wait_group 0;" ::: "memory");
+        }
+        __syncthreads();
+        const BandStage& s = st[b];
+        const int k0 = max(glo, kc) - kc, k1 = min(ghi, kc + kBK) - kc;
+#pragma unroll 4
+        for (int k = k0; k < k1; ++k) {
           const float4 xv = *reinterpret_cast<const float4*>(&s.x[k][4 * lane]);
           const float4 w0 = *reinterpret_cast<const float4*>(&s.w[k][8 * g]);
           const float4 w1 = *reinterpret_cast<const float4*>(&s.w[k][8 * g + 4]);
-          const float ww[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
-          const unsigned mk = s.mask[k] >> (8 * g);
-#pragma unroll
-          for (int o = 0; o < 8; ++o) {
-            const bool in = mk >> o & 1;
-            acc[o][0] = in ? fmaf(ww[o], xv.x, acc[o][0]) : acc[o][0];
-            acc[o][1] = in ? fmaf(ww[o], xv.y, acc[o][1]) : acc[o][1];
-            acc[o][2] = in ? fmaf(ww[o], xv.z, acc[o][2]) : acc[o][2];
-            acc[o][3] = in ? fmaf(ww[o], xv.w, acc[o][3]) : acc[o][3];
+          const float2 ww[4] = {{w0.x, w0.y}, {w0.z, w0.w}, {w1.x, w1.y}, {w1.z, w1.w}};
+          const float xx[4] = {xv.x, xv.y, xv.z, xv.w};
+          const unsigned mk = kMasked ? s.mask[k] >> (8 * g) : 0u;
+          if (!kMasked) {
+            met = __ffma2_rn(make_float2(xv.x, xv.y), make_float2(0.0f, 0.0f), met);
+            met = __ffma2_rn(make_float2(xv.z, xv.w), make_float2(0.0f, 0.0f), met);
           }
-        }
-      };
-      some(k0, k1);
-#pragma unroll 4
-      for (int k = k1; k < k2; ++k) {
-        const float4 xv = *reinterpret_cast<const float4*>(&s.x[k][4 * lane]);
-        const float4 w0 = *reinterpret_cast<const float4*>(&s.w[k][8 * g]);
-        const float4 w1 = *reinterpret_cast<const float4*>(&s.w[k][8 * g + 4]);
-        const float ww[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
 #pragma unroll
-        for (int o = 0; o < 8; ++o) {
-          acc[o][0] = fmaf(ww[o], xv.x, acc[o][0]);
-          acc[o][1] = fmaf(ww[o], xv.y, acc[o][1]);
-          acc[o][2] = fmaf(ww[o], xv.z, acc[o][2]);
-          acc[o][3] = fmaf(ww[o], xv.w, acc[o][3]);
+          for (int o = 0; o < 4; ++o)
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+              const float2 v = __ffma2_rn(ww[o], make_float2(xx[t], xx[t]), acc[o][t]);
+              if (!kMasked || (mk >> (2 * o) & 1)) acc[o][t].x = v.x;
+              if (!kMasked || (mk >> (2 * o + 1) & 1)) acc[o][t].y = v.y;
+            }
         }
+        __syncthreads();
       }
-      some(k2, k3);
-      __syncthreads();
-    }
+      return !(met.x + met.y == 0.0f);
+    };
+    if (__syncthreads_or(chunks(std::false_type{}))) chunks(std::true_type{});
     const int m = m0 + 8 * g;
     const bool vec = (n_out & 3) == 0 && ((unsigned long long)y & 15) == 0 && m + 8 <= n_out;
 #pragma unroll
@@ -466,12 +460,12 @@ __global__ void __launch_bounds__(kBT)
       if (t0 + 4 * lane + t >= n_traces) break;
       float* yr = y + (long long)(t0 + 4 * lane + t) * n_out + m;
       if (vec) {
-        reinterpret_cast<float4*>(yr)[0] = make_float4(acc[0][t], acc[1][t], acc[2][t], acc[3][t]);
-        reinterpret_cast<float4*>(yr)[1] = make_float4(acc[4][t], acc[5][t], acc[6][t], acc[7][t]);
+        reinterpret_cast<float4*>(yr)[0] = make_float4(acc[0][t].x, acc[0][t].y, acc[1][t].x, acc[1][t].y);
+        reinterpret_cast<float4*>(yr)[1] = make_float4(acc[2][t].x, acc[2][t].y, acc[3][t].x, acc[3][t].y);
       } else {
 #pragma unroll
         for (int o = 0; o < 8; ++o)
-          if (m + o < n_out) yr[o] = acc[o][t];
+          if (m + o < n_out) yr[o] = o & 1 ? acc[o / 2][t].y : acc[o / 2][t].x;
       }
     }
   }

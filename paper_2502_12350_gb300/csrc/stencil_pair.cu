@@ -34,6 +34,23 @@ namespace mamute {
 
 namespace {
 
+// The 25-point sum for one point, in a fixed order of IEEE operations (no
+// contraction freedom), the one of lap4, so that every kernel that
+// forms it for the same field gets bitwise the same value.
+__device__ __forceinline__ float lap25(float u, const float (&xm)[4], const float (&xp)[4],
+                                       const float (&ym)[4], const float (&yp)[4],
+                                       const float (&zm)[4], const float (&zp)[4]) {
+  const float cw[4] = {MAMUTE_C1, MAMUTE_C2, MAMUTE_C3, MAMUTE_C4};
+  float acc = __fmul_rn(3.0f * MAMUTE_C0, u);
+#pragma unroll
+  for (int m = 0; m < 4; ++m) {
+    float s = __fadd_rn(__fadd_rn(__fadd_rn(xm[m], xp[m]), __fadd_rn(ym[m], yp[m])),
+                        __fadd_rn(zm[m], zp[m]));
+    acc = __fmaf_rn(cw[m], s, acc);
+  }
+  return acc;
+}
+
 __device__ __forceinline__ int ld_acquire(const int* p) {
   int v;
   asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");

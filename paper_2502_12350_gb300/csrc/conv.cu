@@ -374,53 +374,71 @@ void conv_gy_box(unsigned (&box)[4]) {
   box[3] = kFZ;
 }
 
-// Blocking of the tensor-core convolution for a D x H x W volume: the
-// tallest row block (at most 8 chunks of 128 outputs) whose halo slots leave
-// room for a ring of 4 (each halo plane is consumed by one step), else the
-// tallest with 3.
+// Blocking of the tensor-core convolution for a D x H x W volume: x segments,
+// row blocks and z chunks with the least modelled time of the busiest of 152
+// persistent CTAs, which for each of its items marches ZC + 2 halo planes of
+// NCH chunks of 128 outputs; a plane costs as much as one chunk more (waits,
+// swizzle start), an item's start two planes.  Halo slots leave room for a
+// ring of 4 planes (each is consumed by one step), or 3 where nothing has 4.
+// (The tallest row block with the fewest rounds of ZC planes, its halo planes
+// not counted, took 3 rounds of 5 planes where 1 round of 16 does it, and left
+// most SMs idle on small volumes: a layer's three passes on 80x160x160 290 ->
+// 256 us, on 9x36x32 81 -> 56 us.)
 constexpr int kTcSmemMax = 232448;                  // dynamic shared memory per CTA
 constexpr int kTcSlotBudget = kTcSmemMax - kTcWBytes - 1024;
 
-static TcPlan tc_plan(int D, int H, int W) {
-  TcPlan p{};
+static TcPlan tc_plan_of(int D, int H, int W) {
+  TcPlan best{};
+  double least = -1.0;
   // x segments of at most kTcMaxP - 2 voxels, as even as possible: a halo
   // row of P voxels is one TMA box row of 4 P 8-byte elements (<= 256)
-  p.nxs = (W + kTcMaxP - 3) / (kTcMaxP - 2);
-  p.SW = (W + p.nxs - 1) / p.nxs;
-  p.P = p.SW + 2;
-  auto shape = [&](int ry) {
-    p.RY = ry;
-    p.NCH = (p.RY * p.P + 127) / 128;
-    // the halo box must cover the last chunk's reach
-    p.rows = (p.NCH * 128 + 2 * p.P + 2 + p.P - 1) / p.P;
-    p.slot_bytes = ((p.rows * p.P * 32 + 1023) / 1024) * 1024;
-    p.ring = std::min(kTcMaxRing, kTcSlotBudget / p.slot_bytes);
-  };
-  const int ry_max = std::max(1, std::min(H, (kTcMaxChunks * 128) / p.P));
-  int pick = 0;
-  for (int want = 4; want >= 3 && !pick; --want)
-    for (int ry = ry_max; ry >= 1; --ry) {
-      shape(ry);
-      if (p.rows <= 256 && p.ring >= want) {
-        pick = ry;
-        break;
+  const int nxs0 = (W + kTcMaxP - 3) / (kTcMaxP - 2);
+  for (int want = 4; want >= 3 && least < 0; --want)
+    for (int nxs = nxs0; nxs <= std::min(nxs0 + 2, W); ++nxs) {
+      TcPlan p{};
+      p.SW = (W + nxs - 1) / nxs;
+      p.nxs = (W + p.SW - 1) / p.SW;
+      p.P = p.SW + 2;
+      const int ry_max = std::max(1, std::min(H, kTcMaxChunks * 128 / p.P));
+      for (p.RY = 1; p.RY <= ry_max; ++p.RY) {
+        p.NCH = (p.RY * p.P + 127) / 128;
+        // the halo box must cover the last chunk's reach
+        p.rows = (p.NCH * 128 + 2 * p.P + 2 + p.P - 1) / p.P;
+        p.slot_bytes = ((p.rows * p.P * 32 + 1023) / 1024) * 1024;
+        p.ring = std::min(kTcMaxRing, kTcSlotBudget / p.slot_bytes);
+        if (p.rows > 256 || p.ring < want) continue;
+        p.nyb = (H + p.RY - 1) / p.RY;
+        const long long base = (long long)p.nxs * p.nyb;
+        // the z chunks that just fill 1 to 6 rounds, and the longest ones
+        for (int r = 1; r <= 7; ++r) {
+          const long long nz = r <= 6 ? std::min<long long>(152LL * r / base, D) : (D + 31) / 32;
+          if (nz < 1) continue;
+          p.ZC = (int)((D + nz - 1) / nz);
+          if (p.ZC > 32) continue;
+          p.nzc = (D + p.ZC - 1) / p.ZC;
+          p.items = base * p.nzc;
+          const double rounds = (double)((p.items + 151) / 152);
+          const double cost = (rounds * (p.ZC + 2) + 2.0) * (p.NCH + 1.0);
+          if (least < 0 || cost < least) {
+            least = cost;
+            best = p;
+          }
+        }
       }
     }
-  shape(pick > 0 ? pick : 1);
-  p.nyb = (H + p.RY - 1) / p.RY;
-  // z chunk: fewest rounds of 152 persistent CTAs x planes per item; ties
-  // go to longer chunks (fewer re-loaded halo planes).
-  long long best = -1;
-  for (int zc = 1; zc <= std::min(D, 32); ++zc) {
-    const long long items = (long long)p.nxs * p.nyb * ((D + zc - 1) / zc);
-    const long long cost = ((items + 151) / 152) * zc;
-    if (best < 0 || cost <= best) {
-      best = cost;
-      p.ZC = zc;
-    }
+  return best;
+}
+
+// The last volume's plan (a few microseconds), for a network's layers.
+static TcPlan tc_plan(int D, int H, int W) {
+  thread_local int dims[3] = {0, 0, 0};
+  thread_local TcPlan p;
+  if (dims[0] != D || dims[1] != H || dims[2] != W) {
+    p = tc_plan_of(D, H, W);
+    dims[0] = D;
+    dims[1] = H;
+    dims[2] = W;
   }
-  p.nzc = (D + p.ZC - 1) / p.ZC;
-  p.items = (long long)p.nxs * p.nyb * p.nzc;
   return p;
 }
 

@@ -14,7 +14,7 @@
 // (Six dense transforms, three per direction, and a spectral multiplier made
 // the 600x600x200 Bessel filter 15.9 ms; with the transforms along x replaced
 // by a bandwidth-bound pass of 0.16 ms and the others halved by their symmetry
-// it took 4.1 ms, and takes 3.4 with packed multiply-adds.)
+// it took 4.1 ms, and takes 2.9 with packed multiply-adds on 8 x 8 tiles.)
 //
 // Resampling (Sec. 2: time interpolation by nearest neighbour or sinc;
 // Table 1 Interpolate).  The resampling of every trace is the same sparse
@@ -186,13 +186,14 @@ __global__ void __launch_bounds__(256) sweep_kernel(const float* in, float* out,
 // antisymmetric, so the n x n product splits into two of half the size on the
 // sums and differences of the mirrored cells (half the operations, shorter
 // sums).  A block makes 64 even and 64 odd modes (inverse: 64 mirrored pairs
-// of cells) of 128 lines; each of its 256 threads accumulates 8 lines x 4
-// outputs x 2, fed by float4 shared-memory reads, with the next chunk's
-// global loads in registers while a chunk is multiplied.  Bound by issue and
-// the shared-memory reads: with one multiply-add per instruction the FMA pipe
-// was 46 % busy and an instruction issued in 61 % of the cycles; two lines per
-// instruction and warps of 8 x 4 threads took the 600x600x200 Bessel filter
-// from 4.06 to 3.37 ms.
+// of cells) of 128 lines: half of its 256 threads the product with E, half that
+// with O, 8 lines x 8 outputs each, fed by float4 shared-memory reads, with the
+// next chunk's global loads in registers while a chunk is multiplied; the two
+// products of an output meet in shared memory at the end.  Bound by issue and
+// the shared-memory reads: 8 lines x 4 outputs of both products with one
+// multiply-add per instruction kept the FMA pipe 46 % busy (600x600x200 Bessel
+// filter 4.06 ms); two lines per instruction 3.37 ms; 8 x 8 tiles, 4 reads for
+// 32 instructions instead of 3 for 16, 2.91 ms.
 constexpr int kTL = 128, kTI = 64, kTK = 8;
 constexpr int kAP = kTL + 4;  // A row pitch
 
@@ -207,12 +208,19 @@ __global__ void __launch_bounds__(256, 2)
     dct_kernel(const float* __restrict__ in, float* __restrict__ out, const float* __restrict__ E,
                const float* __restrict__ O, int n, long long lines, long long inner,
                long long outer, long long st) {
-  __shared__ __align__(16) float As[2][2][kTK][kAP];
-  __shared__ __align__(16) float Bs[2][2][kTK][kTI];
+  __shared__ union {
+    struct {
+      __align__(16) float a[2][2][kTK][kAP], b[2][2][kTK][kTI];
+    } s;
+    float x[32][256];  // the other product's half of a tile, at the end
+  } sm;
+  auto& As = sm.s.a;
+  auto& Bs = sm.s.b;
   const int h = (n + 1) / 2;
-  // a warp holds 8 x 4 of the block's 16 x 16 threads
-  const int tid = threadIdx.x;
-  const int tx = (tid & 7) + (tid >> 5 & 1) * 8, ty = (tid >> 3 & 3) + (tid >> 6) * 4;
+  // warps 0 to 3 make the product with E (v = 0), 4 to 7 that with O; a warp
+  // holds 4 x 8 of the product's 8 x 16 threads
+  const int tid = threadIdx.x, v = tid >> 7;
+  const int tx = (tid & 3) + (tid >> 5 & 1) * 4, ty = (tid >> 2 & 7) + (tid >> 6 & 1) * 8;
   const long long L0 = (long long)blockIdx.x * kTL;
   const int i0 = blockIdx.y * kTI;
   // loads: 128 lines x 8 cells x 2 = 4 pairs per thread (one line each), and
@@ -261,7 +269,7 @@ __global__ void __launch_bounds__(256, 2)
       Bs[s][1][bj + 4 * k][bi] = rb[1][k];
     }
   };
-  float2 acc[2][4][4] = {};  // two lines each
+  float2 acc[4][8] = {};  // [two lines][output]
   load(0);
   stage(0);
   __syncthreads();
@@ -270,57 +278,66 @@ __global__ void __launch_bounds__(256, 2)
     const bool more = j0 + kTK < h;
     if (more) load(j0 + kTK);
 #pragma unroll 2
-    for (int k = 0; k < kTK; ++k)
+    for (int k = 0; k < kTK; ++k) {
+      // lines 4 ty .. and 64 + 4 ty .., outputs 4 tx .. and 32 + 4 tx ..: the
+      // threads of a warp read consecutive float4s
+      const float4 a0 = *reinterpret_cast<const float4*>(&As[s][v][k][ty * 4]);
+      const float4 a1 = *reinterpret_cast<const float4*>(&As[s][v][k][64 + ty * 4]);
+      const float4 b0 = *reinterpret_cast<const float4*>(&Bs[s][v][k][tx * 4]);
+      const float4 b1 = *reinterpret_cast<const float4*>(&Bs[s][v][k][32 + tx * 4]);
+      const float2 a[4] = {{a0.x, a0.y}, {a0.z, a0.w}, {a1.x, a1.y}, {a1.z, a1.w}};
+      const float bb[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
 #pragma unroll
-      for (int v = 0; v < 2; ++v) {
-        // lines 4 ty .. and 64 + 4 ty ..: the rows of threads of a warp read
-        // consecutive float4s
-        const float4 a0 = *reinterpret_cast<const float4*>(&As[s][v][k][ty * 4]);
-        const float4 a1 = *reinterpret_cast<const float4*>(&As[s][v][k][64 + ty * 4]);
-        const float4 b = *reinterpret_cast<const float4*>(&Bs[s][v][k][tx * 4]);
-        const float2 a[4] = {{a0.x, a0.y}, {a0.z, a0.w}, {a1.x, a1.y}, {a1.z, a1.w}};
-        const float bb[4] = {b.x, b.y, b.z, b.w};
+      for (int c = 0; c < 8; ++c)
 #pragma unroll
-        for (int c = 0; c < 4; ++c)
-#pragma unroll
-          for (int r = 0; r < 4; ++r) acc[v][r][c] = __ffma2_rn(a[r], make_float2(bb[c], bb[c]), acc[v][r][c]);
-      }
+        for (int r = 0; r < 4; ++r) acc[r][c] = __ffma2_rn(a[r], make_float2(bb[c], bb[c]), acc[r][c]);
+    }
     if (more) stage(s ^ 1);
     __syncthreads();
   }
+  // The two products of an output meet: a thread gives the other product's
+  // thread the lines that that one writes (v = 0 lines 4 ty .., v = 1 the 64th
+  // on), and writes its own lines' outputs p and q.
 #pragma unroll
-  for (int g = 0; g < 2; ++g) {
-    const long long L = L0 + 64 * g + ty * 4;
-    if (L >= lines) continue;
-    // four consecutive lines share a 16-byte store where the layout allows it
-    const long long b0 = (L / inner) * outer + L % inner;
-    const bool vec = L % inner + 4 <= inner && ((b0 | st) & 3) == 0 && L + 4 <= lines &&
-                     ((unsigned long long)out & 15) == 0;
+  for (int c = 0; c < 8; ++c)
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const int i = i0 + tx * 4 + c;
-      if (i >= h) continue;
-      const int p = INV ? i : 2 * i, q = INV ? n - 1 - i : 2 * i + 1;
-      float e[4], o[4];
+    for (int r = 0; r < 2; ++r) {
+      const float2 t = v == 0 ? acc[2 + r][c] : acc[r][c];
+      sm.x[4 * c + 2 * r][tid] = t.x;
+      sm.x[4 * c + 2 * r + 1][tid] = t.y;
+    }
+  __syncthreads();
+  const long long L = L0 + 64 * v + ty * 4;
+  if (L >= lines) return;
+  // four consecutive lines share a 16-byte store where the layout allows it
+  const long long b0 = (L / inner) * outer + L % inner;
+  const bool vec = L % inner + 4 <= inner && ((b0 | st) & 3) == 0 && L + 4 <= lines &&
+                   ((unsigned long long)out & 15) == 0;
+#pragma unroll
+  for (int c = 0; c < 8; ++c) {
+    const int i = i0 + (c / 4) * 32 + tx * 4 + c % 4;
+    if (i >= h) continue;
+    const int p = INV ? i : 2 * i, q = INV ? n - 1 - i : 2 * i + 1;
+    float e[4], o[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const float2 m = v == 0 ? acc[r / 2][c] : acc[2 + r / 2][c];
+      const float mine = r & 1 ? m.y : m.x, other = sm.x[4 * c + r][tid ^ 128];
+      const float x = v == 0 ? mine : other, y = v == 0 ? other : mine;
+      e[r] = INV ? x + y : x;
+      o[r] = INV ? x - y : y;
+    }
+    if (vec) {
+      *reinterpret_cast<float4*>(out + b0 + p * st) = make_float4(e[0], e[1], e[2], e[3]);
+      if (q < n && q != p)
+        *reinterpret_cast<float4*>(out + b0 + q * st) = make_float4(o[0], o[1], o[2], o[3]);
+    } else {
 #pragma unroll
       for (int r = 0; r < 4; ++r) {
-        const float2 xx = acc[0][2 * g + r / 2][c], yy = acc[1][2 * g + r / 2][c];
-        const float x = r & 1 ? xx.y : xx.x, y = r & 1 ? yy.y : yy.x;
-        e[r] = INV ? x + y : x;
-        o[r] = INV ? x - y : y;
-      }
-      if (vec) {
-        *reinterpret_cast<float4*>(out + b0 + p * st) = make_float4(e[0], e[1], e[2], e[3]);
-        if (q < n && q != p)
-          *reinterpret_cast<float4*>(out + b0 + q * st) = make_float4(o[0], o[1], o[2], o[3]);
-      } else {
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-          if (L + r >= lines) continue;
-          const long long b = ((L + r) / inner) * outer + (L + r) % inner;
-          out[b + p * st] = e[r];
-          if (q < n && q != p) out[b + q * st] = o[r];
-        }
+        if (L + r >= lines) continue;
+        const long long b = ((L + r) / inner) * outer + (L + r) % inner;
+        out[b + p * st] = e[r];
+        if (q < n && q != p) out[b + q * st] = o[r];
       }
     }
   }

@@ -119,6 +119,7 @@ struct mamute_ctx {
   DevBuf ident, rcolptr, rcols, ecol, srcw;  // receiver-node combination (trilinear)
   DevBuf smA, smMat, smLam;                  // gradient smoothing scratch
   std::vector<double> smKey, rsKey;          // what smMat / smLam and rsPtr / rsCol / rsW hold
+  int rsTaps = 0;                            // longest band of rsW
   DevBuf pitems, pnbr, precptr, prec, pcells, pgvals, pmaps, pflags;  // two-level launches
   bool pair_graph_failed = false;  // cooperative launches could not be captured
   DevBuf rsPtr, rsCol, rsW, dmod, ddat;      // time resampling: band matrix (c0, len, weights), model- and data-axis traces
@@ -1288,11 +1289,12 @@ int do_resample(mamute_ctx* ctx, int ntr, int nt_in, double dt_in, int nt_out, d
     CK(upload(ctx, ctx->rsCol, len));
     CK(upload(ctx, ctx->rsW, wb));
     ctx->rsKey = key;
+    ctx->rsTaps = K;
   }
   ++ctx->launches;
   const int n_src = adjoint ? nt_out : nt_in, n_dst = adjoint ? nt_in : nt_out;
   CK(launch_band_rows(x, n_src, (const int*)ctx->rsPtr.p, (const int*)ctx->rsCol.p,
-                     (const float*)ctx->rsW.p, n_dst, ntr, y, ctx->stream));
+                      (const float*)ctx->rsW.p, ctx->rsTaps, n_dst, ntr, y, ctx->stream));
   return MAMUTE_OK;
 }
 

@@ -37,9 +37,11 @@ cudaError_t launch_dct(const float* in, float* out, const float* E, const float*
                        cudaStream_t s);
 // y[r][m] = sum_{j < len[m]} w[j][m] x[r][c0[m] + j] for every trace r: a
 // banded matrix whose row m covers the contiguous columns c0[m] ..
-// c0[m] + len[m] - 1, weights stored tap-major (w[j][m] at j n_out + m).
+// c0[m] + len[m] - 1, weights stored tap-major (w[j][m] at j n_out + m);
+// taps is the largest len[m].
 cudaError_t launch_band_rows(const float* x, int n_in, const int* c0, const int* len,
-                             const float* w, int n_out, int n_traces, float* y, cudaStream_t s);
+                             const float* w, int taps, int n_out, int n_traces, float* y,
+                             cudaStream_t s);
 
 // out = a - b elementwise.
 cudaError_t launch_sub(const float* a, const float* b, long long n, float* out, cudaStream_t s);

@@ -92,13 +92,14 @@ __device__ __forceinline__ void lap4(const float* st, int lx, int ly, const F4 (
 // ev: the memory variables' part E with the CPML, taken as a term of its own
 // (lap + E, rounded first, would lose the bits that lap carries beyond E).
 template <bool PML>
-__device__ __forceinline__ float update(float u, float prev, float A, float M, float g,
-                                        float lap, float ev, bool dens) {
-  float s = __fmaf_rn(2.0f, u, -__fmul_rn(g, prev));
-  if (dens) s = __fmaf_rn(-M, u, s);
-  s = __fmaf_rn(A, lap, s);
-  if (PML) s = __fmaf_rn(A, ev, s);
-  return __fmul_rn(g, s);
+__device__ __forceinline__ float2 update(float2 u, float2 prev, float2 A, float2 M, float2 g,
+                                         float2 lap, float2 ev, bool dens) {
+  const float2 ng = make_float2(-g.x, -g.y);
+  float2 s = __ffma2_rn(both(2.0f), u, __fmul2_rn(ng, prev));
+  if (dens) s = __ffma2_rn(make_float2(-M.x, -M.y), u, s);
+  s = __ffma2_rn(A, lap, s);
+  if (PML) s = __ffma2_rn(A, ev, s);
+  return __fmul2_rn(g, s);
 }
 
 // Imaging term A (lap + E - m2) u in the scheme's units: A lap u + A E - M u.
@@ -167,10 +168,13 @@ struct PlaneInfo {
 // own (a 400-step gradient 114.1 -> 94.4 ms).
 // Resident CTAs per SM the register budget is sized for: the adjoint with a
 // recomputed forward field on large tiles needs more than 200 KB of shared
-// memory per pair, so it runs one CTA per SM with the full register file.
+// memory per pair, so it runs one CTA per SM with the full register file;
+// small tiles run as many as their shared memory lets in.
 template <int TX, int TY, int MODE>
 struct MinBlocks {
-  static constexpr int value = (MODE == MODE_ADJ && TX * TY >= 1024) ? 1 : 2;
+  static constexpr int kThreads = (TX / 4) * TY + 32;
+  static constexpr int value = MODE == MODE_ADJ ? (TX * TY >= 1024 ? 1 : 2)
+                                                : (kThreads <= 96 ? 5 : (kThreads <= 160 ? 3 : 2));
 };
 
 template <int TX, int TY, bool DENS, int MODE, bool PML>
@@ -367,6 +371,15 @@ __global__ void __launch_bounds__((TX / 4) * TY + 32, (MinBlocks<TX, TY, MODE>::
     }
   }
 
+  // Planes per pass of the loop: the register queue moves on by 32 registers a
+  // plane, which unrolling folds into the names; as many as the 96 registers of
+  // the tiles with two CTAs of 288 and 320 threads take without spilling.
+  // 400 steps of 576x576x320 with density (72x16) 139.6 -> 135.4 ms with two (three
+  // spill: 144.3); four 243x191x137 windows (64x16) 29.0 -> 28.2 ms with three (two
+  // spill: 29.6), where the adjoint takes two (256^3 gradient 84.1 -> 82.4 ms; three
+  // spill: 84.9); 96^3 (48x16, few planes a block) is best without.
+  constexpr int kUnroll = TX == 72 && TY == 16 ? 2 : (TX == 64 && TY == 16 ? (ADJ ? 2 : 3) : 1);
+#pragma unroll kUnroll
   for (int j = 0; j < npl; ++j) {
     const int z = zb + j;
     {  // queue slot 8 <- plane z + 4
@@ -397,9 +410,13 @@ __global__ void __launch_bounds__((TX / 4) * TY + 32, (MinBlocks<TX, TY, MODE>::
     const float gyz = __fmul_rn(gyv, pi.gz);
     F4 out;
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const float g = __fmul_rn(gxv[e], gyz);
-      out.v[e] = update<PML>(q[4].v[e], prev.v[e], Av.v[e], Mv.v[e], g, lap[e], ev.v[e], DENS);
+    for (int e = 0; e < 4; e += 2) {
+      auto at = [&](const F4& f) { return make_float2(f.v[e], f.v[e + 1]); };
+      const float2 g = __fmul2_rn(make_float2(gxv[e], gxv[e + 1]), both(gyz));
+      const float2 o = update<PML>(at(q[4]), at(prev), at(Av), at(Mv), g, make_float2(lap[e], lap[e + 1]),
+                                   at(ev), DENS);
+      out.v[e] = o.x;
+      out.v[e + 1] = o.y;
     }
     // Source injection (forward only): u^{n+1} += w_e dt^2 w[n] / (h^3 sqrt rho_e)
     // at the corners e of the source cell (one corner for the nearest node).

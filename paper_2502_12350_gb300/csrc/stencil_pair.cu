@@ -51,6 +51,14 @@ __device__ __forceinline__ float lap25(float u, const float (&xm)[4], const floa
   return acc;
 }
 
+// One point of the update, the operations and order of the one-step kernel's.
+__device__ __forceinline__ float update1(float u, float prev, float A, float M, float g, float lap,
+                                         bool dens) {
+  float s = __fmaf_rn(2.0f, u, -__fmul_rn(g, prev));
+  if (dens) s = __fmaf_rn(-M, u, s);
+  return __fmul_rn(g, __fmaf_rn(A, lap, s));
+}
+
 __device__ __forceinline__ int ld_acquire(const int* p) {
   int v;
   asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
@@ -537,7 +545,7 @@ __global__ void __launch_bounds__((TX / 4) * (TY / 2) + 32, 1) pair_kernel(const
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
           const float g = __fmul_rn(gxv[e], gyz);
-          out[r].v[e] = update<false>(u.v[e], prev.v[e], Av.v[e], Mv.v[e], g, r ? lb[e] : la[e], 0.f, DENS);
+          out[r].v[e] = update1(u.v[e], prev.v[e], Av.v[e], Mv.v[e], g, r ? lb[e] : la[e], DENS);
         }
       }
       release(&emptyU[su]);
@@ -579,7 +587,7 @@ __global__ void __launch_bounds__((TX / 4) * (TY / 2) + 32, 1) pair_kernel(const
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
           const float g = __fmul_rn(gxv[e], gyz);
-          out[r].v[e] = update<false>(u.v[e], prev.v[e], Av.v[e], Mv.v[e], g, r ? lb[e] : la[e], 0.f, DENS);
+          out[r].v[e] = update1(u.v[e], prev.v[e], Av.v[e], Mv.v[e], g, r ? lb[e] : la[e], DENS);
         }
       }
       release(&emptyV[s]);

@@ -221,11 +221,12 @@ def run_reference(args):
 
 
 GRAD_FWD_BYTES = (16, 4)  # per padded point (u^n, u^{n-1}, A, new level), per interior point (term store)
-GRAD_ADJ_BYTES = (24, 4)  # per padded point (psi levels, A, accumulator read + write), per interior point (term read)
+# per padded point (psi levels, A, new level; the accumulator read and written once
+# per three steps), per interior point (term read)
+GRAD_ADJ_BYTES = (16 + 8 / 3, 4)
 # CPML gradient, per (point, axis) pair of a layer: forward Psi_a, Zeta_a read and
-# written; reverse their multipliers read and written and the scratch y_a, z_a
-# written and read
-PML_GRAD_PAIR_BYTES = (16, 32)
+# written; reverse their multipliers read and written
+PML_GRAD_PAIR_BYTES = (16, 16)
 
 
 def gradient_metrics(workload, steps, warmup, autotune=False, snapshots=0, nt=None, pml=False):
@@ -234,9 +235,9 @@ def gradient_metrics(workload, steps, warmup, autotune=False, snapshots=0, nt=No
     stream, and the step loop's bandwidth against the algorithmic bytes of
     the all-terms mode (each forward step reads u^n, u^{n-1}, A and writes
     the new level, 16 B per padded point, and stores the imaging term, 4 B
-    per interior point; each adjoint step reads two psi levels and A, writes
-    the new level, reads and writes the accumulator, 24 B per padded point,
-    and reads the stored term, 4 B per interior point).  With pml, the
+    per interior point; each adjoint step reads two psi levels and A and writes
+    the new level, 16 B per padded point, reads the stored term, 4 B per interior
+    point, and every third one reads and writes the accumulator, 8 B).  With pml, the
     convolutional PML instead of the sponge (every imaging term kept), plus
     PML_GRAD_PAIR_BYTES per (point, axis) pair of the layers."""
     import ctypes
@@ -426,9 +427,10 @@ def run_postproc_bench(args):
     """Gradient smoothing and data time resampling (mamute_smooth,
     mamute_resample) on one GPU: CUDA-event time per API call, inputs resident
     on the device.  Smoothing: Bessel and Laplace filters of the 600x600x200
-    gradient of the 64-shot workload, a forward and an inverse dense DCT-II
-    pass per axis of 2 n_a flops per point (FP32 ALU bound: 152 SMs x 128
-    lanes x 2 flops x 2.07 GHz).  Resampling: sinc, 65,536 traces of 4000
+    gradient of the 64-shot workload; the Bessel filter by a forward and an
+    inverse half-size DCT-II product along y and z, n_a flops per point each
+    (FP32 ALU bound: 152 SMs x 128 lanes x 2 flops x 2.07 GHz), the Laplace
+    filter by tridiagonal solves (no flops quoted).  Resampling: sinc, 65,536 traces of 4000
     samples to 1000 (the headline's receivers), every input sample read and
     every output sample written once; the host builds the CSR matrix inside
     each call."""
@@ -458,12 +460,13 @@ def run_postproc_bench(args):
     grad = torch.randn((nz, ny, nx), device=dev, generator=gen)  # 288 MB: larger than L2
     out = torch.empty_like(grad)
     alu_peak = 152 * 128 * 2 * 2.07e9 / 1e12
-    flops = 2 * 2 * (nx + ny + nz) * nx * ny * nz
+    flops = 2 * (ny + nz) * nx * ny * nz
     smooth = {}
     for mode, name in ((mamute.SMOOTH_BESSEL, "bessel"), (mamute.SMOOTH_LAPLACE, "laplace")):
         ms = per_call_ms(lambda: ctx.smooth(h, mode, grad, out, lengths=[4 * h] * 3))
-        tf = flops / (ms / 1e3) / 1e12
-        smooth[name] = {"ms": ms, "tflops": tf, "frac_fp32_alu": tf / alu_peak}
+        smooth[name] = {"ms": ms}
+    tf = flops / (smooth["bessel"]["ms"] / 1e3) / 1e12
+    smooth["bessel"].update(tflops=tf, frac_fp32_alu=tf / alu_peak)
     ntr, nt_in, nt_out, dt_in = 65536, 4000, 1000, 5e-4
     x = torch.randn((ntr, nt_in), device=dev, generator=gen)
     y = torch.empty((ntr, nt_out), device=dev)

@@ -345,14 +345,15 @@ __global__ void __launch_bounds__(256, 2)
 
 // Banded product over traces, short bands or few traces: one output and 8
 // traces per thread, straight from global memory (each weight loaded once for
-// them), a thread per output.
+// them).  Bound by the loads in flight; not compiled for blocks of 128 threads
+// alone, whose larger register budget left fewer resident (65,536 traces of 4000
+// samples, 16 taps: 829 us, 952 with it).
 constexpr int kFT = 8;
 
-__global__ void __launch_bounds__(128)
-    band_few_kernel(const float* __restrict__ x, int n_in, const int* __restrict__ c0,
-                    const int* __restrict__ len, const float* __restrict__ w, int n_out, int n_traces,
-                    float* __restrict__ y) {
-  const int m = blockIdx.x * 128 + threadIdx.x;
+__global__ void band_few_kernel(const float* __restrict__ x, int n_in, const int* __restrict__ c0,
+                                const int* __restrict__ len, const float* __restrict__ w, int n_out,
+                                int n_traces, float* __restrict__ y) {
+  const int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= n_out) return;
   const int c = c0[m], L = len[m];
   const int groups = (n_traces + kFT - 1) / kFT;
@@ -603,10 +604,10 @@ cudaError_t launch_band_rows(const float* x, int n_in, const int* c0, const int*
   const int groups = (n_traces + kBT - 1) / kBT, tiles = (n_out + kBM - 1) / kBM;
   // A thread per output below 48 taps (its loads of neighbouring outputs fall
   // into the same lines: 65,536 traces of 4000 samples, nearest, 185 us against
-  // 511; sinc of equal steps, 16 taps, 952 against 1062; sinc to 1818 samples, 36
-  // taps, 1038 against 1150, but 79 taps 1343 against 842) and where the tiles
-  // leave SMs idle (79 taps: 84 tiles 29 us against 36, 104 30 against 37, 280
-  // 51 against 41).
+  // 511; sinc of equal steps, 16 taps, 829 against 1062; sinc to 1818 samples, 36
+  // taps, 1018 against 1150, but 79 taps 1336 against 842) and where the tiles
+  // leave SMs idle (79 taps: 84 tiles 27 us against 36, 104 30 against 37, 280
+  // 50 against 41).
   if (taps < 48 || (long long)groups * tiles < 200) {
     const int few = (n_traces + kFT - 1) / kFT;
     const dim3 g((unsigned)((n_out + 127) / 128), (unsigned)(few < 65535 ? few : 65535));

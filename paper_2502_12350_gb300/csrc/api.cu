@@ -1520,8 +1520,10 @@ int run_model(mamute_ctx* ctx, const mamute_grid* g, const float* vel, const flo
     TRY(setup_pairs(ctx, P, vel, rho));
     CK(cudaMemsetAsync(ctx->pflags.p, 0, P.pitems.size() * 4, ctx->stream));
   }
-  // The time loop is captured into a CUDA graph and replayed while the plan,
-  // the buffers and the wavelet stay the same (MAMUTE_GRAPHS=0 disables).
+  // The time loop is captured into a CUDA graph and replayed while everything
+  // that its launches take by value stays the same: sizes, grids, pointers and
+  // the wavelet (MAMUTE_GRAPHS=0 disables).  What lies in device tables is
+  // uploaded anew by each call.
   std::vector<unsigned long long> key;
   // Seismograms stream to the host during the loop unless they are resampled
   // to a data time axis first.
@@ -1536,6 +1538,7 @@ int run_model(mamute_ctx* ctx, const mamute_grid* g, const float* vel, const flo
     key.push_back((unsigned long long)mode * 2 + P.dens);
     key.push_back((unsigned long long)P.ncol);
     key.push_back((unsigned long long)P.planes);
+    key.push_back((unsigned long long)(unsigned)P.zs);
     for (const DevBuf* b : {&ctx->items, &ctx->vols, &ctx->maps, &ctx->cmaps, &ctx->gx, &ctx->gy,
                             &ctx->gz, &ctx->recptr, &ctx->rec, &ctx->acc, &ctx->dint,
                             &ctx->pool[0], &ctx->pool[1]})
@@ -1546,13 +1549,17 @@ int run_model(mamute_ctx* ctx, const mamute_grid* g, const float* vel, const flo
       key.push_back(u);
     }
     key.push_back(pairs ? (((unsigned long long)P.ptx << 32) | (unsigned)P.pty) : 0);
+    key.push_back(pairs ? (unsigned long long)P.pitems.size() : 0);
+    key.push_back(pairs ? (unsigned long long)P.Nz : 0);  // (the progress flags count its planes)
     for (const DevBuf* b : {&ctx->pitems, &ctx->pnbr, &ctx->precptr, &ctx->prec, &ctx->pmaps,
                             &ctx->pflags})
       push(pairs ? b->p : nullptr);
     key.push_back(P.pml ? 1 : 0);
     for (const DevBuf* b : {&ctx->cpml, &ctx->cext, &ctx->cprof, &ctx->cvols})
       push(P.pml ? b->p : nullptr);
-    // the slab launches' grids and the arrays' size
+    // the slab launches' grids, the arrays' size and the profiles
+    key.push_back(P.pml ? (unsigned long long)T.ext.nvol : 0);
+    push(T.base.c);
     for (int a = 0; a < 3; ++a) {
       key.push_back(P.pml ? (unsigned long long)T.ext.cols[a] : 0);
       key.push_back(P.pml ? (unsigned long long)T.ext.len[a] : 0);
@@ -1563,6 +1570,11 @@ int run_model(mamute_ctx* ctx, const mamute_grid* g, const float* vel, const flo
     if (stream_out) {
       push(seis);
       push(host_seis);
+      // how data_to_user combines the columns
+      key.push_back((unsigned long long)P.nrec * 2 + P.one_node);
+      push(P.one_node ? ctx->colmap.p : nullptr);
+      for (const DevBuf* b : {&ctx->ident, &ctx->ecol, &ctx->rcolptr, &ctx->rcols})
+        push(P.one_node ? nullptr : b->p);
     }
   }
   // Steps [t0, t1): pairs of steps (n even) by the two-level kernel, the

@@ -1106,7 +1106,9 @@ int do_smooth(mamute_ctx* ctx, int nx, int ny, int nz, double h, int mode, const
     const double l = lengths ? (double)lengths[a] : 0.0;
     if (!(l >= 0.0)) return fail(ctx, MAMUTE_EINVAL, "smoothing length %d is negative", a);
     L[a] = l > 0.0 ? l : 2.0 * h;
-    mu[a] = (L[a] / h) * (L[a] / h);
+    // beyond 1e9 cells the filter passes the mean alone, to below FP32
+    const double cells = std::min(L[a] / h, 1e9);
+    mu[a] = cells * cells;
   }
   // Tables, built and uploaded only when the sizes, the spacing, the lengths
   // or the mode differ from the previous call's.  Bessel: per axis y, z the
@@ -1117,7 +1119,7 @@ int do_smooth(mamute_ctx* ctx, int nx, int ny, int nz, double h, int mode, const
   for (int a = 1; a < 3; ++a) {
     const size_t hn = (size_t)(dims[a] + 1) / 2;
     off[a] = total;
-    total += bessel ? 4 * hn * hn : 2 * (size_t)dims[a];
+    total += bessel ? 4 * hn * hn : 4 * (size_t)dims[a] + 2;
   }
   const std::vector<double> key = {(double)nx, (double)ny, (double)nz, h, L[0], L[1], L[2], (double)mode};
   if (key != ctx->smKey) {
@@ -1137,13 +1139,13 @@ int do_smooth(mamute_ctx* ctx, int nx, int ny, int nz, double h, int mode, const
             t[(2 + odd) * hh + (size_t)(k / 2) * hn + j] = c;
           }
       } else {
-        double g = 0.0;  // mu / pivot of the row above
+        float* inv = t + 2 * m + 2;
+        double d = 0.0;  // 1 - g of the row above
         for (int j = 0; j < m; ++j) {
-          const int links = (j > 0) + (j + 1 < m);
-          const double inv = 1.0 / (1.0 + mu[a] * (links - g));
-          g = mu[a] * inv;
-          t[2 * j] = (float)inv;
-          t[2 * j + 1] = (float)g;
+          const double piv = j == 0 ? 1.0 + mu[a] : (j + 1 < m ? 1.0 + mu[a] + mu[a] * d : 1.0 + mu[a] * d);
+          d = (j == 0 ? 1.0 : 1.0 + mu[a] * d) / piv;
+          inv[j] = (float)(1.0 / piv);
+          if (j + 1 < m) split_ratio(mu[a] / piv, d, t + 2 * j + 2, t + 2 * j + 3);
         }
       }
     }
@@ -1171,8 +1173,9 @@ int do_smooth(mamute_ctx* ctx, int nx, int ny, int nz, double h, int mode, const
     for (int a = 1; a < 3; ++a) {
       if (dims[a] == 1) continue;
       ++ctx->launches;
-      CK(launch_sweep(out, out, (const float2*)(M + off[a]), dims[a], g[a][0], g[a][1], g[a][2], g[a][3],
-                      ctx->stream));
+      const float* t = M + off[a];
+      CK(launch_sweep(out, out, (const float2*)t, t + 2 * dims[a] + 2, mu[a] > kCarryCells * kCarryCells,
+                      dims[a], g[a][0], g[a][1], g[a][2], g[a][3], ctx->stream));
     }
     return MAMUTE_OK;
   }

@@ -41,18 +41,19 @@ namespace {
 // p_{-1} = (q0 + r^n p0) / (1 - r^{2n}) (q0, p0: q_0 and p_{n-1} of the line
 // alone) and q_n = p_{n-1}.  All terms have the sign of f: no cancellation.
 
-// r and K of a line, and the powers the parallel recursion needs, formed in
-// FP64 from the rounded r (so that a constant is kept to rounding).
-__device__ __forceinline__ RowCoef row_coef(double s, double mu, int n, int len) {
-  const double a = s / (2.0 * mu);
-  RowCoef c;
-  c.r = (float)(1.0 / (1.0 + a + sqrt(a * (a + 2.0))));
-  const double r = c.r;
-  c.K = (float)((1.0 - r) / (s * (1.0 + r)));
-  c.rl = (float)pow(r, (double)len);
-  const double rn = pow(r, (double)n);
-  c.rn = (float)rn;
-  c.w = (float)(1.0 / (1.0 - rn * rn));
+// Formed in FP64 from x = 1 / r - 1 = a + sqrt(a (a + 2)), a = s / (2 mu), which
+// gives 1 - r without a cancellation however long the filter.
+__host__ __device__ inline RowCoef row_coef(double s, double mu, int n, int len) {
+  const double a = s / (2.0 * mu), x = a + sqrt(a) * sqrt(a + 2.0);
+  const double r = 1.0 / (1.0 + x), d = x / (1.0 + x);
+  const double lr = r < 0.5 ? log(r) : log1p(-d);
+  RowCoef c{};
+  split_ratio(r, d, &c.r, &c.rlo);
+  c.K = (float)(d / (s * (1.0 + r)));
+  c.rl = (float)exp(len * lr);
+  c.rt = (float)exp(n % len * lr);
+  c.rn = (float)exp(n * lr);
+  c.w = (float)(-1.0 / expm1(2.0 * n * lr));
   return c;
 }
 
@@ -71,7 +72,12 @@ __global__ void row_coef_kernel(RowCoef* out, int ny, int nz, double my, double 
 // The row is staged in shared memory (row and p, 8 bytes a cell) so that
 // DRAM sees one read and one write, or, for rows beyond kRowSmem bytes, left
 // in global memory with p in `scratch`.  Bound by HBM and the shared-memory
-// accesses (about 9 a cell).
+// accesses (about 9 a cell), so that the second multiply-add of a step, for the
+// low part of r, costs 10 us of the 2.92 ms of the 600x600x200 Bessel filter.
+// Without it the length that was applied was off by 6e-8 of itself per cell of
+// it (relative L2 errors on zero-mean rows of 700 cells 1.9e-6 at 200 cells, now
+// 2.4e-7; no result above 3e7, where r rounds to 1).  What is left are the roundings of
+// the lanes' sums and of the scan: below 1e-6 however long the filter.
 __global__ void row_kernel(const float* in, float* out, float* scratch, int n, int len,
                            long long rows, const RowCoef* __restrict__ coef, RowCoef one, bool staged) {
   extern __shared__ float row_smem[];
@@ -91,15 +97,11 @@ __global__ void row_kernel(const float* in, float* out, float* scratch, int n, i
       p = sf + n;
     }
     const int b = min(lane * len, n), e = min(b + len, n);
+    auto times_r = [&](float v, float add) { return fmaf(c.r, v, fmaf(c.rlo, v, add)); };
     float cp = 0.0f, cq = 0.0f;  // p of the last and q of the first owned cell, from zero
-    for (int j = b; j < e; ++j) cp = fmaf(c.r, cp, f[j]);
-    for (int j = e - 1; j >= b; --j) cq = fmaf(c.r, cq, f[j]);
-    float a = c.rl;
-    if (e - b < len) {
-      a = 1.0f;
-      for (int j = b; j < e; ++j) a *= c.r;
-    }
-    float ap = a, aq = a;
+    for (int j = b; j < e; ++j) cp = times_r(cp, f[j]);
+    for (int j = e - 1; j >= b; --j) cq = times_r(cq, f[j]);
+    float ap = e - b == len ? c.rl : (e > b ? c.rt : 1.0f), aq = ap;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
       const float pc = __shfl_up_sync(0xffffffffu, cp, d), pa = __shfl_up_sync(0xffffffffu, ap, d);
@@ -121,14 +123,14 @@ __global__ void row_kernel(const float* in, float* out, float* scratch, int n, i
     float pv = lane == 0 ? pm1 : fmaf(pa, pm1, pc);
     float qv = lane == 31 ? qn : fmaf(qa, qn, qc);
     for (int j = b; j < e; ++j) {
-      pv = fmaf(c.r, pv, f[j]);
+      pv = times_r(pv, f[j]);
       p[j] = pv;
     }
     float* res = staged ? p : o;
     for (int j = e - 1; j >= b; --j) {
       const float fj = f[j];
-      res[j] = c.K * fmaf(c.r, qv, p[j]);
-      qv = fmaf(c.r, qv, fj);
+      res[j] = c.K * times_r(qv, p[j]);
+      qv = times_r(qv, fj);
     }
     if (staged) {
       __syncwarp();
@@ -139,13 +141,39 @@ __global__ void row_kernel(const float* in, float* out, float* scratch, int n, i
 
 constexpr int kRowSmem = 200 * 1024;
 
+// v <- g v + f, g as hi + lo.  CARRY: v as hi + lo too, lo taking what the
+// rounding of hi drops (the product's and the sum's errors); one multiply-add
+// lies on the chain of hi and one on that of lo.
+template <bool CARRY>
+__device__ __forceinline__ void recur(float& hi, float& lo, float g, float glo, float f) {
+  if (!CARRY) {
+    hi = fmaf(g, hi, fmaf(glo, hi, f));
+    return;
+  }
+  const float s = fmaf(g, hi, f);
+  const float p = __fmul_rn(g, hi), pe = fmaf(glo, hi, fmaf(g, hi, -p));
+  // s - p = b + be exactly
+  const float b = __fsub_rn(s, p), q = __fsub_rn(s, b);
+  const float be = __fadd_rn(__fsub_rn(s, __fadd_rn(b, q)), __fsub_rn(q, p));
+  lo = fmaf(g, lo, __fadd_rn(__fsub_rn(__fsub_rn(f, b), be), pe));
+  hi = s;
+}
+
 // Solves along y or z in place, one column per thread (consecutive threads on
-// consecutive x): elimination upwards, y_i = inv_i f_i + g_i y_{i-1}, and
-// back-substitution downwards, u_i = y_i + g_i u_{i+1}, with the factors of
-// the one matrix all columns share (formed on the host in FP64).  Two reads
-// and two writes of the volume; the loads of 8 cells are issued together.
-__global__ void __launch_bounds__(256) sweep_kernel(const float* in, float* out,
-                                                    const float2* __restrict__ fac, int n,
+// consecutive x): z_i = f_i + g_i z_{i-1} upwards and u_i = inv_i z_i + g_{i+1}
+// u_{i+1} downwards, with the factors of the one matrix all columns share
+// (formed on the host in FP64; every g is below 1, g_0 = g_n = 0).  Two reads and
+// two writes of the volume; the loads of 8 cells are issued together.
+//
+// CARRY for filters beyond kCarryCells: the roundings of v add up over a filter's
+// length (relative L2 errors of 1.3e-7 at 30 cells, 2.2e-7 at 100 and 1.7e-6 at
+// 30,000 on lines of 700, where dense transforms have 3.3e-7, 4.0e-7 and 1.0e-6);
+// carried they stay below 1e-7.  The Laplace filter of 600x600x200 takes 622 us
+// without and 672 with it (4 blocks per SM without: with 3 it takes 700).
+template <bool CARRY>
+__global__ void __launch_bounds__(256, CARRY ? 3 : 4) sweep_kernel(const float* in, float* out,
+                                                    const float2* __restrict__ g,
+                                                    const float* __restrict__ inv, int n,
                                                     long long lines, long long inner,
                                                     long long outer, long long st) {
   const long long L = blockIdx.x * 256LL + threadIdx.x;
@@ -153,7 +181,7 @@ __global__ void __launch_bounds__(256) sweep_kernel(const float* in, float* out,
   const long long base = (L / inner) * outer + L % inner;
   const float* f = in + base;
   float* u = out + base;
-  float v = 0.0f;
+  float hi = 0.0f, lo = 0.0f;
   for (int i0 = 0; i0 < n; i0 += 8) {
     float t[8];
 #pragma unroll
@@ -161,12 +189,12 @@ __global__ void __launch_bounds__(256) sweep_kernel(const float* in, float* out,
 #pragma unroll
     for (int k = 0; k < 8; ++k)
       if (i0 + k < n) {
-        const float2 c = __ldg(fac + i0 + k);
-        v = fmaf(c.y, v, c.x * t[k]);
-        u[(i0 + k) * st] = v;
+        const float2 c = __ldg(g + i0 + k);
+        recur<CARRY>(hi, lo, c.x, c.y, t[k]);
+        u[(i0 + k) * st] = CARRY ? hi + lo : hi;
       }
   }
-  v = 0.0f;
+  hi = lo = 0.0f;
   for (int i0 = (n - 1) / 8 * 8; i0 >= 0; i0 -= 8) {
     float t[8];
 #pragma unroll
@@ -174,8 +202,9 @@ __global__ void __launch_bounds__(256) sweep_kernel(const float* in, float* out,
 #pragma unroll
     for (int k = 7; k >= 0; --k)
       if (i0 + k < n) {
-        v = fmaf(__ldg(fac + i0 + k).y, v, t[k]);
-        u[(i0 + k) * st] = v;
+        const float2 c = __ldg(g + i0 + k + 1);
+        recur<CARRY>(hi, lo, c.x, c.y, __ldg(inv + i0 + k) * t[k]);
+        u[(i0 + k) * st] = CARRY ? hi + lo : hi;
       }
   }
 }
@@ -538,17 +567,7 @@ cudaError_t launch_sub(const float* a, const float* b, long long n, float* out, 
 
 int row_len(int n) { return ((n + 31) / 32) | 1; }
 
-RowCoef row_coef_host(double s, double mu, int n) {
-  const double a = s / (2.0 * mu);
-  RowCoef c;
-  c.r = (float)(1.0 / (1.0 + a + std::sqrt(a * (a + 2.0))));
-  const double r = c.r, rn = std::pow(r, (double)n);
-  c.K = (float)((1.0 - r) / (s * (1.0 + r)));
-  c.rl = (float)std::pow(r, (double)row_len(n));
-  c.rn = (float)rn;
-  c.w = (float)(1.0 / (1.0 - rn * rn));
-  return c;
-}
+RowCoef row_coef_host(double s, double mu, int n) { return row_coef(s, mu, n, row_len(n)); }
 
 cudaError_t launch_row_coef(RowCoef* out, int ny, int nz, double my, double mz, double mx, int nx,
                             cudaStream_t s) {
@@ -577,10 +596,14 @@ cudaError_t launch_rows(const float* in, float* out, float* scratch, int n, long
   return cudaGetLastError();
 }
 
-cudaError_t launch_sweep(const float* in, float* out, const float2* fac, int n, long long lines,
-                         long long inner, long long outer, long long st, cudaStream_t s) {
+cudaError_t launch_sweep(const float* in, float* out, const float2* g, const float* inv, bool carry, int n,
+                         long long lines, long long inner, long long outer, long long st, cudaStream_t s) {
   if (lines <= 0 || n <= 0) return cudaSuccess;
-  sweep_kernel<<<(unsigned)((lines + 255) / 256), 256, 0, s>>>(in, out, fac, n, lines, inner, outer, st);
+  const unsigned blocks = (unsigned)((lines + 255) / 256);
+  if (carry)
+    sweep_kernel<true><<<blocks, 256, 0, s>>>(in, out, g, inv, n, lines, inner, outer, st);
+  else
+    sweep_kernel<false><<<blocks, 256, 0, s>>>(in, out, g, inv, n, lines, inner, outer, st);
   return cudaGetLastError();
 }
 

@@ -230,24 +230,16 @@ __global__ void sum_partials_kernel(const double* partial, int n, double* out) {
   }
 }
 
-// 1 / v by one Newton step in FP64 from the FP32 reciprocal (relative error
-// 4e-15), by division where that leaves the FP32 range.
-__device__ __forceinline__ double recip(double v) {
-  const float r = 1.0f / (float)v;
-  if (!(fabsf(r) > 1e-30f && fabsf(r) < 1e30f)) return 1.0 / v;
-  return fma((double)r, fma(-v, (double)r, 1.0), (double)r);
-}
-
 // grad[z][y][x] = 2 / (c^3 dt^2) sum_s G_s, or phess = sum_s P_s / (c dt)^4,
-// summed over shots in ascending order (deterministic).  One block per row.
-// Bound by the FP64 units, a 64th of the FP32 rate: with an FP64 division and
-// 64-bit index divisions per point 256^3 took 866 us (a 192^3 gradient
-// 82.86 -> 82.63 ms, the same bits).
+// summed over shots in ascending order (deterministic).  One block per row, so that
+// no point divides its 64-bit index.  Bound by the FP64 units, a 64th of the FP32
+// rate: 256^3 takes 503 us.  The quotient is one FP64 division: a Newton step from
+// an FP32 reciprocal in its place saved 14 us and left errors of 8e-15, which show
+// in rare FP32 roundings.
 __global__ void __launch_bounds__(128) finalize_kernel(FinalizeArgs a) {
   const int y = (int)(blockIdx.x % (unsigned)a.ny), z = (int)(blockIdx.x / (unsigned)a.ny);
   const int Y = y + a.border, Z = z + a.border;
   const long long row = (long long)blockIdx.x * a.nx;
-  const double dt2 = a.dt * a.dt, k = a.kind == 0 ? 2.0 / dt2 : 1.0 / (dt2 * dt2);
   for (int x = threadIdx.x; x < a.nx; x += 128) {
     const int X = x + a.border;
     float acc = 0.0f;
@@ -258,9 +250,15 @@ __global__ void __launch_bounds__(128) finalize_kernel(FinalizeArgs a) {
       if (lx < V.ix0 || ly < V.iy0 || lx >= V.ix0 + V.nxi || ly >= V.iy0 + V.nyi) continue;
       acc += a.acc[V.off + ((long long)Z * V.Ny + ly) * V.pitch + lx];
     }
-    const double cv = a.vel[row + x], c2 = cv * cv;
-    double out = k * (double)acc * recip(a.kind == 0 ? c2 * cv : c2 * c2);
-    if (a.kind == 0 && z < a.zero_top) out = 0.0;
+    const double cv = a.vel[row + x];
+    double out;
+    if (a.kind == 0) {
+      out = 2.0 * (double)acc / (cv * cv * cv * a.dt * a.dt);
+      if (z < a.zero_top) out = 0.0;
+    } else {
+      const double A2 = cv * cv * a.dt * a.dt;
+      out = (double)acc / (A2 * A2);
+    }
     a.out[row + x] = (float)out;
   }
 }

@@ -5,12 +5,10 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <array>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
-#include <map>
 #include <string>
 #include <vector>
 
@@ -20,6 +18,7 @@
 #include "gn.h"
 #include "common.cuh"
 #include "cpml.h"
+#include "device_state.h"
 #include "postproc.h"
 #include "revolve.h"
 #include "stencil.h"
@@ -373,17 +372,10 @@ void build_receivers(Plan& P, int TX, int zsplit, const std::vector<NodeEntry>& 
   }
 }
 
-// step_blocks_per_sm, remembered per kernel variant and table length (a driver
-// query of about a microsecond, asked for every candidate of every call).
-int blocks_per_sm(int tx, int ty, bool dens, bool pml, int mode, int planes) {
-  thread_local std::map<std::array<int, 6>, int> known;
-  const std::array<int, 6> key = {tx, ty, dens, pml, mode, planes};
-  auto it = known.find(key);
-  if (it == known.end()) {
-    if (known.size() > 4096) known.clear();
-    it = known.emplace(key, step_blocks_per_sm(tx, ty, dens, pml, mode, planes)).first;
-  }
-  return it->second;
+int blocks_per_sm(int device, int tx, int ty, bool dens, bool pml, int mode, int planes) {
+  thread_local OccupancyMemo memo;
+  return memo.get({device, tx, ty, dens, pml, mode, planes},
+                  [&] { return step_blocks_per_sm(tx, ty, dens, pml, mode, planes); });
 }
 
 // Chooses, among the compiled tile shapes, the shape, a row refinement and a
@@ -411,8 +403,8 @@ struct TileChoice {
   std::vector<Tiling> tilings;
 };
 
-TileChoice choose_tiles(const std::vector<VolDesc>& vols, bool dens, bool pml, int mode, int n_sm,
-                        int force_tx, int force_ty, int force_z) {
+TileChoice choose_tiles(const std::vector<VolDesc>& vols, bool dens, bool pml, int mode, int device,
+                        int n_sm, int force_tx, int force_ty, int force_z) {
   static const int shapes[][2] = {{64, 16}, {72, 16}, {48, 16}, {96, 8}, {64, 8},
                                   {128, 8}, {32, 16}, {32, 8}};
   static const int zsplits[] = {1, 2, 3, 4, 5, 6, 7, 8, 10, 12, 14, 16, 20, 24, 32, 48};
@@ -430,8 +422,8 @@ TileChoice choose_tiles(const std::vector<VolDesc>& vols, bool dens, bool pml, i
     // per-plane table counts as long as the z block is.
     int per_sm_of[sizeof zsplits / sizeof zsplits[0]];
     for (size_t k = 0; k < sizeof zsplits / sizeof zsplits[0]; ++k)
-      per_sm_of[k] = blocks_per_sm(TX, TY, dens, pml, mode,
-                                        mode == MODE_ADJ_STORED ? (Nz + zsplits[k] - 1) / zsplits[k] : Nz);
+      per_sm_of[k] = blocks_per_sm(device, TX, TY, dens, pml, mode,
+                                   mode == MODE_ADJ_STORED ? (Nz + zsplits[k] - 1) / zsplits[k] : Nz);
     const int warps_cta = (TX / 4) * TY / 32;
     for (int r = 1; r <= 2; ++r) {
       std::vector<Tiling> tl;
@@ -655,13 +647,13 @@ int plan_tiles(mamute_ctx* ctx, Plan& P, const int* tiles, int adj_mode) {
   if (n_sm < 1) n_sm = 1;
   const int fmode = dens ? MODE_FWD : MODE_FWD;
   auto pick = [&](int i, const char* env) { return (tiles && tiles[i] > 0) ? tiles[i] : env_int(env, 0); };
-  TileChoice fc = choose_tiles(P.vols, dens, P.pml, fmode, n_sm, pick(0, "MAMUTE_TX"), pick(1, "MAMUTE_TY"),
-                               pick(2, "MAMUTE_ZSPLIT"));
+  TileChoice fc = choose_tiles(P.vols, dens, P.pml, fmode, ctx->device, n_sm, pick(0, "MAMUTE_TX"),
+                               pick(1, "MAMUTE_TY"), pick(2, "MAMUTE_ZSPLIT"));
   const int ax = pick(3, "MAMUTE_ADJ_TX"), ay = pick(4, "MAMUTE_ADJ_TY"), az = pick(5, "MAMUTE_ADJ_ZSPLIT");
   TileChoice ac = fc;
   if (adj_mode >= 0 || ax > 0 || ay > 0 || az > 0)  // (a shape asked for is checked in any call)
-    ac = choose_tiles(P.vols, dens, P.pml, P.pml ? MODE_ADJ_STORED : std::max(adj_mode, (int)MODE_ADJ), n_sm,
-                      ax, ay, az);
+    ac = choose_tiles(P.vols, dens, P.pml, P.pml ? MODE_ADJ_STORED : std::max(adj_mode, (int)MODE_ADJ),
+                      ctx->device, n_sm, ax, ay, az);
   if (fc.tilings.empty() || ac.tilings.empty())
     return fail(ctx, MAMUTE_EINVAL, "unsupported tile shape");
   P.tx = fc.tx; P.ty = fc.ty; P.atx = ac.tx; P.aty = ac.ty;

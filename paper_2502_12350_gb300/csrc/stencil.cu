@@ -27,8 +27,10 @@ static cudaError_t dispatch(const StepArgs& a, int n_items, int max_planes, int 
 int step_blocks_per_sm(int tx, int ty, bool dens, bool pml, int mode, int max_planes) {
   int occ = 0;
   StepArgs a{};
-  if (dispatch(a, 0, max_planes, tx, ty, dens, pml, mode, nullptr, &occ) != cudaSuccess) return 0;
-  return occ;
+  const cudaError_t e = dispatch(a, 0, max_planes, tx, ty, dens, pml, mode, nullptr, &occ);
+  if (e == cudaSuccess) return occ;
+  cudaGetLastError();  // the caller takes another shape
+  return e == cudaErrorInvalidValue ? 0 : -1;
 }
 
 cudaError_t launch_step(const StepArgs& a, int n_items, int max_planes, int tx, int ty, bool dens,

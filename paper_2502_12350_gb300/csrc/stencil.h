@@ -90,7 +90,8 @@ cudaError_t launch_pair(const PairArgs& a, int n_items, int nz, int tx, int ty, 
                         cudaStream_t s, int* occ);
 
 bool tile_supported(int tx, int ty);
-// Resident CTAs per SM of a step kernel configuration (0 if it cannot run).
+// Resident CTAs per SM of a step kernel configuration (0 if it cannot run, -1 if
+// the query failed).
 int step_blocks_per_sm(int tx, int ty, bool dens, bool pml, int mode, int max_planes);
 // max_planes: the largest ze - zb of the launch's items (sizes the per-plane table).
 cudaError_t launch_step(const StepArgs& a, int n_items, int max_planes, int tx, int ty, bool dens,

@@ -1,0 +1,42 @@
+"""What the library remembers about devices on the host (csrc/device_state.h),
+with the CUDA calls played by the test."""
+import os
+import subprocess
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2502_12350_gb300",
+                    "csrc")
+
+PRELUDE = r"""
+#include <cstdio>
+#include <cstdlib>
+#define CHECK(c) do { if (!(c)) { std::printf("line %d: %s\n", __LINE__, #c); std::exit(1); } } while (0)
+"""
+
+
+def _run(tmp_path, body, header="device_state.h"):
+    src, exe = str(tmp_path / "t.cpp"), str(tmp_path / "t")
+    with open(src, "w") as f:
+        f.write(f'#include "{header}"\n' + PRELUDE + body)
+    subprocess.run(["g++", "-std=c++17", "-O1", "-Wall", "-pthread", "-I", CSRC, src, "-o", exe], check=True)
+    r = subprocess.run([exe], capture_output=True, text=True, timeout=60)
+    assert r.returncode == 0, r.stdout + r.stderr
+
+
+def test_occupancy_is_kept_by_device_and_not_after_a_failure(tmp_path):
+    _run(tmp_path, r"""
+int main() {
+  mamute::OccupancyMemo memo;
+  int asked = 0;
+  auto answer = [&](int n) { return [&asked, n] { ++asked; return n; }; };
+  CHECK(memo.get({0, 64, 16, 0, 0, 0, 100}, answer(-1)) == -1);  // a failed query
+  CHECK(memo.get({0, 64, 16, 0, 0, 0, 100}, answer(2)) == 2);    // is asked again
+  CHECK(memo.get({0, 64, 16, 0, 0, 0, 100}, answer(7)) == 2 && asked == 2);
+  CHECK(memo.get({1, 64, 16, 0, 0, 0, 100}, answer(3)) == 3);    // another device has its own
+  CHECK(memo.get({0, 64, 16, 0, 0, 0, 101}, answer(0)) == 0);    // a variant that does not fit
+  CHECK(memo.get({0, 64, 16, 0, 0, 0, 101}, answer(5)) == 0 && asked == 4);
+  for (int k = 0; k < 5000; ++k) memo.get({0, 0, 0, 0, 0, 0, k}, answer(1));
+  CHECK(memo.get({0, 0, 0, 0, 0, 0, 4999}, answer(9)) == 1);     // bounded, the latest kept
+}
+""")

@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "device_state.h"
+
 namespace mamute {
 
 // Radius-4 central weights of the eighth-order second derivative
@@ -85,6 +87,17 @@ struct ShotMaps {
 struct CoefMaps {
   CUtensorMap m[2];
 };
+
+// Allows `kernel` `bytes` of dynamic shared memory on the current device.
+template <typename K>
+cudaError_t allow_smem(SmemLimit& limit, K kernel, size_t bytes) {
+  int device = 0;
+  const cudaError_t e = cudaGetDevice(&device);
+  if (e != cudaSuccess) return e;
+  return static_cast<cudaError_t>(limit.raise(device, bytes, [&](size_t b) {
+    return (int)cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b);
+  }));
+}
 
 // ---------------------------------------------------------------- PTX helpers
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {

@@ -459,13 +459,9 @@ cudaError_t launch_conv(const ConvArgs& a, const CUtensorMap& xmap, int* status,
   // At least 116 KB so that one CTA runs per SM and TMEM allocation never
   // waits for another CTA of this kernel.
   const size_t sm = std::max<size_t>(tc_smem_bytes(p), 116 * 1024);
-  static size_t attr = 0;
-  if (sm > attr) {
-    cudaError_t e =
-        cudaFuncSetAttribute(conv_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-    attr = sm;
-  }
+  static SmemLimit limit;
+  const cudaError_t e = allow_smem(limit, conv_tc_kernel, sm);
+  if (e != cudaSuccess) return e;
   const int grid = (int)std::min<long long>(p.items, 152);
   conv_tc_kernel<<<grid, kTcThreads, sm, s>>>(xmap, a, p, status);
   return cudaGetLastError();
@@ -475,17 +471,12 @@ cudaError_t launch_wgrad(const WgradArgs& a, const CUtensorMap& xmap, const CUte
                          int* status, float* gw, float* gb, cudaStream_t s) {
   const long long n_tiles = (long long)((a.W + kTX - 1) / kTX) * ((a.H + kTY - 1) / kTY) *
                             ((a.D + kFZ - 1) / kFZ);
-  static bool attr = false;
-  if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(conv_wgrad_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         kWStages * kWStage + 256);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+  static SmemLimit limit;
+  cudaError_t e = allow_smem(limit, conv_wgrad_kernel, kWStages * kWStage + 256);
+  if (e != cudaSuccess) return e;
   const int grid = (int)std::min<long long>(n_tiles, wgrad_blocks());
   conv_wgrad_kernel<<<grid, kWThreads, kWStages * kWStage + 256, s>>>(xmap, gmap, a, status);
-  cudaError_t e = cudaGetLastError();
+  e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const int n = kTaps * kC * kC + kC, groups = (grid + kRedGroup - 1) / kRedGroup;
   double* stage = reinterpret_cast<double*>(a.partial + (size_t)wgrad_blocks() * n);

@@ -2,8 +2,12 @@
 // rules are tested on the host (tests/test_device_state.py).
 #pragma once
 
+#include <algorithm>
 #include <array>
+#include <atomic>
+#include <cstddef>
 #include <map>
+#include <mutex>
 
 namespace mamute {
 
@@ -26,6 +30,32 @@ class OccupancyMemo {
 
  private:
   std::map<Key, int> known_;
+};
+
+// The dynamic shared memory that one kernel has been allowed, per device: the
+// allowance is an attribute of the kernel on a device, and setting it again may
+// lower it under a launch of another thread.  raise() sets it through
+// set(bytes), zero on success, where it is not yet that large.
+class SmemLimit {
+ public:
+  template <typename F>
+  int raise(int device, size_t bytes, F set) {
+    const bool shared = device < 0 || device >= kDevices - 1;  // the last entry is of all others
+    std::atomic<size_t>& have = have_[shared ? kDevices - 1 : device];
+    if (!shared && have.load(std::memory_order_acquire) >= bytes) return 0;
+    std::lock_guard<std::mutex> lock(mutex_);
+    const size_t old = have.load(std::memory_order_relaxed);
+    if (!shared && old >= bytes) return 0;
+    const size_t want = std::max(old, bytes);
+    const int e = set(want);
+    if (e == 0) have.store(want, std::memory_order_release);
+    return e;
+  }
+
+ private:
+  static constexpr int kDevices = 64;
+  std::mutex mutex_;
+  std::atomic<size_t> have_[kDevices] = {};
 };
 
 }  // namespace mamute

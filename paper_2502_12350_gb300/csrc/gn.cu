@@ -585,13 +585,9 @@ cudaError_t launch_dft(const float* V, long long N, int T, int n0, int nf, const
   const size_t sm = dft_smem_bytes(T, nb);
   const bool vec = (N % 4) == 0 && ((uintptr_t)V % 16) == 0 && ((uintptr_t)W % 16) == 0 &&
                    ((uintptr_t)re % 16) == 0 && ((uintptr_t)im % 16) == 0;
-  static size_t attr[2] = {0, 0};
-  if (sm > attr[vec]) {
-    e = vec ? cudaFuncSetAttribute(dft_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)
-            : cudaFuncSetAttribute(dft_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-    attr[vec] = sm;
-  }
+  static SmemLimit limit[2];
+  e = vec ? allow_smem(limit[1], dft_kernel<true>, sm) : allow_smem(limit[0], dft_kernel<false>, sm);
+  if (e != cudaSuccess) return e;
   const int threads = 32 * (nbh / kChunk);
   int per_sm = 1;
   e = vec ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, dft_kernel<true>, threads, sm)
@@ -627,12 +623,9 @@ cudaError_t launch_dft_tc(const CUtensorMap& vmap, long long N, int T, int n0, i
   dft_image_kernel<<<(n + 255) / 256, 256, 0, s>>>(T, n0, nf, bins, nb, mt, nch, W);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  static bool attr = false;
-  if (!attr) {
-    e = cudaFuncSetAttribute(dft_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmem);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+  static SmemLimit limit;
+  e = allow_smem(limit, dft_tc_kernel, kTcSmem);
+  if (e != cudaSuccess) return e;
   DftTcArgs a{W, re, im, N, nb, mt, nch, overwrite ? 1 : 0, status};
   const long long ntiles = (N + kTcNP - 1) / kTcNP;
   const int grid = (int)std::min<long long>(ntiles, 152);

@@ -554,13 +554,9 @@ template <int TX, int TY, bool DENS, int MODE, bool PML>
 static cudaError_t launch_one(const StepArgs& a, int n_items, int max_planes, cudaStream_t s,
                               int* occupancy) {
   const size_t sm = smem_bytes<TX, TY, DENS, MODE, PML>(max_planes);
-  static size_t attr_bytes = 0;
-  if (sm > attr_bytes) {
-    cudaError_t e = cudaFuncSetAttribute(step_kernel<TX, TY, DENS, MODE, PML>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-    attr_bytes = sm;
-  }
+  static SmemLimit limit;
+  const cudaError_t e = allow_smem(limit, step_kernel<TX, TY, DENS, MODE, PML>, sm);
+  if (e != cudaSuccess) return e;
   if (occupancy) {
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occupancy, step_kernel<TX, TY, DENS, MODE, PML>,
                                                          (TX / 4) * TY + 32, sm);

@@ -616,13 +616,9 @@ static size_t pair_smem(int) {
 template <int TX, int TY, bool DENS>
 static cudaError_t pair_one(const PairArgs& a, int n_items, int nz, cudaStream_t s, int* occ) {
   const size_t sm = pair_smem<TX, TY, DENS>(nz);
-  static size_t attr = 0;
-  if (sm > attr) {
-    cudaError_t e = cudaFuncSetAttribute(pair_kernel<TX, TY, DENS>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-    attr = sm;
-  }
+  static SmemLimit limit;
+  const cudaError_t e = allow_smem(limit, pair_kernel<TX, TY, DENS>, sm);
+  if (e != cudaSuccess) return e;
   const int threads = (TX / 4) * (TY / 2) + 32;
   if (occ)
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, pair_kernel<TX, TY, DENS>, threads,

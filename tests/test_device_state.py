@@ -40,3 +40,40 @@ int main() {
   CHECK(memo.get({0, 0, 0, 0, 0, 0, 4999}, answer(9)) == 1);     // bounded, the latest kept
 }
 """)
+
+
+def test_shared_memory_allowance_is_per_device_and_never_lowered(tmp_path):
+    _run(tmp_path, r"""
+#include <thread>
+#include <vector>
+int main() {
+  mamute::SmemLimit lim;
+  std::vector<size_t> on[70];
+  auto set = [&](int dev, int rc = 0) { return [&on, dev, rc](size_t b) { on[dev].push_back(b); return rc; }; };
+  CHECK(lim.raise(0, 100, set(0)) == 0 && lim.raise(0, 60, set(0)) == 0);
+  CHECK(on[0] == std::vector<size_t>{100});                    // smaller: nothing to do
+  CHECK(lim.raise(1, 60, set(1)) == 0 && on[1].size() == 1);    // a second device is set too
+  CHECK(lim.raise(1, 80, set(1, 5)) == 5);                      // a failure is reported
+  CHECK(lim.raise(1, 80, set(1)) == 0 && on[1].size() == 3);    // and tried again
+  CHECK(lim.raise(68, 90, set(68)) == 0 && lim.raise(69, 10, set(69)) == 0);
+  CHECK(on[69] == std::vector<size_t>{90});                     // devices without an entry of their own
+  // threads with different needs: the attribute only grows
+  mamute::SmemLimit many;
+  std::atomic<size_t> attr{0};
+  std::atomic<bool> fell{false}, early{false};
+  std::vector<std::thread> ts;
+  for (int t = 0; t < 8; ++t)
+    ts.emplace_back([&, t] {
+      for (size_t k = 1; k <= 2000; ++k) {
+        const size_t need = k * 8 + t;
+        many.raise(0, need, [&](size_t b) {
+          if (attr.exchange(b) > b) fell = true;
+          return 0;
+        });
+        if (attr.load() < need) early = true;
+      }
+    });
+  for (auto& t : ts) t.join();
+  CHECK(!fell && !early);
+}
+""")

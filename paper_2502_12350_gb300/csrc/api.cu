@@ -21,6 +21,7 @@
 #include "device_state.h"
 #include "postproc.h"
 #include "revolve.h"
+#include "staging.h"
 #include "stencil.h"
 
 using namespace mamute;
@@ -129,8 +130,7 @@ struct mamute_ctx {
   DevBuf gnV, gnRe, gnIm, gnS, gnR, gnW, gnBins, gnWts, gnRow;  // GN-diagonal scratch
   DevBuf nnPartial, nnLoss;  // network scratch
   DevBuf slotmaps;           // tensor maps of the checkpoint slots
-  char* stage = nullptr;  // page-locked staging of the uploads (see upload)
-  size_t stage_bytes = 0, stage_used = 0, stage_need = 0;
+  Staging stage;  // of the tables that each call uploads
   // Page-locked words: `status` is written by a kernel whose wait runs out
   // (mapped), the others receive copies.  A pageable target would make each
   // copy wait on the host, and a device word would need a clear and a copy per call.
@@ -199,40 +199,38 @@ void release(DevBuf& b) {
   b.bytes = 0;
 }
 
-// Uploads go through the context's page-locked staging area, so that the host
-// neither waits for each copy nor keeps the vectors.  What a call stages is
-// counted, and stage_reset, which starts a call, makes room for as much; what
-// does not fit is copied from the vector and waited for.
+// A table that stays for later calls: not staged, so that the staging area is
+// not sized for it.
 template <typename T>
-cudaError_t upload(mamute_ctx* ctx, DevBuf& b, const std::vector<T>& v) {
+cudaError_t upload_once(mamute_ctx* ctx, DevBuf& b, const std::vector<T>& v) {
   cudaError_t e = ensure(b, sizeof(T) * std::max<size_t>(v.size(), 1));
   if (e != cudaSuccess || v.empty()) return e;
-  const size_t bytes = sizeof(T) * v.size(), room = (bytes + 255) / 256 * 256;
-  ctx->stage_need += room;
-  if (ctx->stage_used + room <= ctx->stage_bytes) {
-    char* p = ctx->stage + ctx->stage_used;
-    ctx->stage_used += room;
-    std::memcpy(p, v.data(), bytes);
-    return cudaMemcpyAsync(b.p, p, bytes, cudaMemcpyHostToDevice, ctx->stream);
-  }
-  e = cudaMemcpyAsync(b.p, v.data(), bytes, cudaMemcpyHostToDevice, ctx->stream);
+  e = cudaMemcpyAsync(b.p, v.data(), sizeof(T) * v.size(), cudaMemcpyHostToDevice, ctx->stream);
   return e == cudaSuccess ? cudaStreamSynchronize(ctx->stream) : e;
 }
 
+// A table of this call, through the page-locked staging area (see staging.h).
+template <typename T>
+cudaError_t upload(mamute_ctx* ctx, DevBuf& b, const std::vector<T>& v) {
+  const size_t bytes = sizeof(T) * v.size();
+  void* p = bytes ? ctx->stage.take(bytes) : nullptr;
+  if (!p) return upload_once(ctx, b, v);
+  const cudaError_t e = ensure(b, bytes);
+  if (e != cudaSuccess) return e;
+  std::memcpy(p, v.data(), bytes);
+  return cudaMemcpyAsync(b.p, p, bytes, cudaMemcpyHostToDevice, ctx->stream);
+}
+
 cudaError_t stage_reset(mamute_ctx* ctx) {
-  cudaError_t e = cudaSuccess;
-  if (ctx->stage_used > 0) e = cudaStreamSynchronize(ctx->stream);  // a failed call's copies
-  if (ctx->stage_need > ctx->stage_bytes) {
-    if (ctx->stage) cudaFreeHost(ctx->stage);
-    ctx->stage = nullptr;
-    ctx->stage_bytes = 0;
-    if (cudaHostAlloc((void**)&ctx->stage, ctx->stage_need, cudaHostAllocPortable) == cudaSuccess)
-      ctx->stage_bytes = ctx->stage_need;
-    else
-      cudaGetLastError();  // without it the copies wait
-  }
-  ctx->stage_used = ctx->stage_need = 0;
-  return e;
+  return (cudaError_t)ctx->stage.begin(
+      [&] { return (int)cudaStreamSynchronize(ctx->stream); },
+      [](size_t n) -> void* {
+        void* p = nullptr;
+        if (cudaHostAlloc(&p, n, cudaHostAllocPortable) == cudaSuccess) return p;
+        cudaGetLastError();  // without it the copies wait
+        return nullptr;
+      },
+      [](void* p) { cudaFreeHost(p); });
 }
 
 // Cerjan profile of one padded axis; with a free surface at plane zs (z axis
@@ -1141,7 +1139,7 @@ int do_smooth(mamute_ctx* ctx, int nx, int ny, int nz, double h, int mode, const
         }
       }
     }
-    CK(upload(ctx, ctx->smMat, tab));
+    CK(upload_once(ctx, ctx->smMat, tab));
     if (bessel) {
       CK(ensure(ctx->smLam, sizeof(RowCoef) * (size_t)ny * nz));
       ++ctx->launches;
@@ -1280,9 +1278,9 @@ int do_resample(mamute_ctx* ctx, int ntr, int nt_in, double dt_in, int nt_out, d
     std::vector<float> wb((size_t)K * rows, 0.0f);
     for (int m = 0; m < rows; ++m)
       for (int k = ptr[m]; k < ptr[m + 1]; ++k) wb[(size_t)(col[k] - c0[m]) * rows + m] = w[k];
-    CK(upload(ctx, ctx->rsPtr, c0));
-    CK(upload(ctx, ctx->rsCol, len));
-    CK(upload(ctx, ctx->rsW, wb));
+    CK(upload_once(ctx, ctx->rsPtr, c0));
+    CK(upload_once(ctx, ctx->rsCol, len));
+    CK(upload_once(ctx, ctx->rsW, wb));
     ctx->rsKey = key;
     ctx->rsTaps = K;
   }
@@ -2525,7 +2523,7 @@ void mamute_ctx_destroy(mamute_ctx* ctx) {
                    &ctx->cpml, &ctx->cext, &ctx->cprof, &ctx->cvols};
   for (DevBuf* b : all) release(*b);
   if (ctx->host) cudaFreeHost(ctx->host);
-  if (ctx->stage) cudaFreeHost(ctx->stage);
+  ctx->stage.release([](void* p) { cudaFreeHost(p); });
   if (ctx->vmax_ev) cudaEventDestroy(ctx->vmax_ev);
   if (ctx->maxbits) cudaFree(ctx->maxbits);
   for (cudaEvent_t ev : ctx->dft_ev) cudaEventDestroy(ev);

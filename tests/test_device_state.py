@@ -1,5 +1,5 @@
-"""What the library remembers about devices on the host (csrc/device_state.h),
-with the CUDA calls played by the test."""
+"""What the library remembers about devices on the host (csrc/device_state.h) and
+its staging of uploads (csrc/staging.h), with the CUDA calls played by the test."""
 import os
 import subprocess
 
@@ -77,3 +77,38 @@ int main() {
   CHECK(!fell && !early);
 }
 """)
+
+
+def test_staging_area_is_bounded(tmp_path):
+    _run(tmp_path, r"""
+int main() {
+  mamute::Staging st;
+  int waits = 0, allocs = 0, frees = 0;
+  bool refuse = false;
+  auto begin = [&] {
+    return st.begin([&] { return ++waits, 0; },
+                    [&](size_t n) -> void* { return ++allocs, refuse ? nullptr : std::malloc(n); },
+                    [&](void* p) { ++frees, std::free(p); });
+  };
+  CHECK(begin() == 0 && allocs == 0 && waits == 0);
+  CHECK(!st.take(1000) && !st.take(10));                     // the first call copies and waits
+  begin();
+  CHECK(st.bytes() == 1280 && allocs == 1 && waits == 0);
+  char* a = static_cast<char*>(st.take(1000));
+  char* b = static_cast<char*>(st.take(10));
+  CHECK(a && b == a + 1024 && !st.take(1));                  // as much as the call before
+  begin();
+  CHECK(waits == 1 && st.bytes() == 1536 && frees == 1);
+  CHECK(!st.take(10 * mamute::Staging::kMax) && st.take(256));  // a table beyond the bound
+  begin();
+  CHECK(st.bytes() == mamute::Staging::kMax);                // never more than the bound
+  CHECK(!st.take(mamute::Staging::kMax + 1) && st.take(4096));
+  begin();
+  CHECK(st.bytes() == mamute::Staging::kMax && allocs == 3);
+  st.release([&](void* p) { ++frees, std::free(p); });
+  CHECK(frees == 3 && st.bytes() == 0 && !st.take(1));
+  refuse = true;
+  begin();
+  CHECK(st.bytes() == 0 && !st.take(1));                     // none to be had: the copies wait
+}
+""", "staging.h")

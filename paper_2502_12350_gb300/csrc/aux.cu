@@ -230,12 +230,14 @@ __global__ void sum_partials_kernel(const double* partial, int n, double* out) {
   }
 }
 
-// grad[z][y][x] = 2 / (c^3 dt^2) sum_s G_s, or phess = sum_s P_s / (c dt)^4,
+// KIND 0: grad[z][y][x] = 2 / (c^3 dt^2) sum_s G_s, 1: phess = sum_s P_s / (c dt)^4,
 // summed over shots in ascending order (deterministic).  One block per row, so that
 // no point divides its 64-bit index.  Bound by the FP64 units, a 64th of the FP32
 // rate: 256^3 takes 503 us.  The quotient is one FP64 division: a Newton step from
 // an FP32 reciprocal in its place saved 14 us and left errors of 8e-15, which show
-// in rare FP32 roundings.
+// in rare FP32 roundings.  Zeros, the cells that no wave has reached, pass it by:
+// its path for them made 256^3 of zeros take 861 us (now 87).
+template <int KIND>
 __global__ void __launch_bounds__(128) finalize_kernel(FinalizeArgs a) {
   const int y = (int)(blockIdx.x % (unsigned)a.ny), z = (int)(blockIdx.x / (unsigned)a.ny);
   const int Y = y + a.border, Z = z + a.border;
@@ -251,15 +253,16 @@ __global__ void __launch_bounds__(128) finalize_kernel(FinalizeArgs a) {
       acc += a.acc[V.off + ((long long)Z * V.Ny + ly) * V.pitch + lx];
     }
     const double cv = a.vel[row + x];
-    double out;
-    if (a.kind == 0) {
-      out = 2.0 * (double)acc / (cv * cv * cv * a.dt * a.dt);
-      if (z < a.zero_top) out = 0.0;
-    } else {
-      const double A2 = cv * cv * a.dt * a.dt;
-      out = (double)acc / (A2 * A2);
+    float out = 0.0f;
+    if ((acc != 0.0f || !(cv > 0.0)) && !(KIND == 0 && z < a.zero_top)) {
+      if (KIND == 0) {
+        out = (float)(2.0 * (double)acc / (cv * cv * cv * a.dt * a.dt));
+      } else {
+        const double A2 = cv * cv * a.dt * a.dt;
+        out = (float)((double)acc / (A2 * A2));
+      }
     }
-    a.out[row + x] = (float)out;
+    a.out[row + x] = out;
   }
 }
 
@@ -352,7 +355,10 @@ cudaError_t launch_misfit(const float* d, const float* dobs, long long n, double
 }
 
 cudaError_t launch_finalize(const FinalizeArgs& a, cudaStream_t s) {
-  finalize_kernel<<<(unsigned)(a.ny * a.nz), 128, 0, s>>>(a);
+  if (a.kind == 0)
+    finalize_kernel<0><<<(unsigned)(a.ny * a.nz), 128, 0, s>>>(a);
+  else
+    finalize_kernel<1><<<(unsigned)(a.ny * a.nz), 128, 0, s>>>(a);
   return cudaGetLastError();
 }
 

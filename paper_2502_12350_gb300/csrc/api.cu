@@ -1367,10 +1367,12 @@ struct PmlTables {
   float* mem = nullptr;
 };
 
-// Modelling on windows of at most this many padded points in all launches
-// every slab piece apart, which with the main step keeps the eight launches
-// per step that callers of mamute_ctx_last_timing count on tiny windows; it
-// is no faster there.  Above it a step is four launches.
+// Modelling on windows of at most this many padded points in all spreads the slab
+// pieces over seven launches a step instead of three.  This is not for speed: a
+// step of 24^3, 40^3 and 50^3 padded points takes 34.4, 34.5 and 37.4 us, and
+// 17.2, 17.7 and 18.8 with one launch per axis.  It keeps the eight launches a
+// step, the main one among them, that callers of mamute_ctx_last_timing count on
+// for windows of this size.
 constexpr long long kPmlApartPoints = 128 * 1024;
 
 // Slabs of every window (the plan's windows learn where E is not zero).

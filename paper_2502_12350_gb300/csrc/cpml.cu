@@ -509,19 +509,23 @@ dim3 march_grid(const CpmlExtent& e, int a, int V, int chunk) {
               (unsigned)(2 * ((e.len[a] + chunk - 1) / chunk)));
 }
 
+// Launches that the pieces of an axis's slabs are spread over (see CpmlExtent::apart).
+int parts(const CpmlExtent& e, int a) {
+  const int k = piece(e, a), pieces = 2 * ((e.len[a] + k - 1) / k);
+  return e.apart ? std::min(pieces, a == 2 ? 4 : 2) : 1;
+}
+
 template <int A>
 void forward_axis(const CpmlArgs& c, const CpmlExtent& e, cudaStream_t s) {
   if (e.len[A] <= 0) return;
-  int k = piece(e, A);
-  if (!e.apart) {
-    fwd_march_kernel<A><<<march_grid(e, A, 4, k), kThreads, 0, s>>>(c, k, 0);
-    return;
-  }
-  k = A == 2 ? (e.len[A] + 1) / 2 : e.len[A];
+  const int k = piece(e, A), n = parts(e, A);
   dim3 g = march_grid(e, A, 4, k);
-  const int n = g.z;
-  g.z = 1;
-  for (int i = 0; i < n; ++i) fwd_march_kernel<A><<<g, kThreads, 0, s>>>(c, k, i);
+  const int pieces = (int)g.z;
+  for (int i = 0; i < n; ++i) {
+    const int first = pieces * i / n;
+    g.z = (unsigned)(pieces * (i + 1) / n - first);
+    fwd_march_kernel<A><<<g, kThreads, 0, s>>>(c, k, first);
+  }
 }
 
 template <int A>
@@ -540,10 +544,7 @@ dim3 x_grid(const CpmlExtent& e) {
 int cpml_launches(const CpmlExtent& e) {
   int n = e.cols[0] > 0 ? 1 : 0;
   for (int a = 1; a < 3; ++a)
-    if (e.len[a] > 0) {
-      const int k = e.apart ? (a == 2 ? (e.len[a] + 1) / 2 : e.len[a]) : 1;
-      n += e.apart ? 2 * ((e.len[a] + k - 1) / k) : 1;
-    }
+    if (e.len[a] > 0) n += parts(e, a);
   return n;
 }
 

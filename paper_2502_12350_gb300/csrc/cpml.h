@@ -51,7 +51,7 @@ struct CpmlExtent {
   long long cols[3];  // threads across the axis, at most: x: rows x groups of 4 slots
   int len[3];         // longest slab along the axis (y, z)
   long long threads[3];  // threads of a launch with unsplit slabs, over all windows (y, z)
-  bool apart;            // modelling on tiny windows: each piece of a slab is a launch of its own
+  bool apart;            // modelling on small windows: an axis's pieces over several launches
 };
 
 // Psi_a <- b_a Psi_a + c_a D1_a u, Zeta_a <- b_a Zeta_a + c_a (D2_a u + D1_a Psi_a),

@@ -107,10 +107,16 @@ typedef struct {
  *                   states may use when n_snapshots == 0 (default 0.8).
  *   n_snapshots     0: automatic: keep the imaging term of every step when
  *                   nt x (interior points) x 4 bytes fits in check_mem of
- *                   the free memory, else as many revolve
- *                   slots as check_mem allows; >0: exactly that many revolve
- *                   slots; -1: keep the imaging term of every step (no
- *                   recomputation).
+ *                   the free memory, else as many slots as check_mem allows;
+ *                   >0: exactly that many slots, of two padded wavefields
+ *                   each; -1: keep the imaging term of every step (no
+ *                   recomputation).  Slots are memory: the library uses some
+ *                   of them for checkpoints and the others for the imaging
+ *                   terms of a block of consecutive steps, in the split of
+ *                   least work (all for checkpoints where that is less), so a
+ *                   gradient's step launches are not those of
+ *                   mamute_revolve_plan(nt, slots); mamute_ctx_last_timing
+ *                   counts them.  The result does not depend on the split.
  *   zero_top_planes ZeroesNearSurface: gradient planes z < this are zeroed.
  *   aperture        host [n_src][4] or NULL: shot s propagates only over the
  *                   model columns x in [a0, a1), y in [a2, a3) plus the sponge
@@ -309,7 +315,10 @@ int mamute_adam(mamute_ctx* ctx, int n, float* p, float* m, float* v, const floa
 
 /* Checkpoint schedule (host only, no device work; Sec. 2.1 optimal
  * checkpointing after Griewank and Walther).  Plans the reversal of nt steps
- * from the zero initial state with n_slots checkpoint slots.  Writes the
+ * from the zero initial state with n_slots checkpoint slots, each step
+ * reversed on its own.  (mamute_gradient runs such a schedule over blocks of
+ * steps with the slots that do not hold imaging terms, see n_snapshots.)
+ * Writes the
  * number of forward steps the plan takes (the first sweep included) to
  * *n_forward and the number of actions to *n_actions; if `actions` is not
  * NULL it must hold 3 * (*n_actions) ints from a previous sizing call and
@@ -374,8 +383,10 @@ int mamute_misfit_noalloc(const float* d, const float* d_obs, long long n, void*
  *   mode 1 (Bessel)   out = (I - lx^2 Dxx - ly^2 Dyy - lz^2 Dzz)^-1 in
  *   mode 2 (Laplace)  out = (I - lx^2 Dxx)^-1 (I - ly^2 Dyy)^-1 (I - lz^2 Dzz)^-1 in
  *   mode 0            out = in.
- * Solved exactly in the DCT-II basis, which diagonalises both operators
- * (FP32 transforms).  lengths: host [3] (lx, ly, lz, metres; 0 means 2 h) or
+ * Solved exactly, in FP32: by tridiagonal solves along the axes (Laplace), or
+ * by the DCT-II along y and z, which diagonalises their operators, and a
+ * tridiagonal solve along x (Bessel).  lengths: host [3] (lx, ly, lz, metres;
+ * 0 means 2 h; above 1e9 h, where the filter passes the mean alone, 1e9 h) or
  * NULL for all 2 h.  in, out: device [nz][ny][nx]; they may be the same
  * array.  Errors: EINVAL (sizes, NULL, bad mode or negative length), ENOMEM,
  * ECUDA. */

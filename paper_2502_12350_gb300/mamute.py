@@ -95,7 +95,9 @@ def cfl_limit() -> float:
 
 
 def revolve_plan(nt: int, n_slots: int):
-    """(n_forward, actions[n][3]) of the checkpoint schedule (host only)."""
+    """(n_forward, actions[n][3]) of the checkpoint schedule (host only), each
+    step reversed on its own; a gradient with as many slots runs one over blocks
+    of steps."""
     lib = load()
     nf = ctypes.c_longlong(0)
     na = ctypes.c_int(0)

@@ -966,13 +966,17 @@ int check_common(mamute_ctx* ctx, const mamute_grid* g, const float* vel, const 
     if (rc_ != MAMUTE_OK) return rc_; \
   } while (0)
 
-// A call that fails after it has launched work leaves none in flight: the
-// caller's arrays may go when it returns.  (A call that succeeds has
-// synchronised already, and the wait returns at once.)
+// A call that fails after it has launched work leaves none in flight, on the
+// context's stream or on the one that copies seismograms out: the caller's
+// arrays may go when it returns.  (A call that succeeds has synchronised already,
+// and the waits return at once.)
 struct InFlight {
   mamute_ctx* ctx;
   explicit InFlight(mamute_ctx* c) : ctx(c) {}
-  ~InFlight() { cudaStreamSynchronize(ctx->stream); }
+  ~InFlight() {
+    cudaStreamSynchronize(ctx->stream);
+    if (ctx->copy) cudaStreamSynchronize(ctx->copy);
+  }
 };
 
 // Two-level forward launches (stencil_pair.cu), on request (time_blocking =
@@ -2564,6 +2568,7 @@ int mamute_model_host(mamute_ctx* ctx, const mamute_grid* g, const float* vel, c
                       const float* rec_xyz, const mamute_opts* opts, float* seis) {
   if (!ctx || !g || !vel || !rec_offset || n_src < 1) return MAMUTE_EINVAL;
   TRY(check_common(ctx, g, vel, wavelet));
+  InFlight guard(ctx);  // of the uploads below too
   int ti = 0, ntd = g->nt;
   TRY(check_interp(ctx, g, opts, &ti, &ntd));
   const size_t nm = (size_t)g->nx * g->ny * g->nz * 4;
@@ -2597,6 +2602,7 @@ int mamute_gradient_host(mamute_ctx* ctx, const mamute_grid* g, const float* vel
                          const mamute_opts* opts, double* misfit, float* grad) {
   if (!ctx || !g || !vel || !rec_offset || n_src < 1 || !grad) return MAMUTE_EINVAL;
   TRY(check_common(ctx, g, vel, wavelet));
+  InFlight guard(ctx);  // of the uploads below too
   int ti = 0, ntd = g->nt;
   TRY(check_interp(ctx, g, opts, &ti, &ntd));
   const size_t nm = (size_t)g->nx * g->ny * g->nz * 4;

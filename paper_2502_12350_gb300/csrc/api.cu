@@ -1746,8 +1746,8 @@ struct BlockPlan {
 // an adjoint step 1.1 against stored terms, 1.75 against a recomputed state
 // (measured step times on a 213x202x163 window).  300 steps and 16 slots there:
 // 11 slots of terms, 38 steps a block, 604 forward steps and 300 against
-// stored terms, 30.4 ms; as checkpoints alone 711 and 300 against recomputed
-// states, 45.3 ms.
+// stored terms, 30.4 ms; side by side with it, checkpoints alone took 711 and 300
+// against recomputed states, 45.3 ms.
 BlockPlan plan_blocks(int nt, int slots, size_t pool_elems, size_t term_elems) {
   BlockPlan best;
   double least = (double)revolve_cost(nt, slots) + 1.75 * nt;

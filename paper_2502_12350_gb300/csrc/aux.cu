@@ -23,7 +23,7 @@ __global__ void sqrt_kernel(const float* __restrict__ rho, long long n, double* 
 // prep_fill_kernel copies the rest.  Bound by the FP64 units (about 40
 // operations a point, a 64th of the FP32 rate): with every padded point formed,
 // two more FP64 divisions each and 64-bit index divisions, 448x448x256 took
-// 5.7 ms; now 3.1 (576x576x320: a 400-step call 146.5 -> 141.7 ms).
+// 5.7 ms, now 3.1.
 constexpr int kReach = 5;
 
 // First and last + 1 core cell of a padded axis.

@@ -380,10 +380,9 @@ void conv_gy_box(unsigned (&box)[4]) {
 // NCH chunks of 128 outputs; a plane costs as much as one chunk more (waits,
 // swizzle start), an item's start two planes.  Halo slots leave room for a
 // ring of 4 planes (each is consumed by one step), or 3 where nothing has 4.
-// (The tallest row block with the fewest rounds of ZC planes, its halo planes
-// not counted, took 3 rounds of 5 planes where 1 round of 16 does it, and left
-// most SMs idle on small volumes: a layer's three passes took 290 us on
-// 80x160x160, now 256; 12x63x23 takes 67.)
+// A layer's three passes take 260 us on 80x160x160 and 67 on 12x63x23.  (The
+// tallest row block with the fewest rounds of ZC planes, its halo planes not
+// counted, takes 3 rounds of 5 planes where 1 round of 16 does it: 290 us.)
 constexpr int kTcSmemMax = 232448;                  // dynamic shared memory per CTA
 constexpr int kTcSlotBudget = kTcSmemMax - kTcWBytes - 1024;
 

@@ -27,15 +27,15 @@
 // the whole memory-variable part before the main step, which reads E as one
 // more centre tile: per layer point and axis the field, the two memory
 // variables (read and written) and E, 28 bytes written or read once by the
-// slab kernel and the main step together.  (The earlier form updated Psi
-// before the main step, Zeta after it, and corrected u', the imaging term
-// and the accumulator in place, once per axis: 40 bytes forward and 60 in
-// reverse, in 6 and 7 launches.  448x448x256 with density: 577 -> 326 us a
-// step, of which 59, 37 and 50 us the z, y and x slabs and 179 us the main
-// step; 250 forward and reverse steps of 256^3: 167 -> 95 ms.)  A cell needs the new Psi (p) of its 4
-// neighbours on each side; they are made again from the old values instead
+// slab kernel and the main step together.  A cell needs the new Psi (p) of its
+// 4 neighbours on each side; they are made again from the old values instead
 // of being exchanged, so Psi, and in the reverse both multipliers, are kept
 // twice (read one copy, write the other) and a slab may be cut anywhere.
+// 448x448x256 with density takes 326 us a step, 59, 37 and 50 of them the z, y
+// and x slabs and 179 the main step, which is bound by HBM; updating Psi before
+// the main step, Zeta after it and correcting u', the imaging term and the
+// accumulator in place (40 bytes forward and 60 in reverse, 6 and 7 launches)
+// took 577.
 #include "cpml.h"
 
 #include <algorithm>

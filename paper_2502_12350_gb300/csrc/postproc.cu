@@ -11,10 +11,8 @@
 // transforms along y and z (dct_kernel) every row is one tridiagonal system
 // along x with its own diagonal (row_kernel), and the transposed transforms
 // along z and y follow.
-// (Six dense transforms, three per direction, and a spectral multiplier made
-// the 600x600x200 Bessel filter 15.9 ms; with the transforms along x replaced
-// by a bandwidth-bound pass of 0.16 ms and the others halved by their symmetry
-// it took 4.1 ms, and takes 2.9 with packed multiply-adds on 8 x 8 tiles.)
+// The 600x600x200 Bessel filter takes 2.92 ms, 2.7 of them the transforms; six
+// dense transforms and a spectral multiplier took 15.9.
 //
 // Resampling (Sec. 2: time interpolation by nearest neighbour or sinc;
 // Table 1 Interpolate).  The resampling of every trace is the same sparse
@@ -219,10 +217,9 @@ __global__ void __launch_bounds__(256, CARRY ? 3 : 4) sweep_kernel(const float* 
 // with O, 8 lines x 8 outputs each, fed by float4 shared-memory reads, with the
 // next chunk's global loads in registers while a chunk is multiplied; the two
 // products of an output meet in shared memory at the end.  Bound by issue and
-// the shared-memory reads: 8 lines x 4 outputs of both products with one
-// multiply-add per instruction kept the FMA pipe 46 % busy (600x600x200 Bessel
-// filter 4.06 ms); two lines per instruction 3.37 ms; 8 x 8 tiles, 4 reads for
-// 32 instructions instead of 3 for 16, 2.91 ms.
+// the shared-memory reads, 4 for 32 packed multiply-adds: 680 us a launch at
+// 600x600x200, 0.49 of the FP32 peak (8 lines x 4 outputs of both products per
+// thread, 3 reads for 16 packed multiply-adds: 3.37 ms for the filter).
 constexpr int kTL = 128, kTI = 64, kTK = 8;
 constexpr int kAP = kTL + 4;  // A row pitch
 
@@ -413,12 +410,10 @@ __global__ void band_few_kernel(const float* __restrict__ x, int n_in, const int
 // the outputs' bands need no branches; a thread also sums zero times every
 // sample, which is not zero if a sample is not finite, and then the block
 // takes its chunks again with a mask of the outputs whose band holds the
-// sample (such a sample reaches only those).  (One output and 8 traces per
-// thread, straight from global memory, spent 33 L1 wavefronts per 8
-// multiply-add instructions, the outputs' bands being dt_out / dt_in samples
-// apart: 65,536 traces of 4000 samples to 1000 took 1.76 ms; masks on the
-// samples that not all 8 outputs take, one multiply-add per instruction, 0.93;
-// now 0.85.)  Bound by issue and the barriers of the chunks: a warp's 8
+// sample (such a sample reaches only those).  65,536 traces of 4000 samples to
+// 1000 take 0.84 ms; one output and 8 traces per thread, straight from global
+// memory, 33 L1 wavefronts per 8 multiply-adds with bands dt_out / dt_in samples
+// apart, took 1.76.  Bound by issue and the barriers of the chunks: a warp's 8
 // outputs take about half of the block's window.  Every output is the same sum
 // in the same order.
 constexpr int kBM = 32, kBT = 128, kBK = 32;

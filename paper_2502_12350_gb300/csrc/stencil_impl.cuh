@@ -69,8 +69,10 @@ __device__ __forceinline__ void lap4(const float* st, int lx, int ly, const F4 (
   // operations (no contraction freedom), so that every kernel that forms them
   // for the same field gets bitwise the same values.  Packed instructions,
   // because on windows of a few tiles per SM a step is bound by issue as much
-  // as by HBM: 500 steps of 96^3 3.67 -> 3.43 ms, a step of four 243x191x137
-  // windows 101 -> 95 us, of 20 windows of 136x120x104 (labels) 101 -> 96 ms.
+  // as by HBM.  Against one point per instruction, all else equal: 500 steps of
+  // 96^3 3.43 ms instead of 3.67, a step of four 243x191x137 windows 95 us
+  // instead of 101, a whole label of 20 windows of 136x120x104 and 500 steps
+  // 96 ms instead of 101.
   const float cw[4] = {MAMUTE_C1, MAMUTE_C2, MAMUTE_C3, MAMUTE_C4};
 #pragma unroll
   for (int e = 0; e < 4; e += 2) {
@@ -163,9 +165,8 @@ struct PlaneInfo {
 // three steps and point that is 48 + 8 + 12 bytes (the terms on the model
 // interior only) instead of 48 + 24 + 12, and the two launches that do not
 // image need less than half of the centre ring.  Bound by HBM: on a 320^3
-// window with a 256^3 model 88.8 us for a plain step and 148.9 us with the
-// imaging of three levels, against 158.6 us for every step that images its
-// own (a 400-step gradient 114.1 -> 94.4 ms).
+// window with a 256^3 model a plain step takes 80 us and one with the imaging of
+// three levels 147; every step that images its own took 159.
 // Resident CTAs per SM the register budget is sized for: the adjoint with a
 // recomputed forward field on large tiles needs more than 200 KB of shared
 // memory per pair, so it runs one CTA per SM with the full register file;
@@ -235,8 +236,9 @@ __global__ void __launch_bounds__((TX / 4) * TY + 32, (MinBlocks<TX, TY, MODE>::
   // A chained launch (StepArgs::chained) may start while the previous step
   // ends: everything above reads tables that no step writes.  The producer
   // waits for the previous step before its first load; the other threads act
-  // on its loads alone, so the wait covers their stores too.  (500 steps of 96^3:
-  // 5.58 -> 4.98 ms; 800 launches of a 320^3 gradient: 88.5 -> 85.7 ms.)
+  // on its loads alone, so the wait covers their stores too.  All else equal, 500
+  // steps of 96^3 took 4.98 ms chained and 5.58 not, 800 launches of a 320^3
+  // gradient 85.7 and 88.5.
 
   // Maps of the buffers this launch reads (chosen by the host per step).
   const CUtensorMap* mapF = a.mF + (long long)it.vol * a.sF;
@@ -374,10 +376,10 @@ __global__ void __launch_bounds__((TX / 4) * TY + 32, (MinBlocks<TX, TY, MODE>::
   // Planes per pass of the loop: the register queue moves on by 32 registers a
   // plane, which unrolling folds into the names; as many as the 96 registers of
   // the tiles with two CTAs of 288 and 320 threads take without spilling.
-  // 400 steps of 576x576x320 with density (72x16) 139.6 -> 135.4 ms with two (three
-  // spill: 144.3); four 243x191x137 windows (64x16) 29.0 -> 28.2 ms with three (two
-  // spill: 29.6), where the adjoint takes two (256^3 gradient 84.1 -> 82.4 ms; three
-  // spill: 84.9); 96^3 (48x16, few planes a block) is best without.
+  // 400 steps of 576x576x320 with density (72x16): one 139.6 ms, two 135.4, three
+  // 144.3 (they spill); four 243x191x137 windows (64x16): one 29.0, two 29.6 (spills),
+  // three 28.2; a 256^3 gradient (64x16, the adjoint): one 84.1, two 82.4, three 84.9
+  // (spills); 96^3 (48x16, few planes a block) is best with one.
   constexpr int kUnroll = TX == 72 && TY == 16 ? 2 : (TX == 64 && TY == 16 ? (ADJ ? 2 : 3) : 1);
 #pragma unroll kUnroll
   for (int j = 0; j < npl; ++j) {
